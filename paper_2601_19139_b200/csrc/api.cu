@@ -44,7 +44,7 @@ size_t align_up(size_t v) { return (v + kAlign - 1) / kAlign * kAlign; }
 // Per-step metadata, one contiguous block: header, attention work list, block tables.
 struct MetaLayout {
   int max_blocks_cap, max_work;
-  size_t off_tokens, off_lens, off_slot_base, off_nchunks, off_bt, off_work, bytes;
+  size_t off_tokens, off_lens, off_slot_base, off_nchunks, off_bt, off_work, off_prompt, bytes;
   void init(int max_positions) {
     max_blocks_cap = (max_positions + kBlockSize - 1) / kBlockSize;
     max_work = attention_max_work(kMaxBatch, max_positions);
@@ -55,6 +55,7 @@ struct MetaLayout {
     off_nchunks = o, o += kMaxBatch * 4;
     off_work = o, o += (size_t)max_work * sizeof(int4);
     off_bt = o, o += (size_t)kMaxBatch * max_blocks_cap * 4;
+    off_prompt = align_up(o), o = off_prompt + (size_t)(max_blocks_cap + kPrefillChunk) * 4;  // block table, then tokens
     bytes = align_up(o);
   }
 };
@@ -71,6 +72,12 @@ struct Workspace {
   // of the residual stream, split-KV scratch, argmax partials, barrier/status words, phase table
   size_t f_attn, f_h, f_ss, f_pacc, f_pml, f_attn_counters, f_amax, f_control, f_timeline, chain_status;
   int f_max_items, f_max_ctas, f_n_phases;
+  // prompt processing: up to p_rows tokens at once.  p_u holds qkv, q and the attention output while a layer's first
+  // half runs and the MLP activations in its second half; p_op, p_inv the operand of the coming projection.  MoE: the
+  // (token, expert) pairs sorted by expert (their operand, then their outputs, in p_pairs).
+  size_t p_x, p_u, p_q, p_attn, p_op, p_inv, p_y, p_idx, p_wgt, p_pos, p_counts, p_cursor, p_units, p_pairs, p_pairs_inv, p_eh, p_eop,
+      p_eop_inv;
+  int p_rows;
 };
 
 // The CTA count the whole-step kernel is sized for: one per SM of the current device (148 when there is none).
@@ -194,6 +201,29 @@ Workspace carve(const q4d_shape& s, const MetaLayout& ml) {
     w.f_amax = take((size_t)w.f_max_ctas * 16 * sizeof(float2));
     w.f_control = take(256);
     w.f_timeline = take((size_t)(w.f_n_phases + 1) * 8);
+  }
+  {
+    const size_t R = (size_t)std::min(kPrefillChunk, (s.max_positions + 15) / 16 * 16), H = s.hidden;
+    w.p_rows = (int)R;
+    w.p_x = take(R * H * 2);
+    const size_t first_half = align_up(R * nqkv * 2) + 2 * align_up(R * qdim * 2);
+    w.p_u = take(std::max(first_half, s.n_experts ? (size_t)0 : R * s.mlp_inter * 2));
+    w.p_q = w.p_u + align_up(R * nqkv * 2), w.p_attn = w.p_q + align_up(R * qdim * 2);
+    size_t width = std::max<size_t>(H, qdim);
+    if (!s.n_experts) width = std::max<size_t>(width, s.mlp_inter);
+    w.p_op = take(R * prefill_operand_stride((int)width) * 2);
+    w.p_inv = take(R * 4);
+    w.p_y = w.p_idx = w.p_wgt = w.p_pos = w.p_counts = w.p_cursor = w.p_units = w.p_pairs = w.p_pairs_inv = w.p_eh = w.p_eop = w.p_eop_inv = 0;
+    if (s.n_experts) {
+      const size_t P = R * s.top_k + 256, E = s.n_experts;
+      w.p_y = take(R * H * 2);
+      w.p_idx = take(R * s.top_k * 4), w.p_wgt = take(R * s.top_k * 4), w.p_pos = take(R * s.top_k * 4);
+      w.p_counts = take(E * 4), w.p_cursor = take(E * 4);
+      w.p_units = take((E + P / 16 + 2) * sizeof(int4));  // units of at least 16 rows; the count sits in the last entry
+      w.p_pairs = take(P * prefill_operand_stride(s.hidden) * 2), w.p_pairs_inv = take(P * 4);
+      w.p_eh = take(P * s.expert_inter * 2);
+      w.p_eop = take(P * prefill_operand_stride(s.expert_inter) * 2), w.p_eop_inv = take(P * 4);
+    }
   }
   w.bytes = o;
   return w;
@@ -433,6 +463,16 @@ int run_fused(q4d_model* m, q4d_kv_pool* pool, int n, const int32_t* lens, const
   return Q4D_OK;
 }
 
+// Reads the chain's status word back behind the work enqueued so far (one read-back in flight at a time).
+int read_back_status(q4d_model* m, cudaStream_t s) {
+  if (m->status_pending) return Q4D_OK;
+  cudaError_t e = cudaMemcpyAsync(m->host_status, m->ws + m->lay.chain_status, sizeof(uint32_t), cudaMemcpyDeviceToHost, s);
+  if (e == cudaSuccess) e = cudaEventRecord(m->status_done, s);
+  if (e != cudaSuccess) return fail_cuda(e, "status read-back");
+  m->status_pending = true;
+  return Q4D_OK;
+}
+
 // The launch sequence of a step.  A whole step embeds the tokens, runs every layer and the head, and advances the
 // requests.  The parity export runs only layers [layer_begin, layer_end) from a given hidden state (x_in) and
 // returns the hidden state (x_out) without advancing anything.
@@ -658,16 +698,128 @@ int step_impl(q4d_model* m, q4d_kv_pool* pool, int32_t n, const int64_t* ids, co
   Q4D_LAUNCH(Q4D_K_LM_HEAD, launch_q4_gemm(lm, s));
   Q4D_LAUNCH(Q4D_K_ARGMAX, launch_argmax_finish(amax, lm_blocks, n, next_dev, s));
 #undef Q4D_LAUNCH
-  if (!m->status_pending) {
-    cudaError_t se = cudaMemcpyAsync(m->host_status, m->ws + m->lay.chain_status, sizeof(uint32_t), cudaMemcpyDeviceToHost, s);
-    if (se == cudaSuccess) se = cudaEventRecord(m->status_done, s);
-    if (se != cudaSuccess) return fail_cuda(se, "status read-back");
-    m->status_pending = true;
+  {
+    const int rc = read_back_status(m, s);
+    if (rc != Q4D_OK) return rc;
   }
 
   if (!pf)
     for (int r = 0; r < n; ++r) pool->lens[ids[r]] = lens[r] + 1;
   return Q4D_OK;
+}
+
+// Prompt processing of many tokens: `rows` consecutive tokens of one request from position `start`, all layers; with
+// `head`, the logits and the greedy token after the last of them.
+int prefill_rows(q4d_model* m, q4d_kv_pool* pool, const int32_t* tokens, int rows, int start, const int32_t* block_table, bool head,
+                 int32_t* next_dev, float* logits_dev, cudaStream_t s) {
+  const q4d_shape& sh = m->sh;
+  const Workspace& lay = m->lay;
+  const MetaLayout& ml = m->ml;
+  {
+    const int rc = fused_check_status(m, false);
+    if (rc != Q4D_OK) return rc;
+  }
+  const int slot = m->staging_next;
+  m->staging_next = (slot + 1) % kStagingSlots;
+  if (m->staging_used[slot]) {
+    cudaError_t e = cudaEventSynchronize(m->staging_done[slot]);
+    if (e != cudaSuccess) return fail_cuda(e, "staging wait");
+  }
+  int32_t* h_bt = reinterpret_cast<int32_t*>(m->staging[slot] + ml.off_prompt);
+  int32_t* h_tokens = h_bt + ml.max_blocks_cap;
+  const int blocks = (start + rows + kBlockSize - 1) / kBlockSize;
+  for (int i = 0; i < ml.max_blocks_cap; ++i) h_bt[i] = i < blocks ? block_table[i] : 0;
+  memcpy(h_tokens, tokens, (size_t)rows * 4);
+  const size_t meta_bytes = (size_t)(ml.max_blocks_cap + rows) * 4;
+  unsigned char* dmeta = m->ws + lay.meta + ml.off_prompt;
+  cudaError_t e = cudaMemcpyAsync(dmeta, h_bt, meta_bytes, cudaMemcpyHostToDevice, s);
+  if (e != cudaSuccess) return fail_cuda(e, "metadata copy");
+  cudaEventRecord(m->staging_done[slot], s);
+  m->staging_used[slot] = true;
+  m->last_h2d = (int64_t)meta_bytes, m->last_d2h = 0;
+  const int32_t* d_bt = reinterpret_cast<const int32_t*>(dmeta);
+  const int32_t* d_tokens = d_bt + ml.max_blocks_cap;
+
+  const int H = sh.hidden, nq = sh.n_q_heads, nkv = sh.n_kv_heads, I = sh.mlp_inter, V = sh.vocab, qdim = nq * kHeadDim;
+  const int nqkv = (nq + 2 * nkv) * kHeadDim;
+  uint16_t *x = at<uint16_t>(m, lay.p_x), *qkv = at<uint16_t>(m, lay.p_u), *attn = at<uint16_t>(m, lay.p_attn), *h = at<uint16_t>(m, lay.p_u);
+  uint16_t* op = at<uint16_t>(m, lay.p_op);
+  float* inv = at<float>(m, lay.p_inv);
+  const size_t layer_elems = (size_t)pool->num_blocks * nkv * kBlockSize * kHeadDim;
+  auto gemm = [&](const q4d_qtensor& t, int N, int K, const uint16_t* operand, int operand_rows, const float* scale, int n_rows, int epi,
+                  uint16_t* out, int out_stride) {
+    PrefillGemmArgs a;
+    a.qw = t.q, a.scales = t.scales, a.biases = t.biases, a.N = N, a.K = K, a.operand = operand, a.operand_rows = operand_rows;
+    a.inv_scale = scale, a.rows = n_rows, a.epilogue = epi, a.out = out, a.out_stride = out_stride;
+    a.status = at<unsigned int>(m, lay.chain_status);
+    return a;
+  };
+
+#define Q4D_LAUNCH(cls, expr)                                                 \
+  do {                                                                        \
+    cudaError_t le = timed(m, cls, s, [&]() -> cudaError_t { return expr; }); \
+    if (le != cudaSuccess) return fail_cuda(le, #cls);                        \
+  } while (0)
+
+  Q4D_LAUNCH(Q4D_K_EMBED, launch_embed(m->w.embed.q, m->w.embed.scales, m->w.embed.biases, V, H, d_tokens, rows, x, s));
+  for (int l = 0; l < sh.n_layers; ++l) {
+    const q4d_layer_weights& lw = m->layers[l];
+    PrefillAttnArgs pa;
+    pa.qkv = qkv, pa.q = at<uint16_t>(m, lay.p_q), pa.q_norm = sh.qk_norm ? lw.q_norm : nullptr, pa.k_norm = sh.qk_norm ? lw.k_norm : nullptr;
+    pa.eps = sh.rms_eps, pa.rope = m->w.rope_cos_sin, pa.rows = rows, pa.start = start, pa.nq = nq, pa.nkv = nkv, pa.block_table = d_bt;
+    pa.kpool = pool->mem + (size_t)(2 * l) * layer_elems, pa.vpool = pa.kpool + layer_elems, pa.out = attn;
+    Q4D_LAUNCH(Q4D_K_RMSNORM, launch_prefill_pack(x, H, lw.attn_norm, sh.rms_eps, rows, H, nullptr, op, inv, s));
+    Q4D_LAUNCH(Q4D_K_GEMM_QKV, launch_prefill_gemm(gemm(lw.wqkv, nqkv, H, op, lay.p_rows, inv, rows, EPI_BF16, qkv, nqkv), s));
+    Q4D_LAUNCH(Q4D_K_ROPE_APPEND, launch_prefill_rope_append(pa, s));
+    if (l == sh.n_layers - 1 && !head) break;  // nothing reads the hidden state after the last layer's K, V
+    Q4D_LAUNCH(Q4D_K_ATTENTION, launch_prefill_attention(pa, s));
+    Q4D_LAUNCH(Q4D_K_ATTN_MERGE, launch_prefill_pack(attn, qdim, nullptr, 0.0f, rows, qdim, nullptr, op, inv, s));
+    Q4D_LAUNCH(Q4D_K_GEMM_O, launch_prefill_gemm(gemm(lw.wo, H, qdim, op, lay.p_rows, inv, rows, EPI_RESIDUAL, x, H), s));
+    if (sh.n_experts == 0) {
+      Q4D_LAUNCH(Q4D_K_RMSNORM, launch_prefill_pack(x, H, lw.mlp_norm, sh.rms_eps, rows, H, nullptr, op, inv, s));
+      Q4D_LAUNCH(Q4D_K_GEMM_GATE_UP, launch_prefill_gemm(gemm(lw.w_gate_up, 2 * I, H, op, lay.p_rows, inv, rows, EPI_SILU_PACK, h, I), s));
+      Q4D_LAUNCH(Q4D_K_GEMM_DOWN, launch_prefill_pack(h, I, nullptr, 0.0f, rows, I, nullptr, op, inv, s));
+      Q4D_LAUNCH(Q4D_K_GEMM_DOWN, launch_prefill_gemm(gemm(lw.w_down, H, I, op, lay.p_rows, inv, rows, EPI_RESIDUAL, x, H), s));
+    } else {
+      const int E = sh.n_experts, Ie = sh.expert_inter, pairs = rows * sh.top_k, cap = lay.p_rows * sh.top_k + 256;
+      PrefillMoeArgs mo;
+      mo.y = at<uint16_t>(m, lay.p_y), mo.router = lw.router, mo.rows = rows, mo.H = H, mo.E = E, mo.top_k = sh.top_k, mo.norm = sh.norm_topk_prob;
+      mo.idx = at<int32_t>(m, lay.p_idx), mo.wgt = at<float>(m, lay.p_wgt), mo.pos = at<int32_t>(m, lay.p_pos);
+      mo.counts = at<int32_t>(m, lay.p_counts), mo.cursor = at<int32_t>(m, lay.p_cursor);
+      mo.units = at<int4>(m, lay.p_units), mo.n_units = reinterpret_cast<int*>(mo.units + (E + cap / 16 + 1));
+      // a unit holds one and a half times an expert's share: most experts are one unit, and little of it is padding
+      mo.unit_rows = std::min(256, std::max(16, (pairs * 3 / (2 * E) + 15) / 16 * 16));
+      mo.operand = op, mo.inv_scale = inv, mo.sorted = at<uint16_t>(m, lay.p_pairs), mo.sorted_inv_scale = at<float>(m, lay.p_pairs_inv);
+      mo.o = mo.sorted, mo.x = x;
+      uint16_t *eh = at<uint16_t>(m, lay.p_eh), *eop = at<uint16_t>(m, lay.p_eop);
+      float* eop_inv = at<float>(m, lay.p_eop_inv);
+      Q4D_LAUNCH(Q4D_K_RMSNORM, launch_prefill_pack(x, H, lw.mlp_norm, sh.rms_eps, rows, H, at<uint16_t>(m, lay.p_y), op, inv, s));
+      Q4D_LAUNCH(Q4D_K_MOE_ROUTER, launch_prefill_route(mo, s));
+      m->launches += 2;
+      PrefillGemmArgs gu = gemm(lw.experts_gate_up, 2 * Ie, H, mo.sorted, cap, mo.sorted_inv_scale, pairs, EPI_SILU_PACK, eh, Ie);
+      gu.units = mo.units, gu.n_units = mo.n_units, gu.unit_rows = mo.unit_rows;
+      Q4D_LAUNCH(Q4D_K_MOE_GATE_UP, launch_prefill_gemm(gu, s));
+      Q4D_LAUNCH(Q4D_K_MOE_DOWN, launch_prefill_pack(eh, Ie, nullptr, 0.0f, pairs, Ie, nullptr, eop, eop_inv, s));
+      PrefillGemmArgs dn = gemm(lw.experts_down, H, Ie, eop, cap, eop_inv, pairs, EPI_BF16, mo.sorted, H);
+      dn.units = mo.units, dn.n_units = mo.n_units, dn.unit_rows = mo.unit_rows;
+      Q4D_LAUNCH(Q4D_K_MOE_DOWN, launch_prefill_gemm(dn, s));
+      Q4D_LAUNCH(Q4D_K_MOE_DOWN, launch_prefill_combine(mo, s));
+    }
+  }
+  if (head) {
+    uint16_t* yp = at<uint16_t>(m, lay.yp);
+    float* ys = at<float>(m, lay.ys);
+    float2* amax = at<float2>(m, lay.amax);
+    Q4D_LAUNCH(Q4D_K_RMSNORM, launch_rmsnorm(x + (size_t)(rows - 1) * H, m->w.final_norm, sh.rms_eps, 1, H, nullptr, yp, ys, gemm_operand_layout(false, 1), s));
+    GemmArgs lm = gemm_args(m, m->w.lm_head, V, H, yp, ys, 1, EPI_F32, logits_dev, V);
+    lm.argmax_partial = amax;
+    const int lm_blocks = gemm_row_blocks(V, H, 1, EPI_F32);
+    if (lm_blocks > lay.amax_blocks) return fail(Q4D_ERR_WORKSPACE_TOO_SMALL, "prefill: argmax scratch too small");
+    Q4D_LAUNCH(Q4D_K_LM_HEAD, launch_q4_gemm(lm, s));
+    Q4D_LAUNCH(Q4D_K_ARGMAX, launch_argmax_finish(amax, lm_blocks, 1, next_dev, s));
+  }
+#undef Q4D_LAUNCH
+  return read_back_status(m, s);
 }
 
 }  // namespace
@@ -718,6 +870,7 @@ int q4d_model_create(const q4d_shape* shape, const q4d_weights* weights, void* w
   if (const char* v = getenv("Q4D_NO_PDL")) set_pdl_enabled(v[0] == '0');
   cudaError_t e = gemm_init();
   if (e == cudaSuccess) e = attention_init();
+  if (e == cudaSuccess) e = prefill_init();
   if (e != cudaSuccess) return fail_cuda(e, "kernel init");
   const Workspace lay = carve(*shape, ml);
   if (workspace_bytes < lay.bytes)
@@ -752,6 +905,7 @@ int q4d_model_create(const q4d_shape* shape, const q4d_weights* weights, void* w
   if (e == cudaSuccess) e = cudaMemset(m->ws + lay.attn_merge_counters, 0, (size_t)16 * shape->n_kv_heads * 4);
   if (e == cudaSuccess && shape->n_experts)
     e = cudaMemset(m->ws + lay.m_ints, 0, (3 * (size_t)shape->n_experts + 3 + kMaxBatch) * 4);
+  if (e == cudaSuccess && shape->n_experts) e = cudaMemset(m->ws + lay.p_counts, 0, (size_t)shape->n_experts * 4);
   if (e == cudaSuccess) e = cudaMemset(m->ws + lay.chain_status, 0, 256);
   if (e == cudaSuccess) e = cudaMallocHost(reinterpret_cast<void**>(&m->host_status), sizeof(uint32_t));
   if (e == cudaSuccess) e = cudaEventCreateWithFlags(&m->status_done, cudaEventDisableTiming);
@@ -935,6 +1089,19 @@ int q4d_prefill(q4d_model* m, q4d_kv_pool* pool, int64_t request_id, const int32
   cudaStream_t s = static_cast<cudaStream_t>(stream);
   int32_t* ws_next = at<int32_t>(m, m->lay.next);
   float* ws_logits = at<float>(m, m->lay.logits);
+  const int widest = std::max(std::max(sh.hidden, sh.n_q_heads * kHeadDim), sh.n_experts ? sh.expert_inter : sh.mlp_inter);
+  // More tokens than one step's rows go through the prompt kernels (one pass over the weights per 2048 tokens); up to
+  // sixteen are one pass of the step's own kernels, which stream the weights faster than any wider tile.
+  if (n_tokens - start_pos > kMaxBatch && widest <= kPrefillMaxWidth) {
+    for (int c = start_pos; c < n_tokens; c += m->lay.p_rows) {
+      const int n = std::min(m->lay.p_rows, n_tokens - c);
+      const int rc = prefill_rows(m, pool, tokens + c, n, c, block_table, c + n == n_tokens, next_token ? next_token : ws_next,
+                                  logits ? logits : ws_logits, s);
+      if (rc != Q4D_OK) return rc;
+    }
+    pool->lens[request_id] = n_tokens;
+    return Q4D_OK;
+  }
   int last_rows = 0;
   for (int c = start_pos; c < n_tokens; c += kMaxBatch) {
     const int n = std::min(kMaxBatch, n_tokens - c);

@@ -181,6 +181,77 @@ struct MoeCombineArgs {
 cudaError_t launch_moe_router(const MoeRouteArgs& a, int n, cudaStream_t s);
 cudaError_t launch_moe_combine(const MoeCombineArgs& a, int n, cudaStream_t s);
 
+// ---- prompt processing (prefill.cu): many tokens of one request at once ------------------
+// Operand of a prompt projection: f16 [rows][prefill_operand_stride(K)], every row scaled by a power of two of its own
+// (inv_scale[row] undoes it): K features (chunks of 8 in the order 0,4,1,5,2,6,3,7), then the sums of every group of 64
+// features as two f16 terms, laid out against the biases and scales of the weights (see prefill.cu).
+constexpr int kPrefillChunk = 2048;      // tokens per pass over the weights
+constexpr int kPrefillMaxWidth = 32768;  // widest operand row
+__host__ __device__ __forceinline__ int prefill_operand_stride(int K) { return K + 64 * ((K + 1023) / 1024); }
+// rows of bf16 x (optionally RMS-normalised with w first, the normalised row also written to y) -> operand
+cudaError_t launch_prefill_pack(const uint16_t* x, int x_stride, const uint16_t* norm_w, float eps, int rows, int K,
+                                uint16_t* y, uint16_t* operand, float* inv_scale, cudaStream_t s);
+struct PrefillGemmArgs {
+  const uint32_t* qw;
+  const uint16_t* scales;
+  const uint16_t* biases;
+  int N, K;                // N a multiple of 128
+  const uint16_t* operand;
+  int operand_rows;        // rows the operand buffer holds (bound of the tensor map)
+  const float* inv_scale;
+  int rows;                // tokens
+  int epilogue;            // EPI_BF16, EPI_RESIDUAL, or EPI_SILU_PACK: h = silu(gate) * up, plain bf16 [rows][N / 2]
+  uint16_t* out;
+  int out_stride;
+  unsigned int* status;
+  // grouped mode (mixture of experts): `units` is a device list of {expert, first operand row, rows <= unit_rows, 0}
+  const int4* units = nullptr;
+  const int* n_units = nullptr;
+  int unit_rows = 0;
+};
+cudaError_t launch_prefill_gemm(const PrefillGemmArgs& a, cudaStream_t s);
+struct PrefillAttnArgs {
+  const uint16_t* qkv;     // bf16 [rows][(nq + 2 nkv) * 128]
+  uint16_t* q;             // bf16 [rows][nq][128] scratch: prepared queries
+  const uint16_t* q_norm;  // or NULL
+  const uint16_t* k_norm;
+  float eps;
+  const float* rope;
+  int rows, start;         // row r is the token at position start + r
+  int nq, nkv;
+  const int32_t* block_table;
+  uint16_t* kpool;         // this layer of the pool
+  uint16_t* vpool;
+  uint16_t* out;           // bf16 [rows][nq][128]
+};
+cudaError_t launch_prefill_rope_append(const PrefillAttnArgs& a, cudaStream_t s);
+cudaError_t launch_prefill_attention(const PrefillAttnArgs& a, cudaStream_t s);
+cudaError_t prefill_init();
+
+// Routing of many tokens: the experts of each token, then every (token, expert) pair as a row of an operand sorted by
+// expert, and the list of units (runs of at most unit_rows rows of one expert) the grouped projections walk.
+struct PrefillMoeArgs {
+  const uint16_t* y;       // normed hidden state bf16 [rows][H]
+  const uint16_t* router;  // bf16 [E][H]
+  int rows, H, E, top_k, norm;
+  int32_t* idx;            // [rows][top_k]
+  float* wgt;              // [rows][top_k]
+  int32_t* pos;            // [rows][top_k]: row of the pair in the sorted operand
+  int32_t* counts;         // [E], zero between calls
+  int32_t* cursor;         // [E]
+  int4* units;
+  int* n_units;
+  int unit_rows;
+  const uint16_t* operand; // operand of the tokens and its scales
+  const float* inv_scale;
+  uint16_t* sorted;        // operand of the pairs and its scales
+  float* sorted_inv_scale;
+  const uint16_t* o;       // expert outputs bf16 [pairs][H]
+  uint16_t* x;             // residual stream bf16 [rows][H], updated in place
+};
+cudaError_t launch_prefill_route(const PrefillMoeArgs& a, cudaStream_t s);    // idx, wgt, counts -> units -> sorted operand
+cudaError_t launch_prefill_combine(const PrefillMoeArgs& a, cudaStream_t s);
+
 // ---- sampling ------------------------------------------------------------------------
 struct SampleArgs {  // passed to the kernel by value: the per-request settings travel with the launch
   const float* logits;  // f32 [n][vocab]

@@ -27,14 +27,13 @@
 //
 // K is cut into parts across CTAs where the tiles alone would not fill the machine; the parts of a tile meet in
 // global scratch and the last CTA to arrive adds them in part order (deterministic) and applies the epilogue.
-#include <cuda.h>
-
 #include <mutex>
 #include <unordered_map>
 
 #include "common.cuh"
 #include "kernels.h"
 #include "launch.h"
+#include "tcgen05.cuh"
 
 namespace q4d {
 
@@ -73,59 +72,6 @@ __device__ __forceinline__ uint32_t and_or(uint32_t a, uint32_t b, uint32_t c) {
   return d;
 }
 
-__device__ __forceinline__ void um_mbar_init(uint64_t* bar, uint32_t count) {
-  asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(smem_u32(bar)), "r"(count) : "memory");
-}
-__device__ __forceinline__ void um_mbar_arrive(uint64_t* bar) {
-  asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(smem_u32(bar)) : "memory");
-}
-__device__ __forceinline__ void um_mbar_expect_tx(uint64_t* bar, uint32_t bytes) {
-  asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(smem_u32(bar)), "r"(bytes) : "memory");
-}
-__device__ __forceinline__ void um_bulk_g2s(void* smem_dst, const void* gsrc, uint32_t bytes, uint64_t* bar) {
-  asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(
-                   smem_u32(smem_dst)),
-               "l"(gsrc), "r"(bytes), "r"(smem_u32(bar))
-               : "memory");
-}
-// A box of the tensor map at element (x, row y) into shared memory (this GPU's memory only, no multicast).
-__device__ __forceinline__ void um_tma_2d(void* smem_dst, const CUtensorMap* map, int x, int y, uint64_t* bar) {
-  asm volatile("cp.async.bulk.tensor.2d.shared::cluster.global.tile.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3}], [%4];" ::"r"(
-                   smem_u32(smem_dst)),
-               "l"(reinterpret_cast<uint64_t>(map)), "r"(x), "r"(y), "r"(smem_u32(bar))
-               : "memory");
-}
-// Waits for the phase of the given parity.  Each try suspends the thread in hardware until the phase completes or the
-// hint (in nanoseconds) runs out, so that waiting warps do not occupy issue slots and the shared-memory pipeline;
-// gives up (false) after a bounded number of tries (about two seconds).
-__device__ __forceinline__ bool um_mbar_wait(uint64_t* bar, uint32_t parity) {
-  for (int tries = 0; tries < 20000; ++tries) {
-    uint32_t done;
-    asm volatile(
-        "{\n\t.reg .pred p;\n\tmbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2, %3;\n\tselp.u32 %0, 1, 0, p;\n\t}"
-        : "=r"(done)
-        : "r"(smem_u32(bar)), "r"(parity), "r"(100000u)
-        : "memory");
-    if (done) return true;
-  }
-  return false;
-}
-// The same for a whole warp: every lane polls, the verdict is the warp's (uniform control flow for the callers).
-__device__ __forceinline__ bool um_mbar_wait_warp(uint64_t* bar, uint32_t parity) {
-  for (int tries = 0; tries < 20000; ++tries) {
-    uint32_t done;
-    asm volatile(
-        "{\n\t.reg .pred p;\n\tmbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2, %3;\n\tselp.u32 %0, 1, 0, p;\n\t}"
-        : "=r"(done)
-        : "r"(smem_u32(bar)), "r"(parity), "r"(100000u)
-        : "memory");
-    if (__all_sync(0xffffffffu, done != 0u)) return true;
-  }
-  return false;
-}
-__device__ __forceinline__ void tc_fence_before() { asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory"); }
-__device__ __forceinline__ void tc_fence_after() { asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory"); }
-
 // D(128 x 16, f32, tensor memory) (+)= A(128 x 16 bf16, tensor memory) * B(16 x 16 bf16, shared memory, K-major)
 __device__ __forceinline__ void umma_bf16(uint32_t d_tmem, uint32_t a_tmem, uint64_t b_desc, uint32_t idesc, uint32_t accumulate) {
   asm volatile(
@@ -133,10 +79,6 @@ __device__ __forceinline__ void umma_bf16(uint32_t d_tmem, uint32_t a_tmem, uint
       "r"(a_tmem), "l"(b_desc), "r"(idesc), "r"(accumulate)
       : "memory");
 }
-__device__ __forceinline__ void umma_commit(uint64_t* bar) {
-  asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(smem_u32(bar)) : "memory");
-}
-
 __device__ __forceinline__ void tmem_st32(uint32_t taddr, const uint32_t (&r)[32]) {
   asm volatile(
       "tcgen05.st.sync.aligned.32x32b.x32.b32 [%0], {%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15,%16,%17,%18,%19,%20,%21,"
@@ -522,10 +464,6 @@ q4_umma_kernel(const UmmaParams p, const __grid_constant__ CUtensorMap map_codes
 }
 
 // ---- tensor maps of the packed codes, one per tensor, made on first use ----
-typedef CUresult (*EncodeTiledFn)(CUtensorMap*, CUtensorMapDataType, cuuint32_t, void*, const cuuint64_t*, const cuuint64_t*,
-                                  const cuuint32_t*, const cuuint32_t*, CUtensorMapInterleave, CUtensorMapSwizzle,
-                                  CUtensorMapL2promotion, CUtensorMapFloatOOBfill);
-
 struct MapKey {
   const void* ptr;
   long long rows, row_bytes;
@@ -539,7 +477,6 @@ struct MapKeyHash {
 
 std::mutex g_map_mutex;
 std::unordered_map<MapKey, CUtensorMap, MapKeyHash> g_maps;
-EncodeTiledFn g_encode = nullptr;
 bool g_umma_init = false;
 
 // The packed codes as a 2-D byte tensor [rows][K/2]; a box is 64 rows x 128 bytes (256 codes), 128-byte swizzle.
@@ -552,20 +489,15 @@ cudaError_t codes_map(const uint32_t* qw, long long rows, int K, CUtensorMap* ou
     *out = it->second;
     return cudaSuccess;
   }
-  if (!g_encode) {
-    void* fn = nullptr;
-    cudaDriverEntryPointQueryResult qres;
-    cudaError_t e = cudaGetDriverEntryPointByVersion("cuTensorMapEncodeTiled", &fn, 12000, cudaEnableDefault, &qres);
-    if (e != cudaSuccess) return e;
-    if (qres != cudaDriverEntryPointSuccess || !fn) return cudaErrorNotSupported;
-    g_encode = reinterpret_cast<EncodeTiledFn>(fn);
-  }
+  EncodeTiledFn encode = nullptr;
+  const cudaError_t ee = encode_tiled_fn(&encode);
+  if (ee != cudaSuccess) return ee;
   if (reinterpret_cast<uintptr_t>(qw) % 16 || (K / 2) % 16) return cudaErrorInvalidValue;
   const cuuint64_t dims[2] = {(cuuint64_t)(K / 2), (cuuint64_t)rows};
   const cuuint64_t strides[1] = {(cuuint64_t)(K / 2)};
   const cuuint32_t box[2] = {128u, 64u}, elem[2] = {1u, 1u};
   CUtensorMap m;
-  const CUresult r = g_encode(&m, CU_TENSOR_MAP_DATA_TYPE_UINT8, 2, const_cast<uint32_t*>(qw), dims, strides, box, elem,
+  const CUresult r = encode(&m, CU_TENSOR_MAP_DATA_TYPE_UINT8, 2, const_cast<uint32_t*>(qw), dims, strides, box, elem,
                               CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_128B,
                               CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
   if (r != CUDA_SUCCESS) return cudaErrorInvalidValue;
