@@ -170,7 +170,7 @@ def gemm_only(args):
     by = N * K * 0.5625
     peak, kind = peaks()
     print(json.dumps({"op": "q4_gemm", "N": N, "K": K, "n": n, "epilogue": "f32", "calls": args.steps,
-                      "kernel": "q4_umma_kernel" if os.environ.get("Q4D_GEMM_KERNEL") == "tcgen05" else "span/round",
+                      "kernel": "q4_umma_kernel" if os.environ.get("Q4D_GEMM_KERNEL") == "tcgen05" else "q4_slice_kernel",
                       "us_per_call": us, "GBps": by / us / 1e3, "frac_of_peak": by / us / 1e3 / peak, "peak_kind": kind,
                       "note": "a call = operand rearrangement kernel + projection kernel"}))
     return 0
@@ -445,17 +445,17 @@ def main():
         if shape.n_experts:  # distinct experts per layer, counted from the routing of the profiled steps
             class_bytes["moe_gate_up"] = touched["mean"] * shp.q4_bytes(2 * shape.expert_inter, H)
             class_bytes["moe_down"] = touched["mean"] * shp.q4_bytes(H, shape.expert_inter)
-        proj = "q4_umma_kernel" if os.environ.get("Q4D_GEMM_KERNEL") == "tcgen05" else "q4_span_kernel"
-        head = "q4_umma_kernel" if os.environ.get("Q4D_GEMM_KERNEL") == "tcgen05" else "q4_round_kernel"
+        proj = "q4_umma_kernel" if os.environ.get("Q4D_GEMM_KERNEL") == "tcgen05" else "q4_slice_kernel"
+        head = "q4_umma_kernel" if os.environ.get("Q4D_GEMM_KERNEL") == "tcgen05" else "q4_slice_kernel"
         class_kernel = {"gemm_qkv": proj, "gemm_o": proj, "gemm_gate_up": proj, "gemm_down": proj, "lm_head": head,
                         "attention": ("paged_attention_t_kernel" if shape.n_q_heads // shape.n_kv_heads <= 8
-                                      else "paged_attention_kernel"), "moe_gate_up": "q4_gemm_kernel",
-                        "moe_down": "q4_gemm_kernel", "rmsnorm": "rmsnorm_kernel", "embed": "embed_kernel",
+                                      else "paged_attention_kernel"), "moe_gate_up": "q4_grouped_kernel",
+                        "moe_down": "q4_grouped_kernel", "rmsnorm": "rmsnorm_kernel", "embed": "embed_kernel",
                         "argmax": "argmax_finish_kernel", "moe_router": "moe_router_kernel"}
         # DRAM bytes per algorithmic byte from one `ncu --set full` capture of each kernel (see profiles/: the span kernel
         # on a gate/up-shaped projection alone, attention on the Llama-3.2-3B-shaped batch-16 case); traffic is
         # proportional to the bytes streamed, so it is scaled to this launch.
-        traffic_ratio = {"q4_span_kernel": 1.005, "paged_attention_t_kernel": 1.037}
+        traffic_ratio = {"q4_slice_kernel": 1.005, "paged_attention_t_kernel": 1.037}
         total_prof_ms = sum(v[0] for v in prof.values())
         classes = {k: {"ms_per_step": v[0] / args.profile_steps, "launches_per_step": v[1] / args.profile_steps,
                        "share": v[0] / total_prof_ms, "kernel": class_kernel.get(k, k)} for k, v in prof.items() if v[1]}

@@ -61,7 +61,7 @@ struct MetaLayout {
 };
 
 struct Workspace {
-  // x: residual stream (plain).  yp/ys, ap/as, hp/hs: GEMM operands in fragment order with their group sums
+  // x: residual stream (plain); yp/ys, ap/as, hp/hs: GEMM operands in fragment order with their group sums
   // (normed hidden state, attention output, silu(gate)*up).
   size_t x, yp, ys, qkv, qbuf, ap, as, hp, hs, logits, next, amax, gemm_partial, gemm_partial_bytes, counters,
       part_acc, part_ml, attn_merge_counters, meta, bytes;
@@ -137,14 +137,14 @@ Workspace carve(const q4d_shape& s, const MetaLayout& ml) {
   const int nqkv = (s.n_q_heads + 2 * s.n_kv_heads) * kHeadDim;
   const size_t qdim = (size_t)s.n_q_heads * kHeadDim;
   w.x = take(B * s.hidden * 2);
-  w.yp = take(operand_elements(OPERAND_SLICED, s.hidden) * 2);  // the largest of the layouts
-  w.ys = take((size_t)(s.hidden / 64) * 16 * 4);
+  w.yp = take(B * s.hidden * 2);
+  w.ys = take(operand_sums_bytes(s.hidden));
   w.qkv = take(B * nqkv * 2);
   w.qbuf = take(B * qdim * 2);
-  w.ap = take(operand_elements(OPERAND_SLICED, qdim) * 2);
-  w.as = take((qdim / 64) * 16 * 4);
-  w.hp = take(operand_elements(OPERAND_SLICED, s.mlp_inter) * 2 + 256);
-  w.hs = take((size_t)(s.mlp_inter / 64) * 16 * 4 + 256);
+  w.ap = take(B * qdim * 2);
+  w.as = take(operand_sums_bytes((int)qdim));
+  w.hp = take(B * s.mlp_inter * 2 + 256);
+  w.hs = take(operand_sums_bytes(s.mlp_inter) + 256);
   w.yplain = w.m_idx = w.m_wgt = w.m_ints = w.m_hp = w.m_hs = w.m_o = 0;
   if (s.n_experts) {
     const size_t E = s.n_experts;
@@ -154,7 +154,7 @@ Workspace carve(const q4d_shape& s, const MetaLayout& ml) {
     // flags[E], expert_ids[E], slot_of[E], counter, n_touched, touched_total, slice_counter[16], then logits[16][E]
     w.m_ints = take((3 * E + 3 + kMaxBatch) * 4 + B * E * 4);
     w.m_hp = take(E * B * s.expert_inter * 2);
-    w.m_hs = take(E * (size_t)(s.expert_inter / 64) * 16 * 4);
+    w.m_hs = take(E * operand_sums_bytes(s.expert_inter));
     w.m_o = take(E * B * s.hidden * 2);
   }
   w.logits = take(B * (size_t)s.vocab * 4);
@@ -242,6 +242,7 @@ struct q4d_model {
   q4d_shape sh;
   std::vector<q4d_layer_weights> layers;
   q4d_weights w;
+  std::vector<GemmMaps> maps;  // of the dense projections: 4 per layer (qkv, o, gate/up, down), then the head
   unsigned char* ws;
   Workspace lay;
   MetaLayout ml;
@@ -308,9 +309,10 @@ cudaError_t timed(q4d_model* m, int cls, cudaStream_t s, F&& f) {
   return e;
 }
 
-GemmArgs gemm_args(q4d_model* m, const q4d_qtensor& t, int N, int K, const uint16_t* xp, const float* xs, int n,
-                   int epi, void* out, int out_stride) {
+GemmArgs gemm_args(q4d_model* m, const q4d_qtensor& t, int N, int K, const uint16_t* xp, const void* xs, int n,
+                   int epi, void* out, int out_stride, int map) {
   GemmArgs a;
+  a.maps = map >= 0 ? &m->maps[map] : nullptr;
   a.qw = t.q, a.scales = t.scales, a.biases = t.biases;
   a.N = N, a.K = K, a.xp = xp, a.xs = xs, a.n = n, a.epilogue = epi;
   a.out = out, a.out_stride = out_stride;
@@ -589,18 +591,18 @@ int step_impl(q4d_model* m, q4d_kv_pool* pool, int32_t n, const int64_t* ids, co
   const int nqkv = (nq + 2 * nkv) * kHeadDim;
   uint16_t* x = at<uint16_t>(m, m->lay.x);
   uint16_t* yp = at<uint16_t>(m, m->lay.yp);
-  float* ys = at<float>(m, m->lay.ys);
+  void* ys = at<unsigned char>(m, m->lay.ys);
   uint16_t* qkv = at<uint16_t>(m, m->lay.qkv);
   uint16_t* qbuf = at<uint16_t>(m, m->lay.qbuf);
   uint16_t* ap = at<uint16_t>(m, m->lay.ap);
-  float* as = at<float>(m, m->lay.as);
+  void* as = at<unsigned char>(m, m->lay.as);
   uint16_t* hp = at<uint16_t>(m, m->lay.hp);
-  float* hs = at<float>(m, m->lay.hs);
+  void* hs = at<unsigned char>(m, m->lay.hs);
   float2* amax = at<float2>(m, m->lay.amax);
   float* logits = logits_dev ? logits_dev : at<float>(m, m->lay.logits);
   const size_t layer_elems = (size_t)pool->num_blocks * nkv * kBlockSize * kHeadDim;
   const int qdim = nq * kHeadDim;
-  const int dense_layout = gemm_operand_layout(false, n);  // of the operands of the dense projections
+  const int dense_layout = gemm_operand_layout(false);  // of the operands of the dense projections
 
 #define Q4D_LAUNCH(cls, expr)                                                 \
   do {                                                                        \
@@ -623,7 +625,7 @@ int step_impl(q4d_model* m, q4d_kv_pool* pool, int32_t n, const int64_t* ids, co
     uint16_t* kpool = pool->mem + (size_t)(2 * l) * layer_elems;
     uint16_t* vpool = kpool + layer_elems;
     Q4D_LAUNCH(Q4D_K_RMSNORM, launch_rmsnorm(x, lw.attn_norm, sh.rms_eps, n, H, nullptr, yp, ys, dense_layout, s));
-    Q4D_LAUNCH(Q4D_K_GEMM_QKV, launch_q4_gemm(gemm_args(m, lw.wqkv, nqkv, H, yp, ys, n, EPI_BF16, qkv, nqkv), s));
+    Q4D_LAUNCH(Q4D_K_GEMM_QKV, launch_q4_gemm(gemm_args(m, lw.wqkv, nqkv, H, yp, ys, n, EPI_BF16, qkv, nqkv, 4 * l), s));
     AttnArgs aa;
     aa.q = qbuf, aa.kpool = kpool, aa.vpool = vpool, aa.block_tables = d_bt, aa.lens = d_lens;
     aa.work = reinterpret_cast<const int4*>(dmeta + ml.off_work);
@@ -646,13 +648,13 @@ int step_impl(q4d_model* m, q4d_kv_pool* pool, int32_t n, const int64_t* ids, co
       aa.qkv = nullptr, aa.after_predecessor = true;
     }
     Q4D_LAUNCH(Q4D_K_ATTENTION, launch_paged_attention(aa, s));
-    Q4D_LAUNCH(Q4D_K_GEMM_O, launch_q4_gemm(gemm_args(m, lw.wo, H, qdim, ap, as, n, EPI_RESIDUAL, x, H), s));
+    Q4D_LAUNCH(Q4D_K_GEMM_O, launch_q4_gemm(gemm_args(m, lw.wo, H, qdim, ap, as, n, EPI_RESIDUAL, x, H, 4 * l + 1), s));
     if (sh.n_experts == 0) {
       Q4D_LAUNCH(Q4D_K_RMSNORM, launch_rmsnorm(x, lw.mlp_norm, sh.rms_eps, n, H, nullptr, yp, ys, dense_layout, s));
-      GemmArgs gu = gemm_args(m, lw.w_gate_up, 2 * I, H, yp, ys, n, EPI_SILU_PACK, nullptr, 0);
+      GemmArgs gu = gemm_args(m, lw.w_gate_up, 2 * I, H, yp, ys, n, EPI_SILU_PACK, nullptr, 0, 4 * l + 2);
       gu.out_xp = hp, gu.out_xs = hs;
       Q4D_LAUNCH(Q4D_K_GEMM_GATE_UP, launch_q4_gemm(gu, s));
-      Q4D_LAUNCH(Q4D_K_GEMM_DOWN, launch_q4_gemm(gemm_args(m, lw.w_down, H, I, hp, dense_layout == OPERAND_BLOCKED ? hs : nullptr, n, EPI_RESIDUAL, x, H), s));
+      Q4D_LAUNCH(Q4D_K_GEMM_DOWN, launch_q4_gemm(gemm_args(m, lw.w_down, H, I, hp, dense_layout == OPERAND_BLOCKED ? hs : nullptr, n, EPI_RESIDUAL, x, H, 4 * l + 3), s));
     } else {
       const int E = sh.n_experts, Ie = sh.expert_inter;
       uint16_t* yplain = at<uint16_t>(m, m->lay.yplain);
@@ -666,18 +668,18 @@ int step_impl(q4d_model* m, q4d_kv_pool* pool, int32_t n, const int64_t* ids, co
       mr.slice_counter = ints + 3 * E + 3;
       mr.logits = reinterpret_cast<float*>(ints + 3 * E + 3 + kMaxBatch);
       uint16_t* ehp = at<uint16_t>(m, m->lay.m_hp);
-      float* ehs = at<float>(m, m->lay.m_hs);
+      void* ehs = at<unsigned char>(m, m->lay.m_hs);
       uint16_t* eo = at<uint16_t>(m, m->lay.m_o);
-      Q4D_LAUNCH(Q4D_K_RMSNORM, launch_rmsnorm(x, lw.mlp_norm, sh.rms_eps, n, H, yplain, yp, ys, gemm_operand_layout(true, n), s));
+      Q4D_LAUNCH(Q4D_K_RMSNORM, launch_rmsnorm(x, lw.mlp_norm, sh.rms_eps, n, H, yplain, yp, ys, gemm_operand_layout(true), s));
       Q4D_LAUNCH(Q4D_K_MOE_ROUTER, launch_moe_router(mr, n, s));
-      GemmArgs gu = gemm_args(m, lw.experts_gate_up, 2 * Ie, H, yp, ys, n, EPI_SILU_PACK, nullptr, 0);
+      GemmArgs gu = gemm_args(m, lw.experts_gate_up, 2 * Ie, H, yp, ys, n, EPI_SILU_PACK, nullptr, 0, -1);
       gu.out_xp = ehp, gu.out_xs = ehs;
       gu.expert_ids = mr.expert_ids, gu.n_touched = mr.n_touched, gu.max_slots = E;
-      gu.out_slot_stride = (size_t)16 * Ie, gu.out_xs_slot_stride = (size_t)(Ie / 64) * 16;
+      gu.out_slot_stride = (size_t)16 * Ie, gu.out_xs_slot_stride = operand_sums_bytes(Ie);
       Q4D_LAUNCH(Q4D_K_MOE_GATE_UP, launch_q4_gemm(gu, s));
-      GemmArgs dn = gemm_args(m, lw.experts_down, H, Ie, ehp, ehs, n, EPI_BF16, eo, H);
+      GemmArgs dn = gemm_args(m, lw.experts_down, H, Ie, ehp, ehs, n, EPI_BF16, eo, H, -1);
       dn.expert_ids = mr.expert_ids, dn.n_touched = mr.n_touched, dn.max_slots = E;
-      dn.xp_slot_stride = (size_t)16 * Ie, dn.xs_slot_stride = (size_t)(Ie / 64) * 16;
+      dn.xp_slot_stride = (size_t)16 * Ie, dn.xs_slot_stride = operand_sums_bytes(Ie);
       dn.out_slot_stride = (size_t)16 * H;
       Q4D_LAUNCH(Q4D_K_MOE_DOWN, launch_q4_gemm(dn, s));
       MoeCombineArgs mc;
@@ -691,7 +693,7 @@ int step_impl(q4d_model* m, q4d_kv_pool* pool, int32_t n, const int64_t* ids, co
   }
   if (pf && !pf->want_head) return Q4D_OK;  // an inner chunk of a prompt: its K, V are in the pool, nothing else is needed
   Q4D_LAUNCH(Q4D_K_RMSNORM, launch_rmsnorm(x, m->w.final_norm, sh.rms_eps, n, H, nullptr, yp, ys, dense_layout, s));
-  GemmArgs lm = gemm_args(m, m->w.lm_head, V, H, yp, ys, n, EPI_F32, logits, V);
+  GemmArgs lm = gemm_args(m, m->w.lm_head, V, H, yp, ys, n, EPI_F32, logits, V, 4 * sh.n_layers);
   lm.argmax_partial = amax;
   const int lm_blocks = gemm_row_blocks(V, H, n, EPI_F32);
   if (lm_blocks > m->lay.amax_blocks) return fail(Q4D_ERR_WORKSPACE_TOO_SMALL, "decode_step: argmax scratch too small");
@@ -808,10 +810,10 @@ int prefill_rows(q4d_model* m, q4d_kv_pool* pool, const int32_t* tokens, int row
   }
   if (head) {
     uint16_t* yp = at<uint16_t>(m, lay.yp);
-    float* ys = at<float>(m, lay.ys);
+    void* ys = at<unsigned char>(m, lay.ys);
     float2* amax = at<float2>(m, lay.amax);
-    Q4D_LAUNCH(Q4D_K_RMSNORM, launch_rmsnorm(x + (size_t)(rows - 1) * H, m->w.final_norm, sh.rms_eps, 1, H, nullptr, yp, ys, gemm_operand_layout(false, 1), s));
-    GemmArgs lm = gemm_args(m, m->w.lm_head, V, H, yp, ys, 1, EPI_F32, logits_dev, V);
+    Q4D_LAUNCH(Q4D_K_RMSNORM, launch_rmsnorm(x + (size_t)(rows - 1) * H, m->w.final_norm, sh.rms_eps, 1, H, nullptr, yp, ys, gemm_operand_layout(false), s));
+    GemmArgs lm = gemm_args(m, m->w.lm_head, V, H, yp, ys, 1, EPI_F32, logits_dev, V, 4 * sh.n_layers);
     lm.argmax_partial = amax;
     const int lm_blocks = gemm_row_blocks(V, H, 1, EPI_F32);
     if (lm_blocks > lay.amax_blocks) return fail(Q4D_ERR_WORKSPACE_TOO_SMALL, "prefill: argmax scratch too small");
@@ -881,6 +883,20 @@ int q4d_model_create(const q4d_shape* shape, const q4d_weights* weights, void* w
   m->layers.assign(weights->layers, weights->layers + shape->n_layers);
   m->w = *weights;
   m->w.layers = m->layers.data();
+  {
+    const int H = shape->hidden, qdim = shape->n_q_heads * kHeadDim, nqkv = (shape->n_q_heads + 2 * shape->n_kv_heads) * kHeadDim;
+    m->maps.resize(4 * (size_t)shape->n_layers + 1);
+    for (int l = 0; l < shape->n_layers; ++l) {
+      const q4d_layer_weights& lw = m->layers[l];
+      GemmMaps* mp = m->maps.data() + 4 * l;
+      if (e == cudaSuccess) e = gemm_make_maps(lw.wqkv.q, lw.wqkv.scales, lw.wqkv.biases, nqkv, H, false, mp);
+      if (e == cudaSuccess) e = gemm_make_maps(lw.wo.q, lw.wo.scales, lw.wo.biases, H, qdim, false, mp + 1);
+      if (shape->n_experts) continue;
+      if (e == cudaSuccess) e = gemm_make_maps(lw.w_gate_up.q, lw.w_gate_up.scales, lw.w_gate_up.biases, 2 * (long long)shape->mlp_inter, H, true, mp + 2);
+      if (e == cudaSuccess) e = gemm_make_maps(lw.w_down.q, lw.w_down.scales, lw.w_down.biases, H, shape->mlp_inter, false, mp + 3);
+    }
+    if (e == cudaSuccess) e = gemm_make_maps(m->w.lm_head.q, m->w.lm_head.scales, m->w.lm_head.biases, shape->vocab, H, false, &m->maps.back());
+  }
   m->ws = static_cast<unsigned char*>(workspace);
   m->lay = lay;
   m->ml = ml;
@@ -1234,8 +1250,8 @@ constexpr size_t kOpAttnMeta = 1ull << 20;
 constexpr size_t kOpPartAcc = 64ull << 20;
 constexpr size_t kOpPartMl = 1ull << 20;
 constexpr int kOpMaxK = 32768;                         // widest operand the pack buffers hold
-constexpr size_t kOpPackXp = (size_t)16 * kOpMaxK * 2 + kOpMaxK;  // fragment-ordered operand, with the sliced layout's padding
-constexpr size_t kOpPackXs = (size_t)(kOpMaxK / 64) * 16 * 4;
+constexpr size_t kOpPackXp = (size_t)16 * kOpMaxK * 2;  // operand
+constexpr size_t kOpPackXs = (size_t)(kOpMaxK / 256) * 16 * 32;
 constexpr size_t kOpPackOff = kOpCounters + kOpGemmPartial + kOpAttnMeta + kOpPartAcc + kOpPartMl;
 }  // namespace
 
@@ -1253,9 +1269,9 @@ int q4d_q4_gemm(const q4d_qtensor* w, int32_t N, int32_t K, const uint16_t* x, i
     return fail(Q4D_ERR_WORKSPACE_TOO_SMALL, "q4_gemm: shape needs more scratch than q4d_op_scratch_bytes provides");
   unsigned char* sc = static_cast<unsigned char*>(scratch);
   uint16_t* xp = reinterpret_cast<uint16_t*>(sc + kOpPackOff);
-  float* xs = reinterpret_cast<float*>(sc + kOpPackOff + kOpPackXp);
+  void* xs = reinterpret_cast<void*>(sc + kOpPackOff + kOpPackXp);
   cudaStream_t st = static_cast<cudaStream_t>(stream);
-  cudaError_t e = launch_pack_operand(x, x_stride, K, n, prologue, xp, xs, gemm_operand_layout(false, n), st);
+  cudaError_t e = launch_pack_operand(x, x_stride, K, n, prologue, xp, xs, gemm_operand_layout(false), st);
   if (e != cudaSuccess) return fail_cuda(e, "q4_gemm (operand)");
   GemmArgs a;
   a.qw = w->q, a.scales = w->scales, a.biases = w->biases, a.N = N, a.K = K, a.xp = xp, a.xs = xs, a.n = n;

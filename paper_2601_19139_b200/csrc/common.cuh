@@ -1,5 +1,6 @@
 // Shared device helpers of the q4decode kernels (sm_100a).
 #pragma once
+#include <cuda_bf16.h>
 #include <cuda_runtime.h>
 #include <stdint.h>
 
@@ -76,22 +77,28 @@ __device__ __forceinline__ void ldmatrix_x4_trans(uint32_t (&r)[4], const void* 
 }
 
 // ---- fragment-ordered GEMM operand ---------------------------------------------------
-// The GEMM reads its activations as bf16 [16][K] with every aligned chunk of 8 elements stored in the order
-// {0,4,1,5,2,6,3,7} (so that a lane's 16 bytes are its B fragments of two k-steps), plus the fp32 sum of every
-// group of 64 elements, [K/64][16].  Producers build both with these helpers, always with the same summation
-// tree: ((e0+e1)+(e2+e3))+((e4+e5)+(e6+e7)) per chunk, then a pairwise tree over the 8 chunks of the group.
-// Element offset of chunk c (8 features) of request r in an operand of K features.  Layout 0 is [16][K]; layout 1 is
-// [K/8][16][8] (all requests of a chunk side by side: the tensor-core kernel copies a K-range as one block); layout
-// 2 is [K/ks][16][ks + 8]: K cut into slices of ks features (operand_slice_features), the 16 rows of a slice side by
-// side, each followed by 8 unused elements -- byte for byte the shared-memory image the mma.sync kernels want (rows
-// 16 bytes apart modulo 128 for conflict-free fragment loads), so that a CTA stages a slice with ONE bulk copy: the
-// time to stage an operand is set by the number of copies, not by their bytes.
+// The GEMM reads its activations as bf16 with every aligned chunk of 8 elements stored in the order {0,4,1,5,2,6,3,7}
+// (so that a lane's 16 bytes are its B fragments of two k-steps), plus the sum of every group of 64 elements.
+// Producers build both with these helpers, always with the same summation tree: ((e0+e1)+(e2+e3))+((e4+e5)+(e6+e7))
+// per chunk, then a pairwise tree over the 8 chunks of the group.
+//
+// Scaling (the mma.sync kernels, OPERAND_ROWS and OPERAND_FRAG).  Those kernels hand the packed codes to the tensor cores as they
+// lie in the word: a 4-bit code in bits 0..3 of a half-word IS the bf16 subnormal q * 2^-133, and one in bits 4..7 is
+// 16 q * 2^-133 (bits 0..7 of bf16 count in steps of 2^-133: the first normal binade has the subnormals' spacing), so
+// unpacking is one AND.  The powers of two go into the activations, exactly: elements 0, 2, 4, 6 of a chunk are stored
+// times 2^64, elements 1, 3, 5, 7 times 2^60.  A product then counts in 2^-69, which the fp32 result loses at the end;
+// activations from 2^-50 to 2^63 keep every bit.  The group sums (times 2^-69) are three bf16 terms, 24 bits, laid out as
+// a B fragment against the biases: 16 values per (256 features, request), 4 per lane t of a fragment row.
+constexpr float kOperandUnscale = 590295810358705651712.0f;            // 2^69
+constexpr float kOperandSumScale = 1.0f / 590295810358705651712.0f;    // 2^-69
+constexpr int kOperandSumBytes = 32;                                    // per (256 features, request)
+// Element offset of chunk c (8 features) of request r in an operand of K features: OPERAND_ROWS is [16][K];
+// OPERAND_BLOCKED is [K/8][16][8] (all requests of a chunk side by side: the tcgen05 kernel copies a K-range as one
+// block); OPERAND_FRAG is [K/64][2][2][32][8]: per group of 64 features and 8 requests, the two 16-byte halves that lane
+// 4 (r % 8) + (c % 8) / 2 of a warp holds as its B fragments, 512 contiguous bytes per half.
 __device__ __forceinline__ size_t operand_chunk_offset(int layout, int K, int r, int c) {
-  if (layout == 2) {
-    const int ks = operand_slice_features(K), k = c * 8, sl = k / ks;
-    return ((size_t)sl * 16 + r) * (ks + 8) + (k - sl * ks);
-  }
-  return layout ? ((size_t)c * 16 + r) * 8 : (size_t)r * K + (size_t)c * 8;
+  if (layout == OPERAND_FRAG) return (((size_t)(c >> 3) * 4 + (r >> 3) * 2 + (c & 1)) * 32 + (r & 7) * 4 + ((c & 7) >> 1)) * 8;
+  return layout == OPERAND_BLOCKED ? ((size_t)c * 16 + r) * 8 : (size_t)r * K + (size_t)c * 8;
 }
 __device__ __forceinline__ uint4 permute_chunk(const uint4 v) {
   uint4 o;
@@ -100,6 +107,40 @@ __device__ __forceinline__ uint4 permute_chunk(const uint4 v) {
   o.z = __byte_perm(v.y, v.w, 0x5410);
   o.w = __byte_perm(v.y, v.w, 0x7632);
   return o;
+}
+// one register of a permuted chunk times 2^64, or 2^60 for an odd register (exact)
+__device__ __forceinline__ uint32_t scale_pair(uint32_t a, bool odd) {
+  uint32_t f = odd ? ((127u + 60u) << 7) * 0x10001u : ((127u + 64u) << 7) * 0x10001u;
+  __nv_bfloat162 r = __hmul2(*reinterpret_cast<__nv_bfloat162*>(&a), *reinterpret_cast<__nv_bfloat162*>(&f));
+  return *reinterpret_cast<uint32_t*>(&r);
+}
+// a permuted chunk times {2^64, 2^60, 2^64, 2^60} by register (exact)
+__device__ __forceinline__ uint4 scale_chunk(const uint4 v) {
+  return make_uint4(scale_pair(v.x, false), scale_pair(v.y, true), scale_pair(v.z, false), scale_pair(v.w, true));
+}
+// sum of the 8 elements of a chunk that scale_chunk has scaled, times 2^64
+__device__ __forceinline__ float scaled_chunk_sum(const uint4 v) {
+  const float even = (__uint_as_float(v.x << 16) + __uint_as_float(v.x & 0xffff0000u)) + (__uint_as_float(v.z << 16) + __uint_as_float(v.z & 0xffff0000u));
+  const float odd = (__uint_as_float(v.y << 16) + __uint_as_float(v.y & 0xffff0000u)) + (__uint_as_float(v.w << 16) + __uint_as_float(v.w & 0xffff0000u));
+  return fmaf(16.0f, odd, even);
+}
+// what lane t of a fragment row holds of those 16 values: groups P, P + 1 with sums v0, v1 (times 2^-69); lanes 0, 1 (`outer`)
+// the first and third terms, lanes 2, 3 the second terms and zeros
+__device__ __forceinline__ uint2 sum_terms_fragment(float v0, float v1, bool outer) {
+  const uint32_t t1 = pack_bf16x2(v0, v1);
+  v0 -= bf16_lo(t1), v1 -= bf16_hi(t1);
+  const uint32_t t2 = pack_bf16x2(v0, v1);
+  v0 -= bf16_lo(t2), v1 -= bf16_hi(t2);
+  return outer ? make_uint2(t1, pack_bf16x2(v0, v1)) : make_uint2(t2, 0u);
+}
+// group gi (0..3) of the 32 bytes of one (256 features, request): the sum, already times 2^-69, in three bf16 terms
+__device__ __forceinline__ void store_sum_terms(unsigned char* dst, int gi, float v) {
+  uint16_t* d = reinterpret_cast<uint16_t*>(dst) + (gi >> 1) * 4 + (gi & 1);
+  const uint16_t t1 = f32_to_bf16(v);
+  v -= bf16_to_f32(t1);
+  const uint16_t t2 = f32_to_bf16(v);
+  v -= bf16_to_f32(t2);
+  d[0] = t1, d[2] = f32_to_bf16(v), d[8] = t2, d[10] = 0;
 }
 __device__ __forceinline__ float chunk_sum(const uint4 v) {  // v in natural order
   return ((bf16_lo(v.x) + bf16_hi(v.x)) + (bf16_lo(v.y) + bf16_hi(v.y))) +
@@ -111,6 +152,18 @@ __device__ __forceinline__ float group_sum_8lanes(float s) {
   s += __shfl_xor_sync(0xffffffffu, s, 2);
   s += __shfl_xor_sync(0xffffffffu, s, 4);
   return s;
+}
+
+// Chunk c (8 features, natural order) of request r, and the sum of 64-feature group `group`, in the given layout.
+__device__ __forceinline__ void store_operand_chunk(int layout, uint16_t* xp, int K, int r, int c, const uint4 v) {
+  const uint4 pv = permute_chunk(v);
+  *reinterpret_cast<uint4*>(xp + operand_chunk_offset(layout, K, r, c)) = layout == OPERAND_BLOCKED ? pv : scale_chunk(pv);
+}
+__device__ __forceinline__ void store_operand_sum(int layout, void* xs, int r, int group, float sum) {
+  if (layout == OPERAND_BLOCKED)
+    reinterpret_cast<float*>(xs)[(size_t)group * 16 + r] = sum;
+  else
+    store_sum_terms(reinterpret_cast<unsigned char*>(xs) + ((size_t)(group >> 2) * 16 + r) * kOperandSumBytes, group & 3, sum * kOperandSumScale);
 }
 
 // ---- warp reductions ----------------------------------------------------------------

@@ -1,5 +1,6 @@
 // Host-side launch interface of the q4decode kernels (internal to the library).
 #pragma once
+#include <cuda.h>
 #include <cuda_runtime.h>
 #include <stddef.h>
 #include <stdint.h>
@@ -18,45 +19,41 @@ void set_pdl_enabled(bool on);
 bool pdl_enabled();
 
 // ---- fragment-ordered GEMM operand ---------------------------------------------------
-// xp bf16 [16][K] (chunks of 8 permuted), xs f32 [K/64][16] (group sums); see common.cuh.
-// Three layouts of the bf16 elements exist: OPERAND_ROWS, [16][K] (the grouped projections of the MoE layers),
-// OPERAND_BLOCKED, [K/8][16][8] (the tcgen05 kernel: a K-range of all requests is one contiguous block that the
-// tensor core reads as 8-request x 16-byte core matrices), and OPERAND_SLICED, [K/ks][16][ks + 8] (the mma.sync
-// kernels of the dense projections: a slice of ks features of all requests is one contiguous block, already padded
-// like its shared-memory image).  All keep the order 0,4,1,5,2,6,3,7 inside a chunk of 8.
+// xp bf16 [16][K] (chunks of 8 permuted, scaled), xs the group sums; see common.cuh.
+// Layouts of the bf16 elements: OPERAND_ROWS, [16][K] (the grouped projections of the MoE layers), OPERAND_BLOCKED (the
+// tcgen05 kernel) and OPERAND_FRAG (the dense projections: a warp's fragments as contiguous 512-byte pieces).  All keep
+// the order 0,4,1,5,2,6,3,7 inside a chunk of 8 and take 16 K elements.
 enum GemmPrologue { PRO_PLAIN = 0, PRO_SILU_MUL = 1 };
-enum OperandLayout { OPERAND_ROWS = 0, OPERAND_BLOCKED = 1, OPERAND_SLICED = 2 };
-__host__ __device__ __forceinline__ int operand_slice_features(int K) {
-  const int quads = K >> 8;  // slices are the largest of 1024, 768, 512, 256 features that divides K
-  for (int c = 4; c > 1; --c)
-    if (quads % c == 0) return c << 8;
-  return 256;
-}
-__host__ __device__ __forceinline__ size_t operand_elements(int layout, int K) {  // elements an operand buffer needs
-  return layout == OPERAND_SLICED ? (size_t)(K / operand_slice_features(K)) * 16 * (operand_slice_features(K) + 8) : (size_t)16 * K;
-}
+enum OperandLayout { OPERAND_ROWS = 0, OPERAND_BLOCKED = 1, OPERAND_FRAG = 2 };
+__host__ __device__ __forceinline__ size_t operand_sums_bytes(int K) { return (size_t)(K / 256) * 16 * 32; }  // any layout
 
-cudaError_t launch_pack_operand(const uint16_t* x, int x_stride, int K, int n, int prologue, uint16_t* xp, float* xs,
+cudaError_t launch_pack_operand(const uint16_t* x, int x_stride, int K, int n, int prologue, uint16_t* xp, void* xs,
                                 int layout, cudaStream_t s);
 
 // ---- 4-bit skinny GEMM ------------------------------------------------------------
 // EPI_SILU_PACK: the tensor has 2*I rows (gate rows then up rows); the output is the operand of the next GEMM,
-// h = bf16(silu(bf16(gate)) * bf16(up)), written in fragment order to out_xp [16][I] and out_xs [I/64][16].
+// h = bf16(silu(bf16(gate)) * bf16(up)), written as an operand to out_xp and out_xs.
 enum GemmEpilogue { EPI_BF16 = 0, EPI_RESIDUAL = 1, EPI_F32 = 2, EPI_SILU_PACK = 3 };
 
+// Tensor maps of a dense projection (gemm_make_maps).
+struct GemmMaps {
+  CUtensorMap codes, scales, biases;
+  bool sb_tma;  // scales and biases have maps
+};
 struct GemmArgs {
   const uint32_t* qw;      // [N][K/8]
+  const GemmMaps* maps = nullptr;  // of a dense projection, or NULL: made for the call
   const uint16_t* scales;  // [N][K/64]
   const uint16_t* biases;  // [N][K/64]
   int N, K;
   const uint16_t* xp;  // fragment-ordered operand
-  const float* xs;
+  const void* xs;      // group sums (NULL: the kernel adds them up itself; not in the grouped mode)
   int n;
   int epilogue;
   void* out;
   int out_stride;
   uint16_t* out_xp;  // EPI_SILU_PACK only
-  float* out_xs;
+  void* out_xs;
   float2* argmax_partial;  // EPI_F32 only, optional: [row blocks][16] = (max, index as float bits) per request
   float* partial;          // split-K partial sums
   size_t partial_bytes;
@@ -68,7 +65,8 @@ struct GemmArgs {
   const int* expert_ids = nullptr;  // [max_slots]
   const int* n_touched = nullptr;   // number of valid slots
   int max_slots = 0;
-  size_t xp_slot_stride = 0, xs_slot_stride = 0, out_slot_stride = 0, out_xs_slot_stride = 0;  // elements
+  size_t xp_slot_stride = 0, out_slot_stride = 0;          // elements
+  size_t xs_slot_stride = 0, out_xs_slot_stride = 0;       // bytes
 };
 
 // Bytes of split-K scratch a GEMM of this shape may use (upper bound over batch sizes).
@@ -76,8 +74,10 @@ size_t gemm_partial_bytes(int N, int K, int epilogue);
 int gemm_counters_needed(int N);
 int gemm_row_blocks(int N, int K, int n, int epilogue);  // grid.x of the launch (size of argmax_partial)
 cudaError_t launch_q4_gemm(const GemmArgs& a, cudaStream_t s);
-// The operand layout launch_q4_gemm expects for this call (grouped: the mixture-of-experts mode).
-int gemm_operand_layout(bool grouped, int n);  // n: requests of the call
+// The operand layout launch_q4_gemm expects (grouped: the mixture-of-experts mode).
+int gemm_operand_layout(bool grouped);
+cudaError_t gemm_make_maps(const uint32_t* qw, const uint16_t* scales, const uint16_t* biases, long long N, int K, bool gate_up,
+                           GemmMaps* out);
 
 // tcgen05 kernel (q4_umma.cu): tiles of 128 rows, K in `parts` across CTAs, stages of 256 features.
 struct UmmaPlan {
@@ -117,7 +117,7 @@ struct AttnArgs {
   float* part_ml;   // [slots][nq][2]
   uint16_t* out;    // plain [n][nq][128], or NULL
   uint16_t* out_xp; // fragment-ordered operand [16][nq*128] of the O projection, or NULL
-  float* out_xs;    // its group sums [nq*2][16]
+  void* out_xs;     // its group sums
   int out_layout = OPERAND_ROWS;  // layout of out_xp
   int* merge_counters = nullptr;  // [16][nkv], zero between launches: the attention kernel merges the chunks itself
   // The kernel requests its first K, V tiles before it waits for the preceding kernel (cached K, V do not depend on
@@ -269,7 +269,7 @@ cudaError_t launch_embed(const uint32_t* q, const uint16_t* scales, const uint16
                          const int32_t* tokens, int n, uint16_t* x, cudaStream_t s);
 // y (plain, optional) and/or the fragment-ordered operand (yp, ys) of the next GEMM.
 cudaError_t launch_rmsnorm(const uint16_t* x, const uint16_t* w, float eps, int n, int H, uint16_t* y,
-                           uint16_t* yp, float* ys, int layout, cudaStream_t s);
+                           uint16_t* yp, void* ys, int layout, cudaStream_t s);
 cudaError_t launch_argmax(const float* logits, int n, int vocab, int32_t* next, cudaStream_t s);
 cudaError_t launch_dequant(const uint32_t* q, const uint16_t* scales, const uint16_t* biases, int N, int K,
                            float* out, cudaStream_t s);

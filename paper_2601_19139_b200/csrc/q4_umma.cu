@@ -549,8 +549,8 @@ cudaError_t launch_q4_umma(const GemmArgs& a, int sm_count, cudaStream_t s) {
   }
   const UmmaPlan t = plan_umma(a.N, a.K, a.epilogue, sm_count);
   UmmaParams p;
-  p.scales = a.scales, p.biases = a.biases, p.xb = a.xp, p.xs = a.xs, p.out = a.out;
-  p.out_xb = a.out_xp, p.out_xs = a.out_xs, p.argmax_partial = a.argmax_partial, p.status = a.status;
+  p.scales = a.scales, p.biases = a.biases, p.xb = a.xp, p.xs = static_cast<const float*>(a.xs), p.out = a.out;
+  p.out_xb = a.out_xp, p.out_xs = static_cast<float*>(a.out_xs), p.argmax_partial = a.argmax_partial, p.status = a.status;
   p.partial = a.partial, p.counters = a.counters;
   p.N = a.N, p.K = a.K, p.n = a.n, p.out_stride = a.out_stride, p.epilogue = a.epilogue;
   p.tiles = t.tiles, p.parts = t.parts, p.ns = t.ns;
