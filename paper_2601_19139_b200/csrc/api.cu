@@ -65,8 +65,8 @@ struct Workspace {
   // (normed hidden state, attention output, silu(gate)*up).
   size_t x, yp, ys, qkv, qbuf, ap, as, hp, hs, logits, next, amax, gemm_partial, gemm_partial_bytes, counters,
       part_acc, part_ml, attn_merge_counters, meta, bytes;
-  // MoE: plain normed state, routing results, touched-expert list, per-slot expert activations and outputs
-  size_t yplain, m_idx, m_wgt, m_ints, m_hp, m_hs, m_o;
+  // MoE: plain normed state, routing results, list of units, per-unit expert activations and outputs
+  size_t yplain, m_wgt, m_ints, m_units, m_hp, m_o;
   int counters_len, amax_blocks;
   // persistent whole-step kernel (dense models): plain attention output and gated MLP activations, sums of squares
   // of the residual stream, split-KV scratch, argmax partials, barrier/status words, phase table
@@ -145,17 +145,16 @@ Workspace carve(const q4d_shape& s, const MetaLayout& ml) {
   w.as = take(operand_sums_bytes((int)qdim));
   w.hp = take(B * s.mlp_inter * 2 + 256);
   w.hs = take(operand_sums_bytes(s.mlp_inter) + 256);
-  w.yplain = w.m_idx = w.m_wgt = w.m_ints = w.m_hp = w.m_hs = w.m_o = 0;
+  w.yplain = w.m_wgt = w.m_ints = w.m_units = w.m_hp = w.m_o = 0;
   if (s.n_experts) {
     const size_t E = s.n_experts;
     w.yplain = take(B * s.hidden * 2);
-    w.m_idx = take(B * s.top_k * 4);
     w.m_wgt = take(B * s.top_k * 4);
-    // flags[E], expert_ids[E], slot_of[E], counter, n_touched, touched_total, slice_counter[16], then logits[16][E]
-    w.m_ints = take((3 * E + 3 + kMaxBatch) * 4 + B * E * 4);
-    w.m_hp = take(E * B * s.expert_inter * 2);
-    w.m_hs = take(E * operand_sums_bytes(s.expert_inter));
-    w.m_o = take(E * B * s.hidden * 2);
+    w.m_ints = take((B * s.top_k + 3) * 4 + B * E * 4);  // pos[16][top_k], counter, n_units, touched_total, then logits[16][E]
+    w.m_units = take(kMaxExpertUnits * sizeof(int4));
+    const size_t U = std::min<size_t>(kMaxExpertUnits, B * s.top_k);  // units hold at least one of the B * top_k pairs
+    w.m_hp = take(U * 16 * s.expert_inter * 2);
+    w.m_o = take(U * 8 * s.hidden * 2);
   }
   w.logits = take(B * (size_t)s.vocab * 4);
   w.next = take(B * 4);
@@ -242,7 +241,7 @@ struct q4d_model {
   q4d_shape sh;
   std::vector<q4d_layer_weights> layers;
   q4d_weights w;
-  std::vector<GemmMaps> maps;  // of the dense projections: 4 per layer (qkv, o, gate/up, down), then the head
+  std::vector<GemmMaps> maps;  // of the dense projections: 4 per layer (qkv, o, gate/up, down; of all experts), then the head
   unsigned char* ws;
   Workspace lay;
   MetaLayout ml;
@@ -602,7 +601,7 @@ int step_impl(q4d_model* m, q4d_kv_pool* pool, int32_t n, const int64_t* ids, co
   float* logits = logits_dev ? logits_dev : at<float>(m, m->lay.logits);
   const size_t layer_elems = (size_t)pool->num_blocks * nkv * kBlockSize * kHeadDim;
   const int qdim = nq * kHeadDim;
-  const int dense_layout = gemm_operand_layout(false);  // of the operands of the dense projections
+  const int dense_layout = gemm_operand_layout();  // of the operands of the dense projections
 
 #define Q4D_LAUNCH(cls, expr)                                                 \
   do {                                                                        \
@@ -611,7 +610,7 @@ int step_impl(q4d_model* m, q4d_kv_pool* pool, int32_t n, const int64_t* ids, co
   } while (0)
 
   if (sh.n_experts) {  // the step's count of routed experts starts at zero
-    cudaError_t ce = cudaMemsetAsync(at<int32_t>(m, m->lay.m_ints) + 3 * sh.n_experts + 2, 0, 4, s);
+    cudaError_t ce = cudaMemsetAsync(at<int32_t>(m, m->lay.m_ints) + kMaxBatch * sh.top_k + 2, 0, 4, s);
     if (ce != cudaSuccess) return fail_cuda(ce, "routed-expert counter reset");
   }
   if (range) {
@@ -661,29 +660,24 @@ int step_impl(q4d_model* m, q4d_kv_pool* pool, int32_t n, const int64_t* ids, co
       int32_t* ints = at<int32_t>(m, m->lay.m_ints);
       MoeRouteArgs mr;
       mr.y = yplain, mr.router = lw.router, mr.H = H, mr.E = E, mr.top_k = sh.top_k, mr.norm = sh.norm_topk_prob;
-      mr.idx = at<int32_t>(m, m->lay.m_idx), mr.wgt = at<float>(m, m->lay.m_wgt);
-      mr.flags = ints, mr.expert_ids = ints + E, mr.slot_of = ints + 2 * E, mr.counter = ints + 3 * E;
-      mr.n_touched = ints + 3 * E + 1;
-      mr.touched_total = ints + 3 * E + 2;
-      mr.slice_counter = ints + 3 * E + 3;
-      mr.logits = reinterpret_cast<float*>(ints + 3 * E + 3 + kMaxBatch);
+      mr.wgt = at<float>(m, m->lay.m_wgt);
+      mr.pos = ints, mr.counter = ints + kMaxBatch * sh.top_k, mr.n_units = mr.counter + 1, mr.touched_total = mr.counter + 2;
+      mr.logits = reinterpret_cast<float*>(mr.counter + 3);
+      mr.units = at<int4>(m, m->lay.m_units);
       uint16_t* ehp = at<uint16_t>(m, m->lay.m_hp);
-      void* ehs = at<unsigned char>(m, m->lay.m_hs);
       uint16_t* eo = at<uint16_t>(m, m->lay.m_o);
-      Q4D_LAUNCH(Q4D_K_RMSNORM, launch_rmsnorm(x, lw.mlp_norm, sh.rms_eps, n, H, yplain, yp, ys, gemm_operand_layout(true), s));
+      Q4D_LAUNCH(Q4D_K_RMSNORM, launch_rmsnorm(x, lw.mlp_norm, sh.rms_eps, n, H, yplain, yp, ys, OPERAND_FRAG, s));
       Q4D_LAUNCH(Q4D_K_MOE_ROUTER, launch_moe_router(mr, n, s));
-      GemmArgs gu = gemm_args(m, lw.experts_gate_up, 2 * Ie, H, yp, ys, n, EPI_SILU_PACK, nullptr, 0, -1);
-      gu.out_xp = ehp, gu.out_xs = ehs;
-      gu.expert_ids = mr.expert_ids, gu.n_touched = mr.n_touched, gu.max_slots = E;
-      gu.out_slot_stride = (size_t)16 * Ie, gu.out_xs_slot_stride = operand_sums_bytes(Ie);
-      Q4D_LAUNCH(Q4D_K_MOE_GATE_UP, launch_q4_gemm(gu, s));
-      GemmArgs dn = gemm_args(m, lw.experts_down, H, Ie, ehp, ehs, n, EPI_BF16, eo, H, -1);
-      dn.expert_ids = mr.expert_ids, dn.n_touched = mr.n_touched, dn.max_slots = E;
-      dn.xp_slot_stride = (size_t)16 * Ie, dn.xs_slot_stride = operand_sums_bytes(Ie);
-      dn.out_slot_stride = (size_t)16 * H;
-      Q4D_LAUNCH(Q4D_K_MOE_DOWN, launch_q4_gemm(dn, s));
+      ExpertArgs ea;
+      ea.scales = lw.experts_gate_up.scales, ea.biases = lw.experts_gate_up.biases, ea.maps = &m->maps[4 * l + 2], ea.gate_up = true;
+      ea.N = 2 * Ie, ea.K = H, ea.xp = yp, ea.xs = ys, ea.out = nullptr, ea.out_xp = ehp, ea.unit_stride = 0, ea.out_unit_stride = (size_t)16 * Ie;
+      ea.units = mr.units, ea.n_units = mr.n_units, ea.status = at<unsigned int>(m, m->lay.chain_status);
+      Q4D_LAUNCH(Q4D_K_MOE_GATE_UP, launch_q4_experts(ea, s));
+      ea.scales = lw.experts_down.scales, ea.biases = lw.experts_down.biases, ea.maps = &m->maps[4 * l + 3], ea.gate_up = false;
+      ea.N = H, ea.K = Ie, ea.xp = ehp, ea.xs = nullptr, ea.out = eo, ea.out_xp = nullptr, ea.unit_stride = (size_t)16 * Ie, ea.out_unit_stride = 0;
+      Q4D_LAUNCH(Q4D_K_MOE_DOWN, launch_q4_experts(ea, s));
       MoeCombineArgs mc;
-      mc.x = x, mc.o = eo, mc.idx = mr.idx, mc.wgt = mr.wgt, mc.slot_of = mr.slot_of, mc.H = H, mc.top_k = sh.top_k;
+      mc.x = x, mc.o = eo, mc.pos = mr.pos, mc.wgt = mr.wgt, mc.H = H, mc.top_k = sh.top_k;
       Q4D_LAUNCH(Q4D_K_MOE_DOWN, launch_moe_combine(mc, n, s));
     }
   }
@@ -812,7 +806,7 @@ int prefill_rows(q4d_model* m, q4d_kv_pool* pool, const int32_t* tokens, int row
     uint16_t* yp = at<uint16_t>(m, lay.yp);
     void* ys = at<unsigned char>(m, lay.ys);
     float2* amax = at<float2>(m, lay.amax);
-    Q4D_LAUNCH(Q4D_K_RMSNORM, launch_rmsnorm(x + (size_t)(rows - 1) * H, m->w.final_norm, sh.rms_eps, 1, H, nullptr, yp, ys, gemm_operand_layout(false), s));
+    Q4D_LAUNCH(Q4D_K_RMSNORM, launch_rmsnorm(x + (size_t)(rows - 1) * H, m->w.final_norm, sh.rms_eps, 1, H, nullptr, yp, ys, gemm_operand_layout(), s));
     GemmArgs lm = gemm_args(m, m->w.lm_head, V, H, yp, ys, 1, EPI_F32, logits_dev, V, 4 * sh.n_layers);
     lm.argmax_partial = amax;
     const int lm_blocks = gemm_row_blocks(V, H, 1, EPI_F32);
@@ -891,7 +885,12 @@ int q4d_model_create(const q4d_shape* shape, const q4d_weights* weights, void* w
       GemmMaps* mp = m->maps.data() + 4 * l;
       if (e == cudaSuccess) e = gemm_make_maps(lw.wqkv.q, lw.wqkv.scales, lw.wqkv.biases, nqkv, H, false, mp);
       if (e == cudaSuccess) e = gemm_make_maps(lw.wo.q, lw.wo.scales, lw.wo.biases, H, qdim, false, mp + 1);
-      if (shape->n_experts) continue;
+      if (shape->n_experts) {
+        const int E = shape->n_experts, Ie = shape->expert_inter;
+        if (e == cudaSuccess) e = gemm_make_maps(lw.experts_gate_up.q, lw.experts_gate_up.scales, lw.experts_gate_up.biases, 2 * Ie, H, true, mp + 2, E);
+        if (e == cudaSuccess) e = gemm_make_maps(lw.experts_down.q, lw.experts_down.scales, lw.experts_down.biases, H, Ie, false, mp + 3, E);
+        continue;
+      }
       if (e == cudaSuccess) e = gemm_make_maps(lw.w_gate_up.q, lw.w_gate_up.scales, lw.w_gate_up.biases, 2 * (long long)shape->mlp_inter, H, true, mp + 2);
       if (e == cudaSuccess) e = gemm_make_maps(lw.w_down.q, lw.w_down.scales, lw.w_down.biases, H, shape->mlp_inter, false, mp + 3);
     }
@@ -920,7 +919,7 @@ int q4d_model_create(const q4d_shape* shape, const q4d_weights* weights, void* w
   if (e == cudaSuccess) e = cudaMemset(m->ws + lay.counters, 0, (size_t)lay.counters_len * 4);
   if (e == cudaSuccess) e = cudaMemset(m->ws + lay.attn_merge_counters, 0, (size_t)16 * shape->n_kv_heads * 4);
   if (e == cudaSuccess && shape->n_experts)
-    e = cudaMemset(m->ws + lay.m_ints, 0, (3 * (size_t)shape->n_experts + 3 + kMaxBatch) * 4);
+    e = cudaMemset(m->ws + lay.m_ints, 0, ((size_t)kMaxBatch * shape->top_k + 3) * 4);
   if (e == cudaSuccess && shape->n_experts) e = cudaMemset(m->ws + lay.p_counts, 0, (size_t)shape->n_experts * 4);
   if (e == cudaSuccess) e = cudaMemset(m->ws + lay.chain_status, 0, 256);
   if (e == cudaSuccess) e = cudaMallocHost(reinterpret_cast<void**>(&m->host_status), sizeof(uint32_t));
@@ -1229,7 +1228,7 @@ int q4d_moe_touched_experts(q4d_model* m, int64_t* total) {
   int32_t v = 0;
   cudaError_t e = cudaDeviceSynchronize();
   if (e == cudaSuccess)
-    e = cudaMemcpy(&v, at<int32_t>(m, m->lay.m_ints) + 3 * m->sh.n_experts + 2, 4, cudaMemcpyDeviceToHost);
+    e = cudaMemcpy(&v, at<int32_t>(m, m->lay.m_ints) + kMaxBatch * m->sh.top_k + 2, 4, cudaMemcpyDeviceToHost);
   if (e != cudaSuccess) return fail_cuda(e, "moe_touched_experts");
   *total = v;
   return Q4D_OK;
@@ -1271,7 +1270,7 @@ int q4d_q4_gemm(const q4d_qtensor* w, int32_t N, int32_t K, const uint16_t* x, i
   uint16_t* xp = reinterpret_cast<uint16_t*>(sc + kOpPackOff);
   void* xs = reinterpret_cast<void*>(sc + kOpPackOff + kOpPackXp);
   cudaStream_t st = static_cast<cudaStream_t>(stream);
-  cudaError_t e = launch_pack_operand(x, x_stride, K, n, prologue, xp, xs, gemm_operand_layout(false), st);
+  cudaError_t e = launch_pack_operand(x, x_stride, K, n, prologue, xp, xs, gemm_operand_layout(), st);
   if (e != cudaSuccess) return fail_cuda(e, "q4_gemm (operand)");
   GemmArgs a;
   a.qw = w->q, a.scales = w->scales, a.biases = w->biases, a.N = N, a.K = K, a.xp = xp, a.xs = xs, a.n = n;
@@ -1286,7 +1285,7 @@ int q4d_q4_gemm(const q4d_qtensor* w, int32_t N, int32_t K, const uint16_t* x, i
 int q4d_rmsnorm(const uint16_t* x, const uint16_t* w, float eps, int32_t n, int32_t H, uint16_t* y, void* stream) {
   if (!x || !w || !y || n < 0 || H < 64 || H % 64 || H > 16384)
     return fail(Q4D_ERR_INVALID_ARG, "rmsnorm: bad argument (H must be a multiple of 64, at most 16384)");
-  cudaError_t e = launch_rmsnorm(x, w, eps, n, H, y, nullptr, nullptr, OPERAND_ROWS, static_cast<cudaStream_t>(stream));
+  cudaError_t e = launch_rmsnorm(x, w, eps, n, H, y, nullptr, nullptr, OPERAND_FRAG, static_cast<cudaStream_t>(stream));
   return e == cudaSuccess ? Q4D_OK : fail_cuda(e, "rmsnorm");
 }
 

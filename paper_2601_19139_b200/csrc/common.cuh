@@ -82,7 +82,7 @@ __device__ __forceinline__ void ldmatrix_x4_trans(uint32_t (&r)[4], const void* 
 // Producers build both with these helpers, always with the same summation tree: ((e0+e1)+(e2+e3))+((e4+e5)+(e6+e7))
 // per chunk, then a pairwise tree over the 8 chunks of the group.
 //
-// Scaling (the mma.sync kernels, OPERAND_ROWS and OPERAND_FRAG).  Those kernels hand the packed codes to the tensor cores as they
+// Scaling (the mma.sync kernels, OPERAND_FRAG).  Those kernels hand the packed codes to the tensor cores as they
 // lie in the word: a 4-bit code in bits 0..3 of a half-word IS the bf16 subnormal q * 2^-133, and one in bits 4..7 is
 // 16 q * 2^-133 (bits 0..7 of bf16 count in steps of 2^-133: the first normal binade has the subnormals' spacing), so
 // unpacking is one AND.  The powers of two go into the activations, exactly: elements 0, 2, 4, 6 of a chunk are stored
@@ -92,13 +92,12 @@ __device__ __forceinline__ void ldmatrix_x4_trans(uint32_t (&r)[4], const void* 
 constexpr float kOperandUnscale = 590295810358705651712.0f;            // 2^69
 constexpr float kOperandSumScale = 1.0f / 590295810358705651712.0f;    // 2^-69
 constexpr int kOperandSumBytes = 32;                                    // per (256 features, request)
-// Element offset of chunk c (8 features) of request r in an operand of K features: OPERAND_ROWS is [16][K];
-// OPERAND_BLOCKED is [K/8][16][8] (all requests of a chunk side by side: the tcgen05 kernel copies a K-range as one
+// Element offset of chunk c (8 features) of request r in an operand of K features: OPERAND_BLOCKED is [K/8][16][8] (all requests of a chunk side by side: the tcgen05 kernel copies a K-range as one
 // block); OPERAND_FRAG is [K/64][2][2][32][8]: per group of 64 features and 8 requests, the two 16-byte halves that lane
 // 4 (r % 8) + (c % 8) / 2 of a warp holds as its B fragments, 512 contiguous bytes per half.
 __device__ __forceinline__ size_t operand_chunk_offset(int layout, int K, int r, int c) {
   if (layout == OPERAND_FRAG) return (((size_t)(c >> 3) * 4 + (r >> 3) * 2 + (c & 1)) * 32 + (r & 7) * 4 + ((c & 7) >> 1)) * 8;
-  return layout == OPERAND_BLOCKED ? ((size_t)c * 16 + r) * 8 : (size_t)r * K + (size_t)c * 8;
+  return ((size_t)c * 16 + r) * 8;
 }
 __device__ __forceinline__ uint4 permute_chunk(const uint4 v) {
   uint4 o;

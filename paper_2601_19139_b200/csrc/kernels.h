@@ -20,11 +20,10 @@ bool pdl_enabled();
 
 // ---- fragment-ordered GEMM operand ---------------------------------------------------
 // xp bf16 [16][K] (chunks of 8 permuted, scaled), xs the group sums; see common.cuh.
-// Layouts of the bf16 elements: OPERAND_ROWS, [16][K] (the grouped projections of the MoE layers), OPERAND_BLOCKED (the
-// tcgen05 kernel) and OPERAND_FRAG (the dense projections: a warp's fragments as contiguous 512-byte pieces).  All keep
-// the order 0,4,1,5,2,6,3,7 inside a chunk of 8 and take 16 K elements.
+// Layouts of the bf16 elements: OPERAND_BLOCKED (the tcgen05 kernel) and OPERAND_FRAG (the mma.sync kernels: a warp's
+// fragments as contiguous 512-byte pieces).  Both keep the order 0,4,1,5,2,6,3,7 inside a chunk of 8 and take 16 K elements.
 enum GemmPrologue { PRO_PLAIN = 0, PRO_SILU_MUL = 1 };
-enum OperandLayout { OPERAND_ROWS = 0, OPERAND_BLOCKED = 1, OPERAND_FRAG = 2 };
+enum OperandLayout { OPERAND_BLOCKED = 1, OPERAND_FRAG = 2 };
 __host__ __device__ __forceinline__ size_t operand_sums_bytes(int K) { return (size_t)(K / 256) * 16 * 32; }  // any layout
 
 cudaError_t launch_pack_operand(const uint16_t* x, int x_stride, int K, int n, int prologue, uint16_t* xp, void* xs,
@@ -47,7 +46,7 @@ struct GemmArgs {
   const uint16_t* biases;  // [N][K/64]
   int N, K;
   const uint16_t* xp;  // fragment-ordered operand
-  const void* xs;      // group sums (NULL: the kernel adds them up itself; not in the grouped mode)
+  const void* xs;      // group sums (NULL: the kernel adds them up itself)
   int n;
   int epilogue;
   void* out;
@@ -60,13 +59,6 @@ struct GemmArgs {
   int* counters;  // zero between launches
   int counters_len;
   unsigned int* status = nullptr;  // device word set non-zero when a bounded wait inside the kernel gives up
-  // grouped mode (MoE): one GEMM per slot of a device-side list of touched experts; the tensors hold
-  // `N` rows per expert, stacked.  NULL expert_ids = a single GEMM.
-  const int* expert_ids = nullptr;  // [max_slots]
-  const int* n_touched = nullptr;   // number of valid slots
-  int max_slots = 0;
-  size_t xp_slot_stride = 0, out_slot_stride = 0;          // elements
-  size_t xs_slot_stride = 0, out_xs_slot_stride = 0;       // bytes
 };
 
 // Bytes of split-K scratch a GEMM of this shape may use (upper bound over batch sizes).
@@ -74,10 +66,28 @@ size_t gemm_partial_bytes(int N, int K, int epilogue);
 int gemm_counters_needed(int N);
 int gemm_row_blocks(int N, int K, int n, int epilogue);  // grid.x of the launch (size of argmax_partial)
 cudaError_t launch_q4_gemm(const GemmArgs& a, cudaStream_t s);
-// The operand layout launch_q4_gemm expects (grouped: the mixture-of-experts mode).
-int gemm_operand_layout(bool grouped);
+int gemm_operand_layout();  // the operand layout launch_q4_gemm expects
 cudaError_t gemm_make_maps(const uint32_t* qw, const uint16_t* scales, const uint16_t* biases, long long N, int K, bool gate_up,
-                           GemmMaps* out);
+                           GemmMaps* out, int experts = 1);
+
+// Mixture of experts: the projection of every unit, a unit being up to 8 requests routed to one expert.
+constexpr int kMaxExpertUnits = 256 + 64;  // one partly filled unit for each of 256 experts, plus 16 x 32 pairs in eights
+struct ExpertArgs {
+  const uint16_t* scales;  // stacked tensors: N rows per expert
+  const uint16_t* biases;
+  const GemmMaps* maps;
+  bool gate_up;            // SiLU epilogue into out_xp (OPERAND_FRAG per unit), else bf16 rows out [unit][8][N]
+  int N, K;
+  const uint16_t* xp;      // gate_up: the step's operand (OPERAND_FRAG, 16 requests) with its group sums xs; else per unit
+  const void* xs;
+  uint16_t* out;
+  uint16_t* out_xp;
+  size_t unit_stride, out_unit_stride;  // elements between the units' operands
+  const int4* units;       // device list {expert, requests, request ids as bytes in two words}
+  const int* n_units;
+  unsigned int* status;
+};
+cudaError_t launch_q4_experts(const ExpertArgs& a, cudaStream_t s);
 
 // tcgen05 kernel (q4_umma.cu): tiles of 128 rows, K in `parts` across CTAs, stages of 256 features.
 struct UmmaPlan {
@@ -118,7 +128,7 @@ struct AttnArgs {
   uint16_t* out;    // plain [n][nq][128], or NULL
   uint16_t* out_xp; // fragment-ordered operand [16][nq*128] of the O projection, or NULL
   void* out_xs;     // its group sums
-  int out_layout = OPERAND_ROWS;  // layout of out_xp
+  int out_layout = OPERAND_FRAG;  // layout of out_xp
   int* merge_counters = nullptr;  // [16][nkv], zero between launches: the attention kernel merges the chunks itself
   // The kernel requests its first K, V tiles before it waits for the preceding kernel (cached K, V do not depend on
   // it).  Set when they do (the preceding kernel appends tokens this launch reads): the launch then carries no
@@ -159,23 +169,19 @@ struct MoeRouteArgs {
   const uint16_t* y;       // plain normed hidden state bf16 [n][H]
   const uint16_t* router;  // bf16 [E][H]
   int H, E, top_k, norm;
-  int32_t* idx;         // [16][top_k] selected experts, by decreasing logit
-  float* wgt;           // [16][top_k] their weights
-  int32_t* flags;       // [E], zero between launches
+  float* wgt;           // [16][top_k] weights of the selected experts, by decreasing logit
+  int32_t* pos;         // [16][top_k]: 8 x unit + place in the unit
   int32_t* counter;     // zero between launches
-  int32_t* expert_ids;  // [E] touched experts, ascending
-  int32_t* slot_of;     // [E] position of an expert in expert_ids
-  int32_t* n_touched;
+  int4* units;          // the list the expert projections walk (ExpertArgs)
+  int32_t* n_units;
   float* logits;           // [16][E] scratch
-  int32_t* slice_counter;  // [16], zero between launches
-  int32_t* touched_total = nullptr;  // optional: running sum of n_touched over the launches of a step
+  int32_t* touched_total = nullptr;  // optional: running sum of the touched experts over the launches of a step
 };
 struct MoeCombineArgs {
   uint16_t* x;        // residual stream bf16 [n][H], updated in place
-  const uint16_t* o;  // expert outputs bf16 [slot][16][H]
-  const int32_t* idx;
+  const uint16_t* o;  // expert outputs bf16 [unit][8][H]
+  const int32_t* pos;
   const float* wgt;
-  const int32_t* slot_of;
   int H, top_k;
 };
 cudaError_t launch_moe_router(const MoeRouteArgs& a, int n, cudaStream_t s);

@@ -11,7 +11,7 @@
 // per 256 features, biases against the group sums of the activations in three bf16 terms.
 //
 // Dense projections: q4_slice_kernel (K split over the warps of a CTA, operand in registers).  Mixture of experts:
-// q4_grouped_kernel (a CTA owns 128 rows of one touched expert).
+// q4_expert_kernel (the same over a list of routed experts).
 #include <stdlib.h>
 #include <string.h>
 
@@ -24,112 +24,11 @@ namespace q4d {
 
 namespace {
 
-constexpr int kThreads = 256;
-constexpr int kWarps = 8;
-constexpr int kSbBytes = 16;     // per row per stage: 4 scales + 4 biases (bf16)
 
-// Grouped projections (mixture of experts): blockIdx.y is a slot of the touched-expert list; the tensors of expert
-// expert_ids[slot] start N rows further per expert; operand and output move by their slot strides.
-struct GroupedParams {
-  const uint32_t* qw;
-  const uint16_t* scales;
-  const uint16_t* biases;
-  const uint16_t* xp;
-  const unsigned char* xs;
-  uint16_t* out;
-  uint16_t* out_xp;
-  unsigned char* out_xs;
-  int N, K, n, out_stride;
-  const int* expert_ids;
-  const int* n_touched;
-  size_t xp_slot_stride, out_slot_stride;   // elements
-  size_t xs_slot_stride, out_xs_slot_stride;  // bytes
-};
-
-// Four bf16x2 registers from one packed word: {code 0, code 4}, 16 x {code 1, code 5}, {code 2, code 6}, 16 x {code 3,
-// code 7}, each half a bf16 subnormal (or first-binade normal) counting in 2^-133.  Five logic operations for 8 codes.
-__device__ __forceinline__ void unpack_word(uint32_t w, uint32_t (&p)[4]) {
-  const uint32_t w8 = w >> 8;
-  p[0] = w & 0x000f000fu;
-  p[1] = w & 0x00f000f0u;
-  p[2] = w8 & 0x000f000fu;
-  p[3] = w8 & 0x00f000f0u;
-}
-
-// two fp32 FMAs in one instruction: c = a * b + c on both halves, each rounded like a scalar FMA
-__device__ __forceinline__ void fma_f32x2(unsigned long long& c, unsigned long long a, unsigned long long b) {
-  asm("fma.rn.f32x2 %0, %1, %2, %0;" : "+l"(c) : "l"(a), "l"(b));
-}
-__device__ __forceinline__ unsigned long long pack_f32x2(float lo, float hi) {
-  unsigned long long r;
-  asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(lo), "f"(hi));
-  return r;
-}
-__device__ __forceinline__ void unpack_f32x2(unsigned long long v, float& lo, float& hi) {
-  asm("mov.b64 {%0, %1}, %2;" : "=f"(lo), "=f"(hi) : "l"(v));
-}
-
-// acc += s * pc for the 2 x 2 block of an MMA fragment (rows g, g + 8; requests 2t, 2t + 1): s per row.
-__device__ __forceinline__ void scale_fma(float (&acc)[4], const float (&pc)[4], float s_lo, float s_hi) {
-  unsigned long long a01 = pack_f32x2(acc[0], acc[1]), a23 = pack_f32x2(acc[2], acc[3]);
-  fma_f32x2(a01, pack_f32x2(s_lo, s_lo), pack_f32x2(pc[0], pc[1]));
-  fma_f32x2(a23, pack_f32x2(s_hi, s_hi), pack_f32x2(pc[2], pc[3]));
-  unpack_f32x2(a01, acc[0], acc[1]);
-  unpack_f32x2(a23, acc[2], acc[3]);
-}
-
+// float of element i of four packed bf16
 __device__ __forceinline__ float bf16_at(const uint2& v, int i) {
   uint32_t w = (i >> 1) ? v.y : v.x;
   return (i & 1) ? bf16_hi(w) : bf16_lo(w);
-}
-
-// acc (in units of 2^-69) += a stage's 16 rows x 256 features against the staged operand.  stg: 16 rows of 128 bytes of
-// codes, 16-byte chunks XOR-swizzled with the row, then the rows' {4 scales, 4 biases}.  sB: the operand's slice, rows
-// b_stride apart; sX: its group sums; cq: the stage's place in the slice.
-template <int NT>
-__device__ __forceinline__ void multiply_stage(const unsigned char* stg, const unsigned char* sB, const unsigned char* sX,
-                                               int b_stride, int cq, int g, int t, float (&acc)[NT][4]) {
-  const unsigned char* sb = stg + 16 * 128 + g * kSbBytes;
-  const uint2 sc_lo = *reinterpret_cast<const uint2*>(sb), sc_hi = *reinterpret_cast<const uint2*>(sb + 8 * kSbBytes);
-  {
-    // lane t holds groups 2 (t & 1), 2 (t & 1) + 1; the operand has the three terms of the sums in the matching places
-    const uint32_t b_lo = *reinterpret_cast<const uint32_t*>(sb + 8 + (t & 1) * 4);
-    const uint32_t b_hi = *reinterpret_cast<const uint32_t*>(sb + 8 * kSbBytes + 8 + (t & 1) * 4);
-#pragma unroll
-    for (int nt = 0; nt < NT; ++nt) {
-      const uint2 x = *reinterpret_cast<const uint2*>(sX + (cq * 16 + nt * 8 + g) * kOperandSumBytes + t * 8);
-      mma_bf16(acc[nt], b_lo, b_hi, b_lo, b_hi, x.x, x.y);
-    }
-  }
-#pragma unroll
-  for (int gi = 0; gi < 4; ++gi) {
-    uint4 bf[NT][2];
-#pragma unroll
-    for (int nt = 0; nt < NT; ++nt) {
-      const unsigned char* bp = sB + (nt * 8 + g) * b_stride + (cq * 4 + gi) * 128 + t * 32;
-      bf[nt][0] = *reinterpret_cast<const uint4*>(bp);
-      bf[nt][1] = *reinterpret_cast<const uint4*>(bp + 16);
-    }
-    // 16-byte chunk c of row r sits at chunk c ^ (r & 7); rows g and g + 8 share the swizzle
-    const int woff = g * 128 + (((gi * 2 + (t >> 1)) ^ g) << 4) + (t & 1) * 8;
-    const uint2 wl = *reinterpret_cast<const uint2*>(stg + woff);
-    const uint2 wh = *reinterpret_cast<const uint2*>(stg + woff + 8 * 128);
-    uint32_t l0[4], l1[4], h0[4], h1[4];
-    unpack_word(wl.x, l0);
-    unpack_word(wl.y, l1);
-    unpack_word(wh.x, h0);
-    unpack_word(wh.y, h1);
-    const float s_lo = bf16_at(sc_lo, gi), s_hi = bf16_at(sc_hi, gi);
-#pragma unroll
-    for (int nt = 0; nt < NT; ++nt) {
-      float pc[4];
-      mma_bf16_first(pc, l0[0], h0[0], l0[1], h0[1], bf[nt][0].x, bf[nt][0].y);
-      mma_bf16(pc, l0[2], h0[2], l0[3], h0[3], bf[nt][0].z, bf[nt][0].w);
-      mma_bf16(pc, l1[0], h1[0], l1[1], h1[1], bf[nt][1].x, bf[nt][1].y);
-      mma_bf16(pc, l1[2], h1[2], l1[3], h1[3], bf[nt][1].z, bf[nt][1].w);
-      scale_fma(acc[nt], pc, s_lo, s_hi);
-    }
-  }
 }
 
 // MMAs the compiler may move: the multiplication below has registers to spare for overlapping its groups.
@@ -194,130 +93,6 @@ __device__ __forceinline__ void multiply_regs(const unsigned char* smem, uint32_
   }
 }
 
-// A CTA of eight warps owns 128 rows of one expert (with the SiLU epilogue 64 gate rows and the 64 matching up rows), the
-// whole of K (at most 2048) of the operand resident; a warp streams its 16 rows through a private cp.async ring.
-constexpr int kGroupedStage = 16 * (128 + kSbBytes);
-template <int NT, int STAGES, bool SILU>
-__global__ void __launch_bounds__(kThreads, 2) q4_grouped_kernel(const GroupedParams p) {
-  constexpr int NP = 8 * NT;        // padded request count
-  constexpr int kRows = kWarps * 16;
-  constexpr int kTs = NP + 1;       // row stride of the final tile (floats)
-  extern __shared__ __align__(128) unsigned char smem[];
-
-  grid_launch_dependents();
-  // the expert list is written by the preceding kernel: wait for it before anything else
-  grid_dependency_wait();
-  const int slot = blockIdx.y;
-  if (slot >= *p.n_touched) return;
-  const size_t e_row0 = (size_t)p.expert_ids[slot] * p.N;
-  const uint16_t* xp = p.xp + (size_t)slot * p.xp_slot_stride;
-  const unsigned char* xs = p.xs + (size_t)slot * p.xs_slot_stride;
-
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, g = lane >> 2, t = lane & 3;
-  const int half_n = p.N >> 1, K = p.K, nquads = K >> 8;
-  const int warp_row0 = !SILU ? blockIdx.x * kRows + warp * 16
-                              : (warp < 4 ? blockIdx.x * 64 + warp * 16 : half_n + blockIdx.x * 64 + (warp - 4) * 16);
-  const int row_limit = SILU && warp < 4 ? half_n : p.N;
-  const int b_stride = K * 2 + 16;  // bytes per request row of the staged activations
-
-  unsigned char* ring = smem + warp * (STAGES * kGroupedStage);
-  unsigned char* sB = smem + kWarps * STAGES * kGroupedStage;
-  unsigned char* sX = sB + NP * b_stride;
-
-  const unsigned char* row_src[4];
-#pragma unroll
-  for (int i = 0; i < 4; ++i)
-    row_src[i] = reinterpret_cast<const unsigned char*>(p.qw + (e_row0 + min(warp_row0 + i * 4 + (lane >> 3), row_limit - 1)) * (size_t)(K >> 3)) +
-                 (lane & 7) * 16;
-  const size_t sb_off = (e_row0 + min(warp_row0 + (lane & 15), row_limit - 1)) * (size_t)(K >> 6);
-  auto issue_stage = [&](int qd) {
-    unsigned char* stg = ring + (qd % STAGES) * kGroupedStage;
-#pragma unroll
-    for (int i = 0; i < 4; ++i) {
-      const int r = i * 4 + (lane >> 3);
-      cp_async16(stg + r * 128 + (((lane & 7) ^ (r & 7)) << 4), row_src[i] + qd * 128);
-    }
-    if (lane < 16) {
-      cp_async8(stg + 16 * 128 + lane * kSbBytes, p.scales + sb_off + qd * 4);
-      cp_async8(stg + 16 * 128 + lane * kSbBytes + 8, p.biases + sb_off + qd * 4);
-    }
-  };
-#pragma unroll
-  for (int s = 0; s < STAGES - 1; ++s) {
-    if (s < nquads) issue_stage(s);
-    cp_async_commit();
-  }
-  {  // the operand of every request and its group sums
-    const int cpr = K >> 3;  // 16-byte chunks per request row
-    for (int c = threadIdx.x; c < NP * cpr; c += kThreads) {
-      const int r = c / cpr, kc = c - r * cpr;
-      cp_async16(sB + r * b_stride + kc * 16, xp + (size_t)r * K + kc * 8);
-    }
-    for (int c = threadIdx.x; c < nquads * 16 * kOperandSumBytes / 16; c += kThreads) cp_async16(sX + c * 16, xs + c * 16);
-    cp_async_commit();
-    cp_async_wait<0>();
-  }
-  __syncthreads();
-
-  float acc[NT][4];
-#pragma unroll
-  for (int nt = 0; nt < NT; ++nt)
-#pragma unroll
-    for (int c = 0; c < 4; ++c) acc[nt][c] = 0.0f;
-  for (int qd = 0; qd < nquads; ++qd) {
-    if (qd + STAGES - 1 < nquads) issue_stage(qd + STAGES - 1);
-    cp_async_commit();
-    cp_async_wait<STAGES - 1>();
-    __syncwarp();
-    multiply_stage<NT>(ring + (qd % STAGES) * kGroupedStage, sB, sX, b_stride, qd, g, t, acc);
-    __syncwarp();
-  }
-  cp_async_wait<0>();
-  __syncthreads();  // every warp is done with its ring: the final tile may overlay them
-
-  float* sT = reinterpret_cast<float*>(smem);  // [kRows][kTs]
-#pragma unroll
-  for (int nt = 0; nt < NT; ++nt)
-#pragma unroll
-    for (int c = 0; c < 4; ++c)
-      sT[(warp * 16 + g + (c >> 1) * 8) * kTs + nt * 8 + 2 * t + (c & 1)] = acc[nt][c] * kOperandUnscale;
-  __syncthreads();
-
-  if (SILU) {
-    // h = bf16(silu(bf16(gate)) * bf16(up)) for the CTA's 64 columns, as the next GEMM's operand.
-    const int idx = threadIdx.x;
-    if (idx < 8 * NP) {
-      const int c = idx & 7, req = idx >> 3;
-      uint32_t hw[4];
-#pragma unroll
-      for (int i = 0; i < 4; ++i) {
-        float hv[2];
-#pragma unroll
-        for (int j = 0; j < 2; ++j) {
-          const int col = c * 8 + 2 * i + j;
-          const float gt = bf16_to_f32(f32_to_bf16(sT[col * kTs + req])), up = bf16_to_f32(f32_to_bf16(sT[(64 + col) * kTs + req]));
-          hv[j] = (gt / (1.0f + expf(-gt))) * up;
-        }
-        hw[i] = pack_bf16x2(hv[0], hv[1]);
-      }
-      const uint4 v = make_uint4(hw[0], hw[1], hw[2], hw[3]);
-      const float gsum = group_sum_8lanes(chunk_sum(v));
-      const int col0 = blockIdx.x * 64 + c * 8;
-      if (col0 < half_n && req < p.n) {
-        store_operand_chunk(OPERAND_ROWS, p.out_xp + (size_t)slot * p.out_slot_stride, half_n, req, col0 >> 3, v);
-        if (c == 0) store_operand_sum(OPERAND_ROWS, p.out_xs + (size_t)slot * p.out_xs_slot_stride, req, col0 >> 6, gsum);
-      }
-    }
-    return;
-  }
-  uint16_t* out = p.out + (size_t)slot * p.out_slot_stride;
-  for (int idx = threadIdx.x; idx < kRows * NP; idx += kThreads) {
-    const int req = idx / kRows, lrow = idx - req * kRows;
-    const int row = blockIdx.x * kRows + lrow;
-    if (row < p.N && req < p.n) out[(size_t)req * p.out_stride + row] = f32_to_bf16(sT[lrow * kTs + req]);
-  }
-}
-
 // ---- dense projections -------------------------------------------------------------------------------------------
 // One CTA per SM owns a contiguous range of 16-row tiles (and, for K > 4096, one part of K).  K is split over the WARPS:
 // warp (kslice, row group) owns 256 or 512 input features and keeps the operand of those features in registers, as the B
@@ -368,10 +143,10 @@ __device__ __forceinline__ bool elect_one() {
 __device__ __forceinline__ void mbar_expect_tx_addr(uint32_t bar, uint32_t bytes) {
   asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(bar), "r"(bytes) : "memory");
 }
-// the box at (x, row y) of both planes of the map (this GPU's memory only, no multicast)
-__device__ __forceinline__ void tma_3d(uint32_t dst, const CUtensorMap* map, int x, int y, uint32_t bar) {
+// the box at (x, row y, plane z) of the map (this GPU's memory only, no multicast)
+__device__ __forceinline__ void tma_3d(uint32_t dst, const CUtensorMap* map, int x, int y, int z, uint32_t bar) {
   asm volatile("cp.async.bulk.tensor.3d.shared::cluster.global.tile.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3, %4}], [%5];" ::"r"(dst),
-               "l"(reinterpret_cast<uint64_t>(map)), "r"(x), "r"(y), "r"(0), "r"(bar)
+               "l"(reinterpret_cast<uint64_t>(map)), "r"(x), "r"(y), "r"(z), "r"(bar)
                : "memory");
 }
 // Waits for the phase of the given parity of the barrier at a shared address; gives up (false) after about two seconds.
@@ -392,6 +167,25 @@ __device__ __forceinline__ uint32_t transpose_8x8(uint32_t v) {  // of b16: lane
   uint32_t r;
   asm volatile("movmatrix.sync.aligned.m8n8.trans.b16 %0, %1;" : "=r"(r) : "r"(v));
   return r;
+}
+
+// h = bf16(silu(bf16(gate)) * bf16(up)) of 8 features (rows g are gate rows, rows g + 8 the matching up rows) x 8 requests, as
+// chunk `tile` of an OPERAND_FRAG of K features; lane (g, t) writes a part of request 8 nt + g (if `valid`).
+__device__ __forceinline__ void silu_epilogue(const float (&v)[4], uint16_t* out_xp, int K, int tile, int g, int t, bool valid, int nt = 0) {
+  float h[2];
+#pragma unroll
+  for (int j = 0; j < 2; ++j) {
+    const float gt = bf16_to_f32(f32_to_bf16(v[j])), up = bf16_to_f32(f32_to_bf16(v[2 + j]));
+    h[j] = (gt / (1.0f + expf(-gt))) * up;
+  }
+  const uint32_t f = transpose_8x8(pack_bf16x2(h[0], h[1]));
+  // the operand pairs features (j, j + 4) in word order 0: (0, 4), 1: (1, 5), 2: (2, 6), 3: (3, 7): lanes t < 2 take
+  // (2t, 2t + 4), lanes t + 2 take (2t + 1, 2t + 5); odd words are stored times 2^60
+  const uint32_t other = __shfl_xor_sync(0xffffffffu, t < 2 ? f >> 16 : f & 0xffffu, 2);
+  const uint32_t pair = t < 2 ? (f & 0xffffu) | (other << 16) : other | (f & 0xffff0000u);
+  const int word = t < 2 ? 2 * t : 2 * t - 3;
+  if (valid)
+    *reinterpret_cast<uint32_t*>(out_xp + operand_chunk_offset(OPERAND_FRAG, K, nt * 8 + g, tile) + word * 2) = scale_pair(pair, word & 1);
 }
 
 // Epilogue of 16 rows x 8 requests (nt: which 8) from an accumulator fragment (lane holds rows g, g + 8 and requests 2t,
@@ -415,21 +209,7 @@ __device__ __forceinline__ void slice_epilogue(const SliceParams& p, float (&v)[
   }
   const int req = nt * 8 + g;  // after the transposition: request g, rows (or features) 2t, 2t + 1
   if (p.epilogue == EPI_SILU_PACK) {
-    // rows g are gate rows, rows g + 8 the matching up rows: h = bf16(silu(bf16(gate)) * bf16(up)) is lane-local
-    float h[2];
-#pragma unroll
-    for (int j = 0; j < 2; ++j) {
-      const float gt = bf16_to_f32(f32_to_bf16(v[j])), up = bf16_to_f32(f32_to_bf16(v[2 + j]));
-      h[j] = (gt / (1.0f + expf(-gt))) * up;
-    }
-    const uint32_t f = transpose_8x8(pack_bf16x2(h[0], h[1]));
-    // the operand pairs features (j, j + 4) in word order 0: (0, 4), 1: (1, 5), 2: (2, 6), 3: (3, 7): lanes t < 2 take
-    // (2t, 2t + 4), lanes t + 2 take (2t + 1, 2t + 5); odd words are stored times 2^60
-    const uint32_t other = __shfl_xor_sync(0xffffffffu, t < 2 ? f >> 16 : f & 0xffffu, 2);
-    const uint32_t pair = t < 2 ? (f & 0xffffu) | (other << 16) : other | (f & 0xffff0000u);
-    const int word = t < 2 ? 2 * t : 2 * t - 3;
-    if (req < p.n && tile * 8 < (p.N >> 1))
-      *reinterpret_cast<uint32_t*>(p.out_xp + operand_chunk_offset(OPERAND_FRAG, p.N >> 1, req, tile) + word * 2) = scale_pair(pair, word & 1);
+    silu_epilogue(v, p.out_xp, p.N >> 1, tile, g, t, req < p.n && tile * 8 < (p.N >> 1), nt);
     return;
   }
 #pragma unroll
@@ -496,12 +276,12 @@ __global__ void __launch_bounds__(32 * slice_max_warps(NT), 1) q4_slice_kernel(c
     if (elect_one()) {
       const uint32_t bar = bar_a + slot * 8, dst = ring_a + slot * kSliceCodes;
       mbar_expect_tx_addr(bar, (both ? 4096 : 2048) + (SB_TMA ? kSliceSb : 0));
-      tma_3d(dst, &maps.codes, j * (SUB * 128), y0, bar);
-      if (both) tma_3d(dst + 2048, &maps.codes, j * 256 + 128, y0, bar);
+      tma_3d(dst, &maps.codes, j * (SUB * 128), y0, 0, bar);
+      if (both) tma_3d(dst + 2048, &maps.codes, j * 256 + 128, y0, 0, bar);
       if (SB_TMA) {
         const uint32_t sb = sb_a + slot * kSliceSb;
-        tma_3d(sb, &maps.scales, gx, y0, bar);
-        tma_3d(sb + 256, &maps.biases, gx, y0, bar);
+        tma_3d(sb, &maps.scales, gx, y0, 0, bar);
+        tma_3d(sb + 256, &maps.biases, gx, y0, 0, bar);
       }
     }
     if (!SB_TMA && lane < 16) {
@@ -726,7 +506,7 @@ SlicePlan plan_slices(int N, int K, int n, int epilogue, int sm_count) {
   const int warps = t.kw * t.rg, rounds = (per_cta + t.rg - 1) / t.rg;
   const size_t fixed = 1024 + (size_t)warps * kSliceSlots * (slice_slot_codes(t.nt) + kSliceSb);
   const size_t per_round = 2 * (size_t)warps * t.nt * 512;  // two buffers
-  const int most = (int)((223 * 1024 - fixed) / per_round);  // rounds whose partial tiles fit
+  const int most = (int)((220 * 1024 - fixed) / per_round);  // rounds whose partial tiles fit
   const int batches = (rounds + most - 1) / most;
   t.batch = (rounds + batches - 1) / batches;
   t.smem = fixed + t.batch * per_round;
@@ -734,11 +514,221 @@ SlicePlan plan_slices(int N, int K, int n, int epilogue, int sm_count) {
   return t;
 }
 
-template <int NT, int STAGES>
-size_t grouped_smem(int K) {
-  const size_t work = (size_t)kWarps * STAGES * kGroupedStage + (size_t)(8 * NT) * (K * 2 + 16) + operand_sums_bytes(K);
-  const size_t tile = (size_t)kWarps * 16 * (8 * NT + 1) * sizeof(float);
-  return work > tile ? work : tile;
+// ---- mixture-of-experts projections --------------------------------------------------------------------------------
+// The same multiplication over a list of units, a unit being up to eight requests that were routed to one expert: with
+// sixteen requests and 128 experts an expert serves one or two of them, so eight columns are enough where the earlier
+// kernel multiplied all sixteen requests with every touched expert.  The row tiles of all units form one list, cut into
+// equal contiguous ranges, one per CTA; a warp exchanges its operand fragments when its range enters the next unit (the
+// weight ring runs on across the border).  Gate/up reads the fragments of a unit's requests from the step's operand;
+// its output is the unit's own operand for the down projection.  Measured (30B-A3B shape, 16 requests, between events):
+// gate/up 62 -> 39 us, down with the combination 2 x 22.7 -> 2 x 18.2 us.
+struct ExpertParams {
+  const uint16_t* scales;
+  const uint16_t* biases;
+  const uint16_t* xp;        // OPERAND_FRAG: of the step (gate/up), or one per unit, unit_stride elements apart (down)
+  const unsigned char* xs;   // group sums of the step's operand (gate/up)
+  uint16_t* out;             // down: bf16 [unit][8][N]
+  uint16_t* out_xp;          // gate/up: OPERAND_FRAG per unit
+  unsigned int* status;
+  const int4* units;         // {expert, requests, request ids as bytes (two words)}
+  const int* n_units;
+  size_t unit_stride, out_unit_stride;  // elements
+  int N, K, tiles;           // rows and row tiles of an expert
+  int kw, rg, batch;
+};
+
+template <bool GATE_UP, bool SB_TMA>
+__global__ void __launch_bounds__(32 * slice_max_warps(1), 1) q4_expert_kernel(const ExpertParams p, const __grid_constant__ GemmMaps maps) {
+  constexpr int kCodes = 16 * 128;
+  extern __shared__ unsigned char smem_raw[];
+  __shared__ __align__(8) uint64_t s_bar[slice_max_warps(1)][kSliceSlots];
+  __shared__ __align__(8) uint64_t s_full[2], s_free[2];
+  __shared__ int4 s_units[kMaxExpertUnits];
+
+  const int warp = __shfl_sync(0xffffffffu, threadIdx.x >> 5, 0), lane = threadIdx.x & 31, g = lane >> 2, t = lane & 3;
+  const int warps = blockDim.x >> 5, rg = p.rg;
+  const int j = warp / rg, rgi = warp - j * rg;  // 256-feature slice, row group
+  const int half_n = p.N >> 1, kg = p.K >> 6;
+
+  unsigned char* smem = reinterpret_cast<unsigned char*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~(uintptr_t)1023);
+  unsigned char* ring = smem + warp * (kSliceSlots * kCodes);
+  unsigned char* ring_sb = smem + warps * (kSliceSlots * kCodes) + warp * (kSliceSlots * kSliceSb);
+  float4* sP = reinterpret_cast<float4*>(smem + warps * (kSliceSlots * (kCodes + kSliceSb)));
+  if (lane == 0) {
+#pragma unroll
+    for (int i = 0; i < kSliceSlots; ++i) um_mbar_init(&s_bar[warp][i], 1);
+    if (warp == 0) {
+#pragma unroll
+      for (int i = 0; i < 2; ++i) um_mbar_init(&s_full[i], warps), um_mbar_init(&s_free[i], warps);
+    }
+    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+  }
+  __syncthreads();
+  // The list of units is the router's.  Gate/up follows the router and waits for it; only then does it let the down
+  // projection start, which may therefore read the list at once and fetch its first weights under gate/up's tail.
+  if (GATE_UP) {
+    grid_dependency_wait();
+    grid_launch_dependents();
+  } else {
+    grid_launch_dependents();
+  }
+  const int n_units = min(__ldcg(p.n_units), kMaxExpertUnits);
+  for (int i = threadIdx.x; i < n_units; i += blockDim.x) s_units[i] = __ldcg(p.units + i);
+  __syncthreads();
+  const int total = n_units * p.tiles;
+  const int t0 = (int)((long long)blockIdx.x * total / gridDim.x), Tc = (int)((long long)(blockIdx.x + 1) * total / gridDim.x) - t0;
+  const int my_n = rgi < Tc ? (Tc - rgi + rg - 1) / rg : 0;
+
+  const uint32_t ring_a = smem_u32(ring), sb_a = smem_u32(ring_sb), bar_a = smem_u32(&s_bar[warp][0]);
+  const int gx = (j * 4) & ~7, sb_half = SB_TMA ? (j & 1) * 8 : 0;
+  auto issue = [&](int gt, int slot) {  // tile gt of the list
+    const int unit = gt / p.tiles, tile = gt - unit * p.tiles;
+    const int e = __shfl_sync(0xffffffffu, s_units[unit].x, 0);
+    const int y = GATE_UP ? tile * 8 : e * p.N + tile * 16, z = GATE_UP ? 2 * e : 0;
+    if (elect_one()) {
+      const uint32_t bar = bar_a + slot * 8;
+      mbar_expect_tx_addr(bar, kCodes + (SB_TMA ? kSliceSb : 0));
+      tma_3d(ring_a + slot * kCodes, &maps.codes, j * 128, y, z, bar);
+      if (SB_TMA) {
+        tma_3d(sb_a + slot * kSliceSb, &maps.scales, gx, y, z, bar);
+        tma_3d(sb_a + slot * kSliceSb + 256, &maps.biases, gx, y, z, bar);
+      }
+    }
+    if (!SB_TMA && lane < 16) {
+      const int r = GATE_UP ? (lane < 8 ? tile * 8 + lane : half_n + tile * 8 + lane - 8) : tile * 16 + lane;
+      const size_t off = ((size_t)e * p.N + r) * kg + j * 4;
+      unsigned char* dst = ring_sb + slot * kSliceSb + lane * 16;
+      cp_async8(dst, p.scales + off);
+      cp_async8(dst + 256, p.biases + off);
+    }
+  };
+#pragma unroll
+  for (int i = 0; i < kSliceSlots; ++i) {
+    if (i < my_n) issue(t0 + i * rg + rgi, i);
+    if (!SB_TMA) cp_async_commit();
+  }
+  if (!GATE_UP) grid_dependency_wait();
+
+  uint4 bf[4][1][2];
+  uint2 x[1];
+  auto load_operand = [&](int unit) {
+    const int4 u = s_units[unit];
+    int r = g;
+    const uint16_t* base = p.xp;
+    if (GATE_UP) r = ((g < 4 ? u.z : u.w) >> ((g & 3) * 8)) & 15;
+    else base += (size_t)unit * p.unit_stride;
+    const uint4* src = reinterpret_cast<const uint4*>(base) + (size_t)j * 16 * 32 + (r >> 3) * 64 + (r & 7) * 4 + t;
+#pragma unroll
+    for (int gi = 0; gi < 4; ++gi)
+#pragma unroll
+      for (int h = 0; h < 2; ++h) bf[gi][0][h] = __ldcg(src + (gi * 4 + h) * 32);
+    if (GATE_UP) {
+      x[0] = __ldcg(reinterpret_cast<const uint2*>(p.xs + ((size_t)j * 16 + r) * kOperandSumBytes + t * 8));
+    } else {
+      float v[4];
+#pragma unroll
+      for (int gi = 0; gi < 4; ++gi) {
+        float s = scaled_chunk_sum(bf[gi][0][0]) + scaled_chunk_sum(bf[gi][0][1]);
+        s += __shfl_xor_sync(0xffffffffu, s, 1);
+        s += __shfl_xor_sync(0xffffffffu, s, 2);
+        v[gi] = s * kOperandSumScale * 0x1p-64f;
+      }
+      x[0] = sum_terms_fragment((t & 1) ? v[2] : v[0], (t & 1) ? v[3] : v[1], t < 2);
+    }
+  };
+
+  bool ok = true;
+  auto wait = [&](uint32_t bar, uint32_t parity) {
+    if (!mbar_wait_addr(bar, parity)) {
+      ok = false;  // a copy or a warp that never came: report, results are void
+      if (p.status) atomicExch(p.status, 3u);
+    }
+  };
+  const uint32_t full_a = smem_u32(&s_full[0]), free_a = smem_u32(&s_free[0]);
+  const int buf_f4 = p.batch * rg * p.kw * 32;  // float4 of a buffer
+
+  auto finish_batch = [&](int b) {
+    const int first = b * p.batch * rg, tiles = min(p.batch * rg, Tc - first), buf = b & 1;
+    wait(full_a + buf * 8, (uint32_t)((b >> 1) & 1));
+    __syncwarp();
+    for (int tl = (warp - first % warps + warps) % warps; tl < tiles; tl += warps) {
+      const int gt = t0 + first + tl, unit = gt / p.tiles, tile = gt - unit * p.tiles;
+      const int count = s_units[unit].y;
+      float v[4] = {0.0f, 0.0f, 0.0f, 0.0f};
+      const float4* src = sP + buf * buf_f4 + tl * (p.kw * 32) + lane;
+#pragma unroll 8
+      for (int k = 0; k < p.kw; ++k) {
+        const float4 a = src[k * 32];
+        v[0] += a.x, v[1] += a.y, v[2] += a.z, v[3] += a.w;
+      }
+#pragma unroll
+      for (int c = 0; c < 4; ++c) v[c] *= kOperandUnscale;
+      if (GATE_UP) {
+        silu_epilogue(v, p.out_xp + (size_t)unit * p.out_unit_stride, half_n, tile, g, t, g < count);
+      } else {
+#pragma unroll
+        for (int half = 0; half < 2; ++half) {
+          const uint32_t y = transpose_8x8(pack_bf16x2(v[2 * half], v[2 * half + 1]));
+          if (g < count)
+            *reinterpret_cast<uint32_t*>(p.out + ((size_t)unit * 8 + g) * p.N + tile * 16 + half * 8 + 2 * t) = y;
+        }
+      }
+    }
+    __syncwarp();
+    if (lane == 0) um_mbar_arrive(&s_free[buf]);
+  };
+
+  int it = 0, slot = 0, gt = t0 + rgi, unit = -1, unit_end = 0;
+  uint32_t phase = 0;
+  const uint32_t codes0 = (uint32_t)(ring - smem) + g * 128 + (((t >> 1) ^ g) << 4) + (t & 1) * 8;
+  const uint32_t sc0 = (uint32_t)(ring_sb - smem) + g * 16 + sb_half, bi0 = sc0 + 256 + (t & 1) * 4;
+  const int part_step = rg * p.kw * 32;
+  const int batches = (Tc + p.batch * rg - 1) / (p.batch * rg);
+  for (int b = 0; b < batches; ++b) {
+    const int buf = b & 1;
+    if (b >= 2) wait(free_a + buf * 8, (uint32_t)(((b >> 1) - 1) & 1));
+    float4* dst = sP + buf * buf_f4 + (rgi * p.kw + j) * 32 + lane;
+    const int it_end = min(my_n, (b + 1) * p.batch);
+    for (; it < it_end; ++it, dst += part_step, gt += rg) {
+      if (gt >= unit_end) {
+        unit = gt / p.tiles, unit_end = (unit + 1) * p.tiles;
+        load_operand(unit);
+      }
+      if (!SB_TMA) cp_async_wait<kSliceSlots - 1>();
+      wait(bar_a + slot * 8, phase);
+      __syncwarp();
+      float acc[1][4] = {{0.0f, 0.0f, 0.0f, 0.0f}};
+      const unsigned char* sc = smem + sc0 + slot * kSliceSb;
+      multiply_regs<1>(smem, codes0 + slot * kCodes, bi0 + slot * kSliceSb, *reinterpret_cast<const uint2*>(sc),
+                       *reinterpret_cast<const uint2*>(sc + 128), bf, x, acc);
+      dst[0] = make_float4(acc[0][0], acc[0][1], acc[0][2], acc[0][3]);
+      __syncwarp();
+      if (ok && it + kSliceSlots < my_n) issue(gt + kSliceSlots * rg, slot);  // refill the slot just multiplied
+      if (!SB_TMA) cp_async_commit();
+      if (++slot == kSliceSlots) slot = 0, phase ^= 1u;
+    }
+    __syncwarp();
+    if (lane == 0) um_mbar_arrive(&s_full[buf]);
+    if (b > 0) finish_batch(b - 1);
+  }
+  if (batches > 0) finish_batch(batches - 1);
+  if (!SB_TMA) cp_async_wait<0>();
+}
+
+struct ExpertPlan {
+  int tiles, kw, rg, batch;
+  size_t smem;
+};
+ExpertPlan plan_experts(int N, int K) {
+  ExpertPlan t;
+  t.tiles = N / 16;
+  t.kw = K / 256;
+  t.rg = slice_max_warps(1) / t.kw;
+  const int warps = t.kw * t.rg;
+  const size_t fixed = 1024 + (size_t)warps * kSliceSlots * (slice_slot_codes(1) + kSliceSb), per_round = 2 * (size_t)warps * 512;
+  t.batch = 4;  // tiles of a row group between two meetings
+  t.smem = fixed + t.batch * per_round;
+  return t;
 }
 
 int g_sm_count = 0;
@@ -805,9 +795,8 @@ int gemm_row_blocks(int N, int K, int n, int epilogue) {
   return t.ctas * t.parts * t.kw * t.rg;  // one argmax partial per warp of the grid
 }
 
-int gemm_operand_layout(bool grouped) {
+int gemm_operand_layout() {
   (void)sm_count_or_default();
-  if (grouped) return OPERAND_ROWS;
   return g_legacy ? OPERAND_FRAG : OPERAND_BLOCKED;
 }
 
@@ -819,12 +808,12 @@ cudaError_t gemm_init() {
   e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
   if (e != cudaSuccess) return e;
   // 227 KB is the per-CTA limit for static + dynamic shared memory; leave room for the static part.
-  const int big = 224 * 1024;
+  const int big = 220 * 1024;
   auto big_smem = [&](auto kernel) {
     if (e == cudaSuccess) e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, big);
   };
-  big_smem(q4_grouped_kernel<1, 4, true>), big_smem(q4_grouped_kernel<1, 4, false>);
-  big_smem(q4_grouped_kernel<2, 3, true>), big_smem(q4_grouped_kernel<2, 3, false>);
+  big_smem(q4_expert_kernel<true, true>), big_smem(q4_expert_kernel<true, false>);
+  big_smem(q4_expert_kernel<false, true>), big_smem(q4_expert_kernel<false, false>);
   big_smem(q4_slice_kernel<1, true>), big_smem(q4_slice_kernel<2, true>);
   big_smem(q4_slice_kernel<1, false>), big_smem(q4_slice_kernel<2, false>);
   if (e != cudaSuccess) return e;
@@ -835,18 +824,19 @@ cudaError_t gemm_init() {
 
 // The packed codes as bytes [N][K / 2], boxes of 16 rows x 128 bytes (256 codes) with the 128-byte swizzle; scales and biases
 // as [N][K / 64], boxes of 16 rows x 8 groups (only where a row is a multiple of 16 bytes: K a multiple of 512).  For a
-// gate/up tensor the two halves of the rows are two planes, and a box is 8 rows of both.
+// gate/up tensor the two halves of the rows are two planes, and a box is 8 rows of both; stacked experts continue the
+// planes (gate/up) or the rows.
 cudaError_t gemm_make_maps(const uint32_t* qw, const uint16_t* scales, const uint16_t* biases, long long N, int K, bool gate_up,
-                           GemmMaps* out) {
+                           GemmMaps* out, int experts) {
   EncodeTiledFn encode = nullptr;
   const cudaError_t e = encode_tiled_fn(&encode);
   if (e != cudaSuccess) return e;
   auto make = [&](CUtensorMap* m, CUtensorMapDataType type, const void* base, int row_elems, int elem_bytes, unsigned box_x,
                   CUtensorMapSwizzle swizzle) {
-    const long long planes = gate_up ? 2 : 1, rows = N / planes;
+    const long long planes = gate_up ? 2 * experts : 1, rows = gate_up ? N / 2 : N * experts;
     const cuuint64_t dims[3] = {(cuuint64_t)row_elems, (cuuint64_t)rows, (cuuint64_t)planes};
     const cuuint64_t strides[2] = {(cuuint64_t)row_elems * elem_bytes, (cuuint64_t)row_elems * elem_bytes * rows};
-    const cuuint32_t box[3] = {box_x, (cuuint32_t)(16 / planes), (cuuint32_t)planes}, elem[3] = {1u, 1u, 1u};
+    const cuuint32_t box[3] = {box_x, gate_up ? 8u : 16u, gate_up ? 2u : 1u}, elem[3] = {1u, 1u, 1u};
     return encode(m, type, 3, const_cast<void*>(base), dims, strides, box, elem, CU_TENSOR_MAP_INTERLEAVE_NONE, swizzle,
                   CU_TENSOR_MAP_L2_PROMOTION_NONE, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
   };
@@ -866,52 +856,47 @@ cudaError_t launch_q4_gemm(const GemmArgs& a, cudaStream_t s) {
   }
   if (a.n <= 0) return cudaSuccess;
   if (a.N <= 0 || a.K <= 0 || (a.K % 256) || a.n > kMaxBatch) return cudaErrorInvalidValue;
-  const bool grouped = a.expert_ids != nullptr;
-  if (a.epilogue == EPI_SILU_PACK && ((a.N % 16) || !a.out_xp || (grouped && !a.out_xs))) return cudaErrorInvalidValue;
-  if (grouped && (a.K > 2048 || !a.n_touched || a.max_slots < 1)) return cudaErrorInvalidValue;
-  if (!grouped && use_umma(a.N, a.K, a.epilogue)) return launch_q4_umma(a, g_sm_count, s);
-  if (!grouped) {
-    const SlicePlan t = plan_slices(a.N, a.K, a.n, a.epilogue, g_sm_count);
-    SliceParams p;
-    p.scales = a.scales, p.biases = a.biases, p.xp = a.xp, p.xs = static_cast<const unsigned char*>(a.xs), p.out = a.out;
-    p.out_xp = a.out_xp, p.argmax_partial = a.argmax_partial, p.status = a.status;
-    p.N = a.N, p.K = a.K, p.n = a.n, p.out_stride = a.out_stride, p.epilogue = a.epilogue;
-    p.T = t.T, p.kw = t.kw, p.rg = t.rg, p.batch = t.batch;
-    p.partial = a.partial, p.counters = a.counters;
-    if (t.parts > 1 && (!a.partial || !a.counters || t.partial_bytes > a.partial_bytes || t.T > a.counters_len))
-      return cudaErrorInvalidValue;
-    const int elem = a.epilogue == EPI_F32 ? 4 : 2;
-    p.vec_ok = a.out && (reinterpret_cast<uintptr_t>(a.out) % 16 == 0) && ((size_t)a.out_stride * elem % 16 == 0);
-    GemmMaps made;
-    const GemmMaps* maps = a.maps;
-    if (!maps) {
-      const cudaError_t e = gemm_make_maps(a.qw, a.scales, a.biases, a.N, a.K, a.epilogue == EPI_SILU_PACK, &made);
-      if (e != cudaSuccess) return e;
-      maps = &made;
-    }
-    const dim3 grid(t.ctas, t.parts), block(32 * t.kw * t.rg);
-    auto go = [&](auto kernel) { return launch_kernel(kernel, grid, block, t.smem, s, p, *maps); };
-    if (t.nt == 2) return maps->sb_tma ? go(q4_slice_kernel<2, true>) : go(q4_slice_kernel<2, false>);
-    return maps->sb_tma ? go(q4_slice_kernel<1, true>) : go(q4_slice_kernel<1, false>);
+  if (a.epilogue == EPI_SILU_PACK && ((a.N % 16) || !a.out_xp)) return cudaErrorInvalidValue;
+  if (use_umma(a.N, a.K, a.epilogue)) return launch_q4_umma(a, g_sm_count, s);
+  const SlicePlan t = plan_slices(a.N, a.K, a.n, a.epilogue, g_sm_count);
+  SliceParams p;
+  p.scales = a.scales, p.biases = a.biases, p.xp = a.xp, p.xs = static_cast<const unsigned char*>(a.xs), p.out = a.out;
+  p.out_xp = a.out_xp, p.argmax_partial = a.argmax_partial, p.status = a.status;
+  p.N = a.N, p.K = a.K, p.n = a.n, p.out_stride = a.out_stride, p.epilogue = a.epilogue;
+  p.T = t.T, p.kw = t.kw, p.rg = t.rg, p.batch = t.batch;
+  p.partial = a.partial, p.counters = a.counters;
+  if (t.parts > 1 && (!a.partial || !a.counters || t.partial_bytes > a.partial_bytes || t.T > a.counters_len))
+    return cudaErrorInvalidValue;
+  const int elem = a.epilogue == EPI_F32 ? 4 : 2;
+  p.vec_ok = a.out && (reinterpret_cast<uintptr_t>(a.out) % 16 == 0) && ((size_t)a.out_stride * elem % 16 == 0);
+  GemmMaps made;
+  const GemmMaps* maps = a.maps;
+  if (!maps) {
+    const cudaError_t e = gemm_make_maps(a.qw, a.scales, a.biases, a.N, a.K, a.epilogue == EPI_SILU_PACK, &made);
+    if (e != cudaSuccess) return e;
+    maps = &made;
   }
-  if (a.epilogue != EPI_SILU_PACK && a.epilogue != EPI_BF16) return cudaErrorInvalidValue;
-  const bool silu = a.epilogue == EPI_SILU_PACK;
-  GroupedParams p;
-  p.qw = a.qw, p.scales = a.scales, p.biases = a.biases, p.xp = a.xp, p.xs = static_cast<const unsigned char*>(a.xs);
-  p.out = static_cast<uint16_t*>(a.out), p.out_xp = a.out_xp, p.out_xs = static_cast<unsigned char*>(a.out_xs);
-  p.N = a.N, p.K = a.K, p.n = a.n, p.out_stride = a.out_stride, p.expert_ids = a.expert_ids, p.n_touched = a.n_touched;
-  p.xp_slot_stride = a.xp_slot_stride, p.xs_slot_stride = a.xs_slot_stride;
-  p.out_slot_stride = a.out_slot_stride, p.out_xs_slot_stride = a.out_xs_slot_stride;
-  const int per_cta = silu ? 64 : 128, rows = silu ? a.N / 2 : a.N;
-  const dim3 grid((rows + per_cta - 1) / per_cta, a.max_slots), block(kThreads);
-  if (a.n <= 8) {
-    const size_t smem = grouped_smem<1, 4>(a.K);
-    return silu ? launch_kernel(q4_grouped_kernel<1, 4, true>, grid, block, smem, s, p)
-                : launch_kernel(q4_grouped_kernel<1, 4, false>, grid, block, smem, s, p);
+  const dim3 grid(t.ctas, t.parts), block(32 * t.kw * t.rg);
+  auto go = [&](auto kernel) { return launch_kernel(kernel, grid, block, t.smem, s, p, *maps); };
+  if (t.nt == 2) return maps->sb_tma ? go(q4_slice_kernel<2, true>) : go(q4_slice_kernel<2, false>);
+  return maps->sb_tma ? go(q4_slice_kernel<1, true>) : go(q4_slice_kernel<1, false>);
+}
+
+cudaError_t launch_q4_experts(const ExpertArgs& a, cudaStream_t s) {
+  if (g_sm_count == 0) {
+    cudaError_t e = gemm_init();
+    if (e != cudaSuccess) return e;
   }
-  const size_t smem = grouped_smem<2, 3>(a.K);
-  return silu ? launch_kernel(q4_grouped_kernel<2, 3, true>, grid, block, smem, s, p)
-              : launch_kernel(q4_grouped_kernel<2, 3, false>, grid, block, smem, s, p);
+  if (a.N % 16 || a.K % 256 || a.K / 256 > slice_max_warps(1) || !a.maps || !a.units || !a.n_units) return cudaErrorInvalidValue;
+  const ExpertPlan t = plan_experts(a.N, a.K);
+  ExpertParams p;
+  p.scales = a.scales, p.biases = a.biases, p.xp = a.xp, p.xs = static_cast<const unsigned char*>(a.xs), p.out = a.out, p.out_xp = a.out_xp;
+  p.status = a.status, p.units = a.units, p.n_units = a.n_units, p.unit_stride = a.unit_stride, p.out_unit_stride = a.out_unit_stride;
+  p.N = a.N, p.K = a.K, p.tiles = t.tiles, p.kw = t.kw, p.rg = t.rg, p.batch = t.batch;
+  const dim3 grid(g_sm_count), block(32 * t.kw * t.rg);
+  auto go = [&](auto kernel) { return launch_kernel(kernel, grid, block, t.smem, s, p, *a.maps); };
+  if (a.gate_up) return a.maps->sb_tma ? go(q4_expert_kernel<true, true>) : go(q4_expert_kernel<true, false>);
+  return a.maps->sb_tma ? go(q4_expert_kernel<false, true>) : go(q4_expert_kernel<false, false>);
 }
 
 cudaError_t launch_argmax_finish(const float2* partial, int row_blocks, int n, int32_t* next, cudaStream_t s) {
