@@ -75,7 +75,7 @@ struct Workspace {
   // prompt processing: up to p_rows tokens at once.  p_u holds qkv, q and the attention output while a layer's first
   // half runs and the MLP activations in its second half; p_op, p_inv the operand of the coming projection.  MoE: the
   // (token, expert) pairs sorted by expert (their operand, then their outputs, in p_pairs).
-  size_t p_x, p_u, p_q, p_attn, p_op, p_inv, p_y, p_idx, p_wgt, p_pos, p_counts, p_cursor, p_units, p_pairs, p_pairs_inv, p_eh, p_eop,
+  size_t p_sums, p_x, p_u, p_q, p_attn, p_op, p_inv, p_y, p_idx, p_wgt, p_pos, p_counts, p_cursor, p_units, p_pairs, p_pairs_inv, p_eh, p_eop,
       p_eop_inv;
   int p_rows;
 };
@@ -205,6 +205,7 @@ Workspace carve(const q4d_shape& s, const MetaLayout& ml) {
     const size_t R = (size_t)std::min(kPrefillChunk, (s.max_positions + 15) / 16 * 16), H = s.hidden;
     w.p_rows = (int)R;
     w.p_x = take(R * H * 2);
+    w.p_sums = take(kPrefillSumsBytes);
     const size_t first_half = align_up(R * nqkv * 2) + 2 * align_up(R * qdim * 2);
     w.p_u = take(std::max(first_half, s.n_experts ? (size_t)0 : R * s.mlp_inter * 2));
     w.p_q = w.p_u + align_up(R * nqkv * 2), w.p_attn = w.p_q + align_up(R * qdim * 2);
@@ -474,6 +475,74 @@ int read_back_status(q4d_model* m, cudaStream_t s) {
   return Q4D_OK;
 }
 
+// One launch of class `cls` in a function that has m, s and returns an error code.
+#define Q4D_LAUNCH(cls, expr)                                                 \
+  do {                                                                        \
+    cudaError_t le = timed(m, cls, s, [&]() -> cudaError_t { return expr; }); \
+    if (le != cudaSuccess) return fail_cuda(le, #cls);                        \
+  } while (0)
+
+// What follows the attention in a layer, for n rows of the residual stream x (rows H apart): O projection of the operand
+// the attention left, norm, MLP or experts.
+int layer_tail(q4d_model* m, int l, int n, uint16_t* x, cudaStream_t s) {
+  const q4d_shape& sh = m->sh;
+  const q4d_layer_weights& lw = m->layers[l];
+  const int H = sh.hidden, I = sh.mlp_inter, qdim = sh.n_q_heads * kHeadDim, dense_layout = gemm_operand_layout();
+  uint16_t *yp = at<uint16_t>(m, m->lay.yp), *ap = at<uint16_t>(m, m->lay.ap), *hp = at<uint16_t>(m, m->lay.hp);
+  void *ys = at<unsigned char>(m, m->lay.ys), *as = at<unsigned char>(m, m->lay.as), *hs = at<unsigned char>(m, m->lay.hs);
+  Q4D_LAUNCH(Q4D_K_GEMM_O, launch_q4_gemm(gemm_args(m, lw.wo, H, qdim, ap, as, n, EPI_RESIDUAL, x, H, 4 * l + 1), s));
+  if (sh.n_experts == 0) {
+    Q4D_LAUNCH(Q4D_K_RMSNORM, launch_rmsnorm(x, lw.mlp_norm, sh.rms_eps, n, H, nullptr, yp, ys, dense_layout, s));
+    GemmArgs gu = gemm_args(m, lw.w_gate_up, 2 * I, H, yp, ys, n, EPI_SILU_PACK, nullptr, 0, 4 * l + 2);
+    gu.out_xp = hp, gu.out_xs = hs;
+    Q4D_LAUNCH(Q4D_K_GEMM_GATE_UP, launch_q4_gemm(gu, s));
+    Q4D_LAUNCH(Q4D_K_GEMM_DOWN, launch_q4_gemm(gemm_args(m, lw.w_down, H, I, hp, dense_layout == OPERAND_BLOCKED ? hs : nullptr, n, EPI_RESIDUAL, x, H, 4 * l + 3), s));
+  } else {
+    const int E = sh.n_experts, Ie = sh.expert_inter;
+    uint16_t* yplain = at<uint16_t>(m, m->lay.yplain);
+    int32_t* ints = at<int32_t>(m, m->lay.m_ints);
+    MoeRouteArgs mr;
+    mr.y = yplain, mr.router = lw.router, mr.H = H, mr.E = E, mr.top_k = sh.top_k, mr.norm = sh.norm_topk_prob;
+    mr.wgt = at<float>(m, m->lay.m_wgt);
+    mr.pos = ints, mr.counter = ints + kMaxBatch * sh.top_k, mr.n_units = mr.counter + 1, mr.touched_total = mr.counter + 2;
+    mr.logits = reinterpret_cast<float*>(mr.counter + 3);
+    mr.units = at<int4>(m, m->lay.m_units);
+    uint16_t* ehp = at<uint16_t>(m, m->lay.m_hp);
+    uint16_t* eo = at<uint16_t>(m, m->lay.m_o);
+    Q4D_LAUNCH(Q4D_K_RMSNORM, launch_rmsnorm(x, lw.mlp_norm, sh.rms_eps, n, H, yplain, yp, ys, OPERAND_FRAG, s));
+    Q4D_LAUNCH(Q4D_K_MOE_ROUTER, launch_moe_router(mr, n, s));
+    ExpertArgs ea;
+    ea.scales = lw.experts_gate_up.scales, ea.biases = lw.experts_gate_up.biases, ea.maps = &m->maps[4 * l + 2], ea.gate_up = true;
+    ea.N = 2 * Ie, ea.K = H, ea.xp = yp, ea.xs = ys, ea.out = nullptr, ea.out_xp = ehp, ea.unit_stride = 0, ea.out_unit_stride = (size_t)16 * Ie;
+    ea.units = mr.units, ea.n_units = mr.n_units, ea.status = at<unsigned int>(m, m->lay.chain_status);
+    Q4D_LAUNCH(Q4D_K_MOE_GATE_UP, launch_q4_experts(ea, s));
+    ea.scales = lw.experts_down.scales, ea.biases = lw.experts_down.biases, ea.maps = &m->maps[4 * l + 3], ea.gate_up = false;
+    ea.N = H, ea.K = Ie, ea.xp = ehp, ea.xs = nullptr, ea.out = eo, ea.out_xp = nullptr, ea.unit_stride = (size_t)16 * Ie, ea.out_unit_stride = 0;
+    Q4D_LAUNCH(Q4D_K_MOE_DOWN, launch_q4_experts(ea, s));
+    MoeCombineArgs mc;
+    mc.x = x, mc.o = eo, mc.pos = mr.pos, mc.wgt = mr.wgt, mc.H = H, mc.top_k = sh.top_k;
+    Q4D_LAUNCH(Q4D_K_MOE_DOWN, launch_moe_combine(mc, n, s));
+  }
+  return Q4D_OK;
+}
+
+// Final norm, head and argmax of n rows.
+int head_launches(q4d_model* m, int n, const uint16_t* x, float* logits, int32_t* next_dev, cudaStream_t s) {
+  const q4d_shape& sh = m->sh;
+  const int H = sh.hidden, V = sh.vocab;
+  uint16_t* yp = at<uint16_t>(m, m->lay.yp);
+  void* ys = at<unsigned char>(m, m->lay.ys);
+  float2* amax = at<float2>(m, m->lay.amax);
+  Q4D_LAUNCH(Q4D_K_RMSNORM, launch_rmsnorm(x, m->w.final_norm, sh.rms_eps, n, H, nullptr, yp, ys, gemm_operand_layout(), s));
+  GemmArgs lm = gemm_args(m, m->w.lm_head, V, H, yp, ys, n, EPI_F32, logits, V, 4 * sh.n_layers);
+  lm.argmax_partial = amax;
+  const int lm_blocks = gemm_row_blocks(V, H, n, EPI_F32);
+  if (lm_blocks > m->lay.amax_blocks) return fail(Q4D_ERR_WORKSPACE_TOO_SMALL, "argmax scratch too small");
+  Q4D_LAUNCH(Q4D_K_LM_HEAD, launch_q4_gemm(lm, s));
+  Q4D_LAUNCH(Q4D_K_ARGMAX, launch_argmax_finish(amax, lm_blocks, n, next_dev, s));
+  return Q4D_OK;
+}
+
 // The launch sequence of a step.  A whole step embeds the tokens, runs every layer and the head, and advances the
 // requests.  The parity export runs only layers [layer_begin, layer_end) from a given hidden state (x_in) and
 // returns the hidden state (x_out) without advancing anything.
@@ -586,7 +655,7 @@ int step_impl(q4d_model* m, q4d_kv_pool* pool, int32_t n, const int64_t* ids, co
   }
 
   // ---- the launch sequence ----
-  const int H = sh.hidden, nq = sh.n_q_heads, nkv = sh.n_kv_heads, I = sh.mlp_inter, V = sh.vocab;
+  const int H = sh.hidden, nq = sh.n_q_heads, nkv = sh.n_kv_heads, V = sh.vocab;
   const int nqkv = (nq + 2 * nkv) * kHeadDim;
   uint16_t* x = at<uint16_t>(m, m->lay.x);
   uint16_t* yp = at<uint16_t>(m, m->lay.yp);
@@ -600,14 +669,8 @@ int step_impl(q4d_model* m, q4d_kv_pool* pool, int32_t n, const int64_t* ids, co
   float2* amax = at<float2>(m, m->lay.amax);
   float* logits = logits_dev ? logits_dev : at<float>(m, m->lay.logits);
   const size_t layer_elems = (size_t)pool->num_blocks * nkv * kBlockSize * kHeadDim;
-  const int qdim = nq * kHeadDim;
   const int dense_layout = gemm_operand_layout();  // of the operands of the dense projections
 
-#define Q4D_LAUNCH(cls, expr)                                                 \
-  do {                                                                        \
-    cudaError_t le = timed(m, cls, s, [&]() -> cudaError_t { return expr; }); \
-    if (le != cudaSuccess) return fail_cuda(le, #cls);                        \
-  } while (0)
 
   if (sh.n_experts) {  // the step's count of routed experts starts at zero
     cudaError_t ce = cudaMemsetAsync(at<int32_t>(m, m->lay.m_ints) + kMaxBatch * sh.top_k + 2, 0, 4, s);
@@ -647,53 +710,18 @@ int step_impl(q4d_model* m, q4d_kv_pool* pool, int32_t n, const int64_t* ids, co
       aa.qkv = nullptr, aa.after_predecessor = true;
     }
     Q4D_LAUNCH(Q4D_K_ATTENTION, launch_paged_attention(aa, s));
-    Q4D_LAUNCH(Q4D_K_GEMM_O, launch_q4_gemm(gemm_args(m, lw.wo, H, qdim, ap, as, n, EPI_RESIDUAL, x, H, 4 * l + 1), s));
-    if (sh.n_experts == 0) {
-      Q4D_LAUNCH(Q4D_K_RMSNORM, launch_rmsnorm(x, lw.mlp_norm, sh.rms_eps, n, H, nullptr, yp, ys, dense_layout, s));
-      GemmArgs gu = gemm_args(m, lw.w_gate_up, 2 * I, H, yp, ys, n, EPI_SILU_PACK, nullptr, 0, 4 * l + 2);
-      gu.out_xp = hp, gu.out_xs = hs;
-      Q4D_LAUNCH(Q4D_K_GEMM_GATE_UP, launch_q4_gemm(gu, s));
-      Q4D_LAUNCH(Q4D_K_GEMM_DOWN, launch_q4_gemm(gemm_args(m, lw.w_down, H, I, hp, dense_layout == OPERAND_BLOCKED ? hs : nullptr, n, EPI_RESIDUAL, x, H, 4 * l + 3), s));
-    } else {
-      const int E = sh.n_experts, Ie = sh.expert_inter;
-      uint16_t* yplain = at<uint16_t>(m, m->lay.yplain);
-      int32_t* ints = at<int32_t>(m, m->lay.m_ints);
-      MoeRouteArgs mr;
-      mr.y = yplain, mr.router = lw.router, mr.H = H, mr.E = E, mr.top_k = sh.top_k, mr.norm = sh.norm_topk_prob;
-      mr.wgt = at<float>(m, m->lay.m_wgt);
-      mr.pos = ints, mr.counter = ints + kMaxBatch * sh.top_k, mr.n_units = mr.counter + 1, mr.touched_total = mr.counter + 2;
-      mr.logits = reinterpret_cast<float*>(mr.counter + 3);
-      mr.units = at<int4>(m, m->lay.m_units);
-      uint16_t* ehp = at<uint16_t>(m, m->lay.m_hp);
-      uint16_t* eo = at<uint16_t>(m, m->lay.m_o);
-      Q4D_LAUNCH(Q4D_K_RMSNORM, launch_rmsnorm(x, lw.mlp_norm, sh.rms_eps, n, H, yplain, yp, ys, OPERAND_FRAG, s));
-      Q4D_LAUNCH(Q4D_K_MOE_ROUTER, launch_moe_router(mr, n, s));
-      ExpertArgs ea;
-      ea.scales = lw.experts_gate_up.scales, ea.biases = lw.experts_gate_up.biases, ea.maps = &m->maps[4 * l + 2], ea.gate_up = true;
-      ea.N = 2 * Ie, ea.K = H, ea.xp = yp, ea.xs = ys, ea.out = nullptr, ea.out_xp = ehp, ea.unit_stride = 0, ea.out_unit_stride = (size_t)16 * Ie;
-      ea.units = mr.units, ea.n_units = mr.n_units, ea.status = at<unsigned int>(m, m->lay.chain_status);
-      Q4D_LAUNCH(Q4D_K_MOE_GATE_UP, launch_q4_experts(ea, s));
-      ea.scales = lw.experts_down.scales, ea.biases = lw.experts_down.biases, ea.maps = &m->maps[4 * l + 3], ea.gate_up = false;
-      ea.N = H, ea.K = Ie, ea.xp = ehp, ea.xs = nullptr, ea.out = eo, ea.out_xp = nullptr, ea.unit_stride = (size_t)16 * Ie, ea.out_unit_stride = 0;
-      Q4D_LAUNCH(Q4D_K_MOE_DOWN, launch_q4_experts(ea, s));
-      MoeCombineArgs mc;
-      mc.x = x, mc.o = eo, mc.pos = mr.pos, mc.wgt = mr.wgt, mc.H = H, mc.top_k = sh.top_k;
-      Q4D_LAUNCH(Q4D_K_MOE_DOWN, launch_moe_combine(mc, n, s));
-    }
+    const int rc = layer_tail(m, l, n, x, s);
+    if (rc != Q4D_OK) return rc;
   }
   if (range) {
     cudaError_t ce = cudaMemcpyAsync(range->x_out, x, (size_t)n * H * 2, cudaMemcpyDeviceToDevice, s);
     return ce == cudaSuccess ? Q4D_OK : fail_cuda(ce, "hidden state copy");
   }
   if (pf && !pf->want_head) return Q4D_OK;  // an inner chunk of a prompt: its K, V are in the pool, nothing else is needed
-  Q4D_LAUNCH(Q4D_K_RMSNORM, launch_rmsnorm(x, m->w.final_norm, sh.rms_eps, n, H, nullptr, yp, ys, dense_layout, s));
-  GemmArgs lm = gemm_args(m, m->w.lm_head, V, H, yp, ys, n, EPI_F32, logits, V, 4 * sh.n_layers);
-  lm.argmax_partial = amax;
-  const int lm_blocks = gemm_row_blocks(V, H, n, EPI_F32);
-  if (lm_blocks > m->lay.amax_blocks) return fail(Q4D_ERR_WORKSPACE_TOO_SMALL, "decode_step: argmax scratch too small");
-  Q4D_LAUNCH(Q4D_K_LM_HEAD, launch_q4_gemm(lm, s));
-  Q4D_LAUNCH(Q4D_K_ARGMAX, launch_argmax_finish(amax, lm_blocks, n, next_dev, s));
-#undef Q4D_LAUNCH
+  {
+    const int rc = head_launches(m, n, x, logits, next_dev, s);
+    if (rc != Q4D_OK) return rc;
+  }
   {
     const int rc = read_back_status(m, s);
     if (rc != Q4D_OK) return rc;
@@ -729,10 +757,23 @@ int prefill_rows(q4d_model* m, q4d_kv_pool* pool, const int32_t* tokens, int row
   const size_t meta_bytes = (size_t)(ml.max_blocks_cap + rows) * 4;
   unsigned char* dmeta = m->ws + lay.meta + ml.off_prompt;
   cudaError_t e = cudaMemcpyAsync(dmeta, h_bt, meta_bytes, cudaMemcpyHostToDevice, s);
+  // the last layer's attention of the last token is a decode step's: one request of start + rows - 1 cached tokens
+  unsigned char* dstep = m->ws + lay.meta;
+  AttnPlan plan = {0, 0, 0};
+  size_t last_bytes = 0;
+  if (head) {
+    unsigned char* st = m->staging[slot];
+    int32_t* h_lens = reinterpret_cast<int32_t*>(st + ml.off_lens);
+    h_lens[0] = start + rows - 1;
+    plan = plan_attention(h_lens, 1, sh.n_kv_heads, 0, attention_wave_ctas(sh.n_q_heads, sh.n_kv_heads), reinterpret_cast<int4*>(st + ml.off_work),
+                          reinterpret_cast<int32_t*>(st + ml.off_slot_base), reinterpret_cast<int32_t*>(st + ml.off_nchunks), ml.max_work);
+    last_bytes = ml.off_work + (size_t)plan.n_work * sizeof(int4);
+    if (e == cudaSuccess) e = cudaMemcpyAsync(dstep, st, last_bytes, cudaMemcpyHostToDevice, s);
+  }
   if (e != cudaSuccess) return fail_cuda(e, "metadata copy");
   cudaEventRecord(m->staging_done[slot], s);
   m->staging_used[slot] = true;
-  m->last_h2d = (int64_t)meta_bytes, m->last_d2h = 0;
+  m->last_h2d = (int64_t)(meta_bytes + last_bytes), m->last_d2h = 0;
   const int32_t* d_bt = reinterpret_cast<const int32_t*>(dmeta);
   const int32_t* d_tokens = d_bt + ml.max_blocks_cap;
 
@@ -750,12 +791,30 @@ int prefill_rows(q4d_model* m, q4d_kv_pool* pool, const int32_t* tokens, int row
     a.status = at<unsigned int>(m, lay.chain_status);
     return a;
   };
-
-#define Q4D_LAUNCH(cls, expr)                                                 \
-  do {                                                                        \
-    cudaError_t le = timed(m, cls, s, [&]() -> cudaError_t { return expr; }); \
-    if (le != cudaSuccess) return fail_cuda(le, #cls);                        \
-  } while (0)
+  // A projection that leaves many SMs without a tile is cut into parts of K whose fp32 sums the next kernel adds up.
+  float* sums = at<float>(m, lay.p_sums);
+  auto parts_of = [&](int N, int K) -> int {
+    const int parts = prefill_tiling(N, K, rows).parts;
+    return (size_t)parts * rows * N * sizeof(float) <= kPrefillSumsBytes ? parts : 1;
+  };
+  auto pack = [&](uint16_t* in, int stride, const uint16_t* norm, int n_rows, int K, uint16_t* y, uint16_t* operand, float* scale) {
+    PrefillPackArgs a;
+    a.x = in, a.x_stride = stride, a.norm_w = norm, a.eps = sh.rms_eps, a.rows = n_rows, a.K = K, a.y = y, a.operand = operand, a.inv_scale = scale;
+    return a;
+  };
+  int x_parts = 1;  // parts of the projection whose result the residual stream has yet to take (in sums), or 1
+  auto pack_x = [&](const uint16_t* norm, uint16_t* y) {
+    PrefillPackArgs a = pack(x, H, norm, rows, H, y, op, inv);
+    if (x_parts > 1) a.sums = sums, a.parts = x_parts;
+    x_parts = 1;
+    return a;
+  };
+  auto residual_gemm = [&](const q4d_qtensor& t, int K) {
+    PrefillGemmArgs a = gemm(t, H, K, op, lay.p_rows, inv, rows, EPI_RESIDUAL, x, H);
+    x_parts = parts_of(H, K);
+    if (x_parts > 1) a.sums = sums;
+    return a;
+  };
 
   Q4D_LAUNCH(Q4D_K_EMBED, launch_embed(m->w.embed.q, m->w.embed.scales, m->w.embed.biases, V, H, d_tokens, rows, x, s));
   for (int l = 0; l < sh.n_layers; ++l) {
@@ -764,18 +823,39 @@ int prefill_rows(q4d_model* m, q4d_kv_pool* pool, const int32_t* tokens, int row
     pa.qkv = qkv, pa.q = at<uint16_t>(m, lay.p_q), pa.q_norm = sh.qk_norm ? lw.q_norm : nullptr, pa.k_norm = sh.qk_norm ? lw.k_norm : nullptr;
     pa.eps = sh.rms_eps, pa.rope = m->w.rope_cos_sin, pa.rows = rows, pa.start = start, pa.nq = nq, pa.nkv = nkv, pa.block_table = d_bt;
     pa.kpool = pool->mem + (size_t)(2 * l) * layer_elems, pa.vpool = pa.kpool + layer_elems, pa.out = attn;
-    Q4D_LAUNCH(Q4D_K_RMSNORM, launch_prefill_pack(x, H, lw.attn_norm, sh.rms_eps, rows, H, nullptr, op, inv, s));
-    Q4D_LAUNCH(Q4D_K_GEMM_QKV, launch_prefill_gemm(gemm(lw.wqkv, nqkv, H, op, lay.p_rows, inv, rows, EPI_BF16, qkv, nqkv), s));
+    Q4D_LAUNCH(Q4D_K_RMSNORM, launch_prefill_pack(pack_x(lw.attn_norm, nullptr), s));
+    PrefillGemmArgs gq = gemm(lw.wqkv, nqkv, H, op, lay.p_rows, inv, rows, EPI_BF16, qkv, nqkv);
+    pa.parts = parts_of(nqkv, H), pa.sums = gq.sums = pa.parts > 1 ? sums : nullptr;
+    Q4D_LAUNCH(Q4D_K_GEMM_QKV, launch_prefill_gemm(gq, s));
     Q4D_LAUNCH(Q4D_K_ROPE_APPEND, launch_prefill_rope_append(pa, s));
-    if (l == sh.n_layers - 1 && !head) break;  // nothing reads the hidden state after the last layer's K, V
+    if (l == sh.n_layers - 1) {
+      // Beyond the last layer's K, V only the last token's hidden state is read (and nothing at all between the passes of
+      // a long prompt): the rest of the layer is that of a decode step of one request.
+      if (!head) break;
+      AttnArgs aa;
+      aa.q = pa.q + (size_t)(rows - 1) * qdim, aa.kpool = pa.kpool, aa.vpool = pa.vpool, aa.block_tables = d_bt;
+      aa.lens = reinterpret_cast<const int32_t*>(dstep + ml.off_lens), aa.work = reinterpret_cast<const int4*>(dstep + ml.off_work);
+      aa.slot_base = reinterpret_cast<const int32_t*>(dstep + ml.off_slot_base), aa.nchunks = reinterpret_cast<const int32_t*>(dstep + ml.off_nchunks);
+      aa.n_work = plan.n_work, aa.n = 1, aa.nq = nq, aa.nkv = nkv, aa.max_blocks = ml.max_blocks_cap;
+      aa.part_acc = at<float>(m, lay.part_acc), aa.part_ml = at<float>(m, lay.part_ml);
+      aa.out = nullptr, aa.out_xp = at<uint16_t>(m, lay.ap), aa.out_xs = at<unsigned char>(m, lay.as), aa.out_layout = gemm_operand_layout();
+      aa.merge_counters = at<int>(m, lay.attn_merge_counters), aa.after_predecessor = true;
+      Q4D_LAUNCH(Q4D_K_ATTENTION, launch_paged_attention(aa, s));
+      const int rc = layer_tail(m, l, 1, x + (size_t)(rows - 1) * H, s);
+      if (rc != Q4D_OK) return rc;
+      break;
+    }
     Q4D_LAUNCH(Q4D_K_ATTENTION, launch_prefill_attention(pa, s));
-    Q4D_LAUNCH(Q4D_K_ATTN_MERGE, launch_prefill_pack(attn, qdim, nullptr, 0.0f, rows, qdim, nullptr, op, inv, s));
-    Q4D_LAUNCH(Q4D_K_GEMM_O, launch_prefill_gemm(gemm(lw.wo, H, qdim, op, lay.p_rows, inv, rows, EPI_RESIDUAL, x, H), s));
+    Q4D_LAUNCH(Q4D_K_ATTN_MERGE, launch_prefill_pack(pack(attn, qdim, nullptr, rows, qdim, nullptr, op, inv), s));
+    Q4D_LAUNCH(Q4D_K_GEMM_O, launch_prefill_gemm(residual_gemm(lw.wo, qdim), s));
     if (sh.n_experts == 0) {
-      Q4D_LAUNCH(Q4D_K_RMSNORM, launch_prefill_pack(x, H, lw.mlp_norm, sh.rms_eps, rows, H, nullptr, op, inv, s));
-      Q4D_LAUNCH(Q4D_K_GEMM_GATE_UP, launch_prefill_gemm(gemm(lw.w_gate_up, 2 * I, H, op, lay.p_rows, inv, rows, EPI_SILU_PACK, h, I), s));
-      Q4D_LAUNCH(Q4D_K_GEMM_DOWN, launch_prefill_pack(h, I, nullptr, 0.0f, rows, I, nullptr, op, inv, s));
-      Q4D_LAUNCH(Q4D_K_GEMM_DOWN, launch_prefill_gemm(gemm(lw.w_down, H, I, op, lay.p_rows, inv, rows, EPI_RESIDUAL, x, H), s));
+      Q4D_LAUNCH(Q4D_K_RMSNORM, launch_prefill_pack(pack_x(lw.mlp_norm, nullptr), s));
+      PrefillGemmArgs gu = gemm(lw.w_gate_up, 2 * I, H, op, lay.p_rows, inv, rows, EPI_SILU_PACK, h, I);
+      PrefillPackArgs ph = pack(h, I, nullptr, rows, I, nullptr, op, inv);
+      ph.parts = parts_of(2 * I, H), ph.silu = ph.parts > 1, ph.sums = gu.sums = ph.silu ? sums : nullptr;
+      Q4D_LAUNCH(Q4D_K_GEMM_GATE_UP, launch_prefill_gemm(gu, s));
+      Q4D_LAUNCH(Q4D_K_GEMM_DOWN, launch_prefill_pack(ph, s));
+      Q4D_LAUNCH(Q4D_K_GEMM_DOWN, launch_prefill_gemm(residual_gemm(lw.w_down, I), s));
     } else {
       const int E = sh.n_experts, Ie = sh.expert_inter, pairs = rows * sh.top_k, cap = lay.p_rows * sh.top_k + 256;
       PrefillMoeArgs mo;
@@ -789,32 +869,23 @@ int prefill_rows(q4d_model* m, q4d_kv_pool* pool, const int32_t* tokens, int row
       mo.o = mo.sorted, mo.x = x;
       uint16_t *eh = at<uint16_t>(m, lay.p_eh), *eop = at<uint16_t>(m, lay.p_eop);
       float* eop_inv = at<float>(m, lay.p_eop_inv);
-      Q4D_LAUNCH(Q4D_K_RMSNORM, launch_prefill_pack(x, H, lw.mlp_norm, sh.rms_eps, rows, H, at<uint16_t>(m, lay.p_y), op, inv, s));
+      Q4D_LAUNCH(Q4D_K_RMSNORM, launch_prefill_pack(pack_x(lw.mlp_norm, at<uint16_t>(m, lay.p_y)), s));
       Q4D_LAUNCH(Q4D_K_MOE_ROUTER, launch_prefill_route(mo, s));
       m->launches += 2;
       PrefillGemmArgs gu = gemm(lw.experts_gate_up, 2 * Ie, H, mo.sorted, cap, mo.sorted_inv_scale, pairs, EPI_SILU_PACK, eh, Ie);
-      gu.units = mo.units, gu.n_units = mo.n_units, gu.unit_rows = mo.unit_rows;
+      gu.units = mo.units, gu.n_units = mo.n_units, gu.unit_rows = mo.unit_rows, gu.experts = E;
       Q4D_LAUNCH(Q4D_K_MOE_GATE_UP, launch_prefill_gemm(gu, s));
-      Q4D_LAUNCH(Q4D_K_MOE_DOWN, launch_prefill_pack(eh, Ie, nullptr, 0.0f, pairs, Ie, nullptr, eop, eop_inv, s));
+      Q4D_LAUNCH(Q4D_K_MOE_DOWN, launch_prefill_pack(pack(eh, Ie, nullptr, pairs, Ie, nullptr, eop, eop_inv), s));
       PrefillGemmArgs dn = gemm(lw.experts_down, H, Ie, eop, cap, eop_inv, pairs, EPI_BF16, mo.sorted, H);
-      dn.units = mo.units, dn.n_units = mo.n_units, dn.unit_rows = mo.unit_rows;
+      dn.units = mo.units, dn.n_units = mo.n_units, dn.unit_rows = mo.unit_rows, dn.experts = E;
       Q4D_LAUNCH(Q4D_K_MOE_DOWN, launch_prefill_gemm(dn, s));
       Q4D_LAUNCH(Q4D_K_MOE_DOWN, launch_prefill_combine(mo, s));
     }
   }
   if (head) {
-    uint16_t* yp = at<uint16_t>(m, lay.yp);
-    void* ys = at<unsigned char>(m, lay.ys);
-    float2* amax = at<float2>(m, lay.amax);
-    Q4D_LAUNCH(Q4D_K_RMSNORM, launch_rmsnorm(x + (size_t)(rows - 1) * H, m->w.final_norm, sh.rms_eps, 1, H, nullptr, yp, ys, gemm_operand_layout(), s));
-    GemmArgs lm = gemm_args(m, m->w.lm_head, V, H, yp, ys, 1, EPI_F32, logits_dev, V, 4 * sh.n_layers);
-    lm.argmax_partial = amax;
-    const int lm_blocks = gemm_row_blocks(V, H, 1, EPI_F32);
-    if (lm_blocks > lay.amax_blocks) return fail(Q4D_ERR_WORKSPACE_TOO_SMALL, "prefill: argmax scratch too small");
-    Q4D_LAUNCH(Q4D_K_LM_HEAD, launch_q4_gemm(lm, s));
-    Q4D_LAUNCH(Q4D_K_ARGMAX, launch_argmax_finish(amax, lm_blocks, 1, next_dev, s));
+    const int rc = head_launches(m, 1, x + (size_t)(rows - 1) * H, logits_dev, next_dev, s);
+    if (rc != Q4D_OK) return rc;
   }
-#undef Q4D_LAUNCH
   return read_back_status(m, s);
 }
 

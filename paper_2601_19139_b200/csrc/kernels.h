@@ -194,9 +194,23 @@ cudaError_t launch_moe_combine(const MoeCombineArgs& a, int n, cudaStream_t s);
 constexpr int kPrefillChunk = 2048;      // tokens per pass over the weights
 constexpr int kPrefillMaxWidth = 32768;  // widest operand row
 __host__ __device__ __forceinline__ int prefill_operand_stride(int K) { return K + 64 * ((K + 1023) / 1024); }
-// rows of bf16 x (optionally RMS-normalised with w first, the normalised row also written to y) -> operand
-cudaError_t launch_prefill_pack(const uint16_t* x, int x_stride, const uint16_t* norm_w, float eps, int rows, int K,
-                                uint16_t* y, uint16_t* operand, float* inv_scale, cudaStream_t s);
+// rows of bf16 x (optionally RMS-normalised with norm_w first, the normalised row also written to y) -> operand
+struct PrefillPackArgs {
+  uint16_t* x;
+  int x_stride;
+  const uint16_t* norm_w;
+  float eps;
+  int rows, K;
+  uint16_t* y;  // or NULL
+  uint16_t* operand;
+  float* inv_scale;
+  // the result of a projection cut into parts of K, fp32 [parts][rows][..]: added to x, which takes the sum (silu: the row
+  // is h = silu(gate) * up of its [2 K] results, x is not used)
+  const float* sums = nullptr;
+  int parts = 0;
+  bool silu = false;
+};
+cudaError_t launch_prefill_pack(const PrefillPackArgs& a, cudaStream_t s);
 struct PrefillGemmArgs {
   const uint32_t* qw;
   const uint16_t* scales;
@@ -214,10 +228,22 @@ struct PrefillGemmArgs {
   const int4* units = nullptr;
   const int* n_units = nullptr;
   int unit_rows = 0;
+  int experts = 1;         // experts stacked in the tensors
+  float* sums = nullptr;   // given: the results go there instead, as fp32 [parts][rows][N] (parts: prefill_tiling)
 };
 cudaError_t launch_prefill_gemm(const PrefillGemmArgs& a, cudaStream_t s);
+constexpr int kPrefillMaxParts = 16;
+struct PrefillTiling {
+  int tok_tiles, n_tile;
+  int parts;  // of K, worth using where the reader of the result can add fp32 sums up (1: none)
+};
+PrefillTiling prefill_tiling(int N, int K, int rows);
+// Bytes of `sums` any projection with parts > 1 needs (a part of K is used only while all tiles fit one wave).
+constexpr size_t kPrefillSumsBytes = (size_t)148 * 128 * 256 * 4;
 struct PrefillAttnArgs {
-  const uint16_t* qkv;     // bf16 [rows][(nq + 2 nkv) * 128]
+  const uint16_t* qkv;     // bf16 [rows][(nq + 2 nkv) * 128], or as fp32 parts of K [parts][rows][..] in sums
+  const float* sums;
+  int parts;
   uint16_t* q;             // bf16 [rows][nq][128] scratch: prepared queries
   const uint16_t* q_norm;  // or NULL
   const uint16_t* k_norm;

@@ -33,19 +33,76 @@ __device__ __forceinline__ uint32_t pack_f16x2(float lo, float hi) { return half
 
 // ---- operand ---------------------------------------------------------------------------------------------------
 // One CTA per row.  The row is held in registers (NCH chunks of 8 elements per thread).
+// fp32 results of a projection whose K was cut into parts, in part order: elements i, i + 1
+__device__ __forceinline__ float2 add_parts(const float* sums, size_t i, int parts, size_t stride) {
+  float2 v = *reinterpret_cast<const float2*>(sums + i);
+  for (int q = 1; q < parts; ++q) {
+    const float2 a = *reinterpret_cast<const float2*>(sums + q * stride + i);
+    v.x += a.x, v.y += a.y;
+  }
+  return v;
+}
+// eight of them, the parts' loads side by side
+__device__ __forceinline__ void add_parts8(const float* sums, size_t i, int parts, size_t stride, float (&v)[8]) {
+#pragma unroll
+  for (int k = 0; k < 8; ++k) v[k] = 0.0f;
+#pragma unroll 4
+  for (int q = 0; q < parts; ++q) {
+    const float4 a = *reinterpret_cast<const float4*>(sums + q * stride + i), b = *reinterpret_cast<const float4*>(sums + q * stride + i + 4);
+    v[0] += a.x, v[1] += a.y, v[2] += a.z, v[3] += a.w, v[4] += b.x, v[5] += b.y, v[6] += b.z, v[7] += b.w;
+  }
+}
+
 template <int NCH, bool NORM>
-__global__ void __launch_bounds__(256) prefill_pack_kernel(const uint16_t* x, int x_stride, const uint16_t* w, float eps, int K,
-                                                            uint16_t* y, uint16_t* operand, float* inv_scale) {
+__global__ void __launch_bounds__(256) prefill_pack_kernel(const PrefillPackArgs p) {
   extern __shared__ float s_sums[];  // [K / 64]
   __shared__ float red[8];
   grid_launch_dependents();
-  const int r = blockIdx.x, nch = K >> 3, warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int K = p.K, r = blockIdx.x, nch = K >> 3, warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const uint16_t* w = p.norm_w;
+  uint16_t* y = p.y;
   grid_dependency_wait();
   uint4 v[NCH];
 #pragma unroll
   for (int i = 0; i < NCH; ++i) {
     const int c = threadIdx.x + i * 256;
-    v[i] = c < nch ? *reinterpret_cast<const uint4*>(x + (size_t)r * x_stride + c * 8) : make_uint4(0u, 0u, 0u, 0u);
+    v[i] = make_uint4(0u, 0u, 0u, 0u);
+    if (c >= nch) continue;
+    uint16_t* px = p.x + (size_t)r * p.x_stride + c * 8;
+    if (!p.sums) {
+      v[i] = *reinterpret_cast<const uint4*>(px);
+      continue;
+    }
+    float a[8];
+    uint32_t o[4];
+    if (p.silu) {  // h = bf16(silu(bf16(gate)) * bf16(up))
+      float b[8];
+      const size_t at = (size_t)r * 2 * K + c * 8, stride = (size_t)p.rows * 2 * K;
+      add_parts8(p.sums, at, p.parts, stride, a);
+      add_parts8(p.sums, at + K, p.parts, stride, b);
+#pragma unroll
+      for (int k = 0; k < 4; ++k) {
+        float h[2];
+#pragma unroll
+        for (int q = 0; q < 2; ++q) {
+          const float gt = bf16_to_f32(f32_to_bf16(a[2 * k + q])), up = bf16_to_f32(f32_to_bf16(b[2 * k + q]));
+          h[q] = (gt / (1.0f + expf(-gt))) * up;
+        }
+        o[k] = pack_bf16x2(h[0], h[1]);
+      }
+      v[i] = make_uint4(o[0], o[1], o[2], o[3]);
+    } else {  // the residual stream takes the projection's result
+      add_parts8(p.sums, (size_t)r * K + c * 8, p.parts, (size_t)p.rows * K, a);
+      const uint4 old = *reinterpret_cast<const uint4*>(px);
+      const uint32_t ow[4] = {old.x, old.y, old.z, old.w};
+#pragma unroll
+      for (int k = 0; k < 4; ++k) {
+        const uint32_t d = pack_bf16x2(a[2 * k], a[2 * k + 1]);
+        o[k] = pack_bf16x2(bf16_lo(ow[k]) + bf16_lo(d), bf16_hi(ow[k]) + bf16_hi(d));
+      }
+      v[i] = make_uint4(o[0], o[1], o[2], o[3]);
+      *reinterpret_cast<uint4*>(px) = v[i];
+    }
   }
   auto block_reduce = [&](float a, bool is_max) -> float {
 #pragma unroll
@@ -70,7 +127,7 @@ __global__ void __launch_bounds__(256) prefill_pack_kernel(const uint16_t* x, in
       for (int j = 0; j < 4; ++j) ss = fmaf(bf16_lo(e[j]), bf16_lo(e[j]), ss), ss = fmaf(bf16_hi(e[j]), bf16_hi(e[j]), ss);
     }
     ss = block_reduce(ss, false);
-    const float inv = 1.0f / sqrtf(ss / (float)K + eps);
+    const float inv = 1.0f / sqrtf(ss / (float)K + p.eps);
 #pragma unroll
     for (int i = 0; i < NCH; ++i) {
       const int c = threadIdx.x + i * 256;
@@ -99,8 +156,8 @@ __global__ void __launch_bounds__(256) prefill_pack_kernel(const uint16_t* x, in
   top = block_reduce(top, true);
   const int ex = range_exponent(top);
   const float sc = pow2f(ex);
-  if (threadIdx.x == 0) inv_scale[r] = pow2f(-ex);
-  uint16_t* row = operand + (size_t)r * prefill_operand_stride(K);
+  if (threadIdx.x == 0) p.inv_scale[r] = pow2f(-ex);
+  uint16_t* row = p.operand + (size_t)r * prefill_operand_stride(K);
 #pragma unroll
   for (int i = 0; i < NCH; ++i) {
     const int c = threadIdx.x + i * 256;
@@ -126,24 +183,30 @@ __global__ void __launch_bounds__(256) prefill_pack_kernel(const uint16_t* x, in
 
 // ---- projections -------------------------------------------------------------------------------------------------
 // Persistent, one CTA per SM.  A tile is 128 weight rows (the lanes of tensor memory) x up to 256 tokens (columns); two
-// accumulators of 256 columns let the epilogue of a tile run under the MMAs of the next.  Roles:
-//   warp 0      producer: TMA loads of the tokens' operand, 64 features a stage (128-byte swizzle)
-//   warp 1      MMA issue (one thread); owns the tensor-memory allocation
+// accumulators of 256 columns let the epilogue of a tile run under the MMAs of the next.  K goes by in blocks of 64
+// features: 128 rows and the tokens as f16 with the 128-byte swizzle, in a ring of four to six stages.  Roles:
+//   warp 0      producer: TMA loads of the packed codes (128 rows x 128 features at a time) and of the tokens' operand
+//   warp 1      MMA issue; owns the tensor-memory allocation
 //   warps 2, 3  the power of two of each weight row of the next tile, the tokens' inverse scales
 //   warps 4..7  epilogue (one per lane quarter of tensor memory)
-//   warps 8..15 dequantisation: two threads per weight row, 32 codes each per stage, straight from global memory
-//               (four stages of codes in registers ahead) into the swizzled A stage
-// A dequantised code costs ~1.6 instructions, so a stage (128 x 64) costs the eight warps about 130 issue cycles per
-// scheduler against 512 cycles of tensor time at 256 tokens.  Measured at 2048 tokens, gate/up of the 8B shape (24576 x
-// 4096): 453 us = 0.91 PFLOP/s; as 128 passes of sixteen tokens the same projection took 3560 us.
+//   warps 8..15 dequantisation, shared memory to shared memory: four pairs, each of which fills every fourth block, a
+//               thread two of its rows
+// A dequantised code costs ~1.6 instructions, a block about 145 issue cycles per scheduler against 512 cycles of tensor
+// time at 256 tokens.  The chain wait - convert - store - fence - arrive - MMA - commit is several times longer than a
+// block, so four blocks are in the making at once and a pair converts its first row before it waits for the stage (all
+// eight warps on one block after another: 513 ns per block whatever the tile's width, 1.07 PFLOP/s on the gate/up
+// projection of the 8B shape at 2048 tokens; a single thread issuing under `lane == 0`: 605 ns, 0.91).  The codes come by
+// TMA: from global memory, 16 rows per load instruction, they cost 110 ns per block.
+// A projection with few tiles is cut along K as well: the parts' fp32 sums go to global memory, and the kernel that reads
+// the result (which exists anyway) adds them up.
 constexpr int kPgThreads = 512;
-constexpr int kPgStages = 4;
-constexpr int kPgAStage = 128 * 128;  // 128 rows x 64 f16
-constexpr int kPgBStage = 256 * 128;  // 256 tokens x 64 f16
-constexpr int kPgSmem = kPgStages * (kPgAStage + kPgBStage) + 1024;
+constexpr int kPgBlockCycles = 600;   // a block takes about this many cycles and one more per token (48 tokens: 650, 256: 840)
+constexpr int kPgABlock = 128 * 128;  // 128 rows x 64 f16
+constexpr int kPgCodes = 128 * 64;    // the codes of two blocks
+constexpr int kPgMaxStages = 6, kPgMaxCodes = 8;
+constexpr int kPgSmemBudget = 223 * 1024;
 
 struct PgParams {
-  const uint32_t* qw;
   const uint16_t* scales;
   const uint16_t* biases;
   const float* inv_scale;
@@ -152,6 +215,9 @@ struct PgParams {
   const int4* units;
   const int* n_units;
   int N, K, rows, n_tile, row_tiles, tok_tiles, out_stride, epilogue;
+  int stages, code_slots;  // depths of the rings
+  int parts;               // of K; `sums` given: the results are fp32 sums [part][rows][N] there
+  float* sums;
 };
 
 // D (128 x N, f32, tensor memory) (+)= A (128 x 16 f16) * B (N x 16 f16), both K-major in shared memory
@@ -177,11 +243,6 @@ __device__ __forceinline__ void tmem_ld16f(uint32_t taddr, float (&v)[16]) {
 #pragma unroll
   for (int i = 0; i < 16; ++i) v[i] = __uint_as_float(u[i]);
 }
-__device__ __forceinline__ uint4 ldg_stream(const void* p) {
-  uint4 v;
-  asm volatile("ld.global.nc.L1::no_allocate.v4.u32 {%0,%1,%2,%3}, [%4];" : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w) : "l"(p));
-  return v;
-}
 
 // 8 codes -> 8 f16 values s (q - 8) in the order 0,4,1,5,2,6,3,7
 __device__ __forceinline__ uint4 dequant_word(uint32_t w, __half2 s2) {
@@ -195,13 +256,20 @@ __device__ __forceinline__ uint4 dequant_word(uint32_t w, __half2 s2) {
   return make_uint4(half2_bits(__hmul2(a, s2)), half2_bits(__hmul2(b, s2)), half2_bits(__hmul2(c, s2)), half2_bits(__hmul2(d, s2)));
 }
 
+// The largest of four scales or biases, folded into a pair of running maxima of magnitudes.
+__device__ __forceinline__ uint32_t max_magnitude(uint32_t m, const uint2 v) {
+  return __vmaxu2(m, __vmaxu2(v.x & 0x7fff7fffu, v.y & 0x7fff7fffu));
+}
+
 struct PgTile {
   int row_tile, tok0, valid, expert;
 };
 
-__global__ void __launch_bounds__(kPgThreads, 1) prefill_gemm_kernel(const PgParams p, const __grid_constant__ CUtensorMap map_b) {
+__global__ void __launch_bounds__(kPgThreads, 1)
+prefill_gemm_kernel(const PgParams p, const __grid_constant__ CUtensorMap map_b, const __grid_constant__ CUtensorMap map_codes) {
   extern __shared__ unsigned char smem_raw[];
-  __shared__ __align__(8) uint64_t full[kPgStages], empty[kPgStages];
+  __shared__ __align__(8) uint64_t full[kPgMaxStages], empty[kPgMaxStages];      // operands of a stage
+  __shared__ __align__(8) uint64_t c_full[kPgMaxCodes], c_empty[kPgMaxCodes];    // codes of two blocks
   __shared__ __align__(8) uint64_t d_full[2], d_empty[2], rs_full[2], rs_empty[2];
   __shared__ uint32_t s_tmem_base;
   __shared__ int s_rexp[2][128];
@@ -210,15 +278,16 @@ __global__ void __launch_bounds__(kPgThreads, 1) prefill_gemm_kernel(const PgPar
   grid_launch_dependents();
 
   unsigned char* smem = reinterpret_cast<unsigned char*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~(uintptr_t)1023);
-  unsigned char* sA = smem;
-  unsigned char* sB = smem + kPgStages * kPgAStage;
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int NS = p.stages, NC = p.code_slots, b_block = p.n_tile * 128, stage_bytes = kPgABlock + b_block;
+  unsigned char* sC = smem + NS * stage_bytes;
+  const int warp = __shfl_sync(0xffffffffu, threadIdx.x >> 5, 0), lane = threadIdx.x & 31;
   const bool grouped = p.units != nullptr, silu = p.epilogue == EPI_SILU_PACK;
   const int half_n = p.N >> 1, K = p.K;
-  const int kb_main = K >> 6, kb_all = prefill_operand_stride(K) >> 6;
+  const int kb_main = K >> 6, kb_all = prefill_operand_stride(K) >> 6, kst = (kb_all + 1) >> 1;  // blocks, pairs of blocks
 
   if (threadIdx.x == 0) {
-    for (int s = 0; s < kPgStages; ++s) um_mbar_init(&full[s], 9), um_mbar_init(&empty[s], 1);
+    for (int s = 0; s < NS; ++s) um_mbar_init(&full[s], 3), um_mbar_init(&empty[s], 1);
+    for (int s = 0; s < NC; ++s) um_mbar_init(&c_full[s], 1), um_mbar_init(&c_empty[s], 4);
     for (int b = 0; b < 2; ++b)
       um_mbar_init(&d_full[b], 1), um_mbar_init(&d_empty[b], 4), um_mbar_init(&rs_full[b], 2), um_mbar_init(&rs_empty[b], 12);
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
@@ -227,15 +296,14 @@ __global__ void __launch_bounds__(kPgThreads, 1) prefill_gemm_kernel(const PgPar
     asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(&s_tmem_base)), "n"(512) : "memory");
     asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
   }
-  tc_fence_before();
-  __syncthreads();
-  tc_fence_after();
-  const uint32_t tbase = s_tmem_base;
-
   if (grouped) grid_dependency_wait();  // the list of units is the preceding kernel's
-  const int total = p.row_tiles * (grouped ? *p.n_units : p.tok_tiles);
+  const int total = p.row_tiles * (grouped ? *p.n_units : p.tok_tiles) * p.parts;
+  // with K in parts, the parts of a tile are neighbours in the list; a part is whole pairs of blocks
+  auto tile_kb0 = [&](int idx) -> int { return p.parts == 1 ? 0 : kst * (idx % p.parts) / p.parts * 2; };
+  auto tile_kb1 = [&](int idx) -> int { return p.parts == 1 ? kb_all : min(kb_all, kst * (idx % p.parts + 1) / p.parts * 2); };
   auto tile_at = [&](int idx) -> PgTile {
     PgTile t;
+    if (p.parts > 1) idx /= p.parts;
     if (grouped) {
       const int u = idx / p.row_tiles;
       const int4 un = p.units[u];
@@ -256,80 +324,138 @@ __global__ void __launch_bounds__(kPgThreads, 1) prefill_gemm_kernel(const PgPar
     }
     return (size_t)t.expert * p.N + r;
   };
+  // exponent of a row over the scales and biases of its whole K, by four neighbouring lanes
+  auto row_exponent = [&](const PgTile& t, int lrow) -> int {
+    const size_t off = tensor_row(t, lrow) * (size_t)kb_main + (lane & 3) * 4;
+    uint32_t ms = 0, mb = 0;
+#pragma unroll 4
+    for (int g = 0; g + (lane & 3) * 4 < kb_main; g += 16) {
+      ms = max_magnitude(ms, __ldg(reinterpret_cast<const uint2*>(p.scales + off + g)));
+      mb = max_magnitude(mb, __ldg(reinterpret_cast<const uint2*>(p.biases + off + g)));
+    }
+    float m = fmaxf(8.0f * fmaxf(bf16_lo(ms), bf16_hi(ms)), fmaxf(bf16_lo(mb), bf16_hi(mb)));
+    m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, 1));
+    m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, 2));
+    return range_exponent(m);
+  };
+  // the first tile's exponents, by everybody at once: nothing can be dequantised without them
+  if ((int)blockIdx.x < total) {
+    const int ex = row_exponent(tile_at(blockIdx.x), threadIdx.x >> 2);
+    if ((lane & 3) == 0) s_rexp[0][threadIdx.x >> 2] = ex;
+  }
+  tc_fence_before();
+  __syncthreads();
+  tc_fence_after();
+  const uint32_t tbase = s_tmem_base;
 
   bool ok = true;
   if (warp == 0) {
-    // ---- producer ----
-    if (lane == 0) {
-      if (!grouped) grid_dependency_wait();
-      int kb = 0;
-      for (int idx = blockIdx.x; idx < total && ok; idx += gridDim.x) {
-        const PgTile t = tile_at(idx);
-        for (int j = 0; j < kb_all; ++j, ++kb) {
-          const int s = kb % kPgStages;
-          if (!um_mbar_wait(&empty[s], (uint32_t)(((kb / kPgStages) & 1) ^ 1))) {
-            ok = false;
-            break;
+    // ---- producer: the whole warp walks, one lane issues.  Codes run ahead of the operand by their ring's depth; they
+    // do not depend on the preceding kernel. ----
+    int c_idx = blockIdx.x, c_kb, c_slot = 0;
+    uint32_t c_phase = 1u;
+    PgTile ct = tile_at(c_idx < total ? c_idx : 0);
+    int c_kb1 = tile_kb1(c_idx);
+    c_kb = tile_kb0(c_idx);
+    // Issues what fits: pairs up to `want` pairs from the start.  A slot that is still being read is left for later; it is
+    // free by the time the operand ring has turned, before anyone can be waiting for it.
+    int want = NC, issued = 0;
+    auto issue_codes = [&]() {
+      while (issued < want && c_idx < total) {
+        // (blocks of group sums have no codes; K is a multiple of 256, so no pair is half weights)
+        if (c_kb < kb_main) {
+          if (!um_mbar_test_warp(&c_empty[c_slot], c_phase)) return;
+          const int row0 = __shfl_sync(0xffffffffu, ct.expert * p.N + (silu ? ct.row_tile * 64 : ct.row_tile * 128), 0);
+          const int row1 = row0 + (silu ? half_n : 64), x = c_kb * 32;
+          if (elect_one()) {
+            um_mbar_expect_tx(&c_full[c_slot], (uint32_t)kPgCodes);
+            um_tma_2d(sC + c_slot * kPgCodes, &map_codes, x, row0, &c_full[c_slot]);
+            um_tma_2d(sC + c_slot * kPgCodes + 64 * 64, &map_codes, x, row1, &c_full[c_slot]);
           }
-          um_mbar_expect_tx(&full[s], (uint32_t)(p.n_tile * 128));
-          um_tma_2d(sB + s * kPgBStage, &map_b, j * 64, t.tok0, &full[s]);
+          __syncwarp();
+          if (++c_slot == NC) c_slot = 0, c_phase ^= 1u;
+        }
+        ++issued;
+        c_kb += 2;
+        if (c_kb >= c_kb1) {
+          c_idx += gridDim.x;
+          if (c_idx < total) ct = tile_at(c_idx), c_kb = tile_kb0(c_idx), c_kb1 = tile_kb1(c_idx);
         }
       }
-      if (!ok && p.status) atomicExch(p.status, 3u);
+    };
+    issue_codes();
+    if (!grouped) grid_dependency_wait();
+    int s = 0;
+    uint32_t phase = 1u;
+    for (int idx = blockIdx.x; idx < total && ok; idx += gridDim.x) {
+      const PgTile t = tile_at(idx);
+      const int tok0 = __shfl_sync(0xffffffffu, t.tok0, 0);
+      const int kb0 = tile_kb0(idx), kb1 = tile_kb1(idx);
+      for (int j = kb0; j < kb1 && ok; ++j) {
+        if (!um_mbar_wait_warp(&empty[s], phase)) {
+          ok = false;
+          break;
+        }
+        if (elect_one()) {
+          um_mbar_expect_tx(&full[s], (uint32_t)b_block);
+          um_tma_2d(smem + s * stage_bytes + kPgABlock, &map_b, j * 64, tok0, &full[s]);
+        }
+        __syncwarp();
+        if (++s == NS) s = 0, phase ^= 1u;
+        if (j & 1) ++want;
+        issue_codes();
+      }
+      if ((kb1 - kb0) & 1) ++want;
     }
-    __syncwarp();
+    if (!ok && lane == 0 && p.status) atomicExch(p.status, 3u);
   } else if (warp == 1) {
-    // ---- MMA issue ----
-    if (lane == 0) {
-      // D f32, A and B f16, both K-major, M = 128
-      const uint32_t idesc = (1u << 4) | ((uint32_t)(p.n_tile >> 3) << 17) | ((128u >> 4) << 24);
-      int kb = 0, it = 0;
-      for (int idx = blockIdx.x; idx < total && ok; idx += gridDim.x, ++it) {
-        const int buf = it & 1;
-        if (!um_mbar_wait(&d_empty[buf], (uint32_t)(((it >> 1) & 1) ^ 1))) ok = false;
+    // ---- MMA issue: the whole warp walks, one lane issues ----
+    // D f32, A and B f16, both K-major, M = 128
+    const uint32_t idesc = (1u << 4) | ((uint32_t)(p.n_tile >> 3) << 17) | ((128u >> 4) << 24);
+    const uint32_t smem_a = smem_u32(smem);
+    int s = 0, it = 0;
+    uint32_t phase = 0u;
+    for (int idx = blockIdx.x; idx < total && ok; idx += gridDim.x, ++it) {
+      const int buf = it & 1, kb0 = tile_kb0(idx), kb1 = tile_kb1(idx);
+      if (!um_mbar_wait_warp(&d_empty[buf], (uint32_t)(((it >> 1) & 1) ^ 1))) ok = false;
+      for (int j = kb0; j < kb1 && ok; ++j) {
+        if (!um_mbar_wait_warp(&full[s], phase)) {
+          ok = false;
+          break;
+        }
         tc_fence_after();
-        for (int j = 0; j < kb_all && ok; ++j, ++kb) {
-          const int s = kb % kPgStages;
-          if (!um_mbar_wait(&full[s], (uint32_t)((kb / kPgStages) & 1))) {
-            ok = false;
-            break;
-          }
-          tc_fence_after();
-          const uint64_t da = desc_sw128(smem_u32(sA + s * kPgAStage)), db = desc_sw128(smem_u32(sB + s * kPgBStage));
+        if (elect_one()) {
+          const uint32_t base = smem_a + (uint32_t)(s * stage_bytes);
+          const uint64_t da = desc_sw128(base), db = desc_sw128(base + kPgABlock);
 #pragma unroll
           for (int ks = 0; ks < 4; ++ks)
-            umma_f16_ss(tbase + (uint32_t)(buf * 256), da + (uint64_t)(ks * 2), db + (uint64_t)(ks * 2), idesc, (j | ks) != 0);
+            umma_f16_ss(tbase + (uint32_t)(buf * 256), da + (uint64_t)(ks * 2), db + (uint64_t)(ks * 2), idesc, j != kb0 || ks != 0);
           umma_commit(&empty[s]);
+          if (j == kb1 - 1) umma_commit(&d_full[buf]);
         }
-        if (ok) umma_commit(&d_full[buf]);
+        __syncwarp();
+        if (++s == NS) s = 0, phase ^= 1u;
       }
-      if (!ok && p.status) atomicExch(p.status, 3u);
     }
-    __syncwarp();
+    if (!ok && lane == 0 && p.status) atomicExch(p.status, 3u);
   } else if (warp < 4) {
-    // ---- row exponents and token scales, a tile ahead ----
+    // ---- token scales of a tile, and the row exponents of the next one ----
     const int tid = threadIdx.x - 64;
+    if (!grouped) grid_dependency_wait();
     int it = 0;
     for (int idx = blockIdx.x; idx < total && ok; idx += gridDim.x, ++it) {
       const PgTile t = tile_at(idx);
       const int buf = it & 1;
-      int ex[2];
+      int ex[8];
+      if (it > 0) {
 #pragma unroll
-      for (int h = 0; h < 2; ++h) {
-        const size_t off = tensor_row(t, tid + 64 * h) * (size_t)(K >> 6);
-        uint32_t ms = 0, mb = 0;
-#pragma unroll 8
-        for (int g = 0; g < (K >> 6); g += 4) {
-          const uint2 a = *reinterpret_cast<const uint2*>(p.scales + off + g), b = *reinterpret_cast<const uint2*>(p.biases + off + g);
-          ms = __vmaxu2(ms, __vmaxu2(a.x & 0x7fff7fffu, a.y & 0x7fff7fffu));
-          mb = __vmaxu2(mb, __vmaxu2(b.x & 0x7fff7fffu, b.y & 0x7fff7fffu));
-        }
-        const float fs = fmaxf(bf16_lo(ms), bf16_hi(ms)), fb = fmaxf(bf16_lo(mb), bf16_hi(mb));
-        ex[h] = range_exponent(fmaxf(8.0f * fs, fb));
+        for (int i = 0; i < 8; ++i) ex[i] = row_exponent(t, i * 16 + (tid >> 2));
       }
-      if (it == 0 && !grouped) grid_dependency_wait();
       if (!um_mbar_wait_warp(&rs_empty[buf], (uint32_t)(((it >> 1) & 1) ^ 1))) ok = false;
-      s_rexp[buf][tid] = ex[0], s_rexp[buf][tid + 64] = ex[1];
+      if (it > 0 && (lane & 3) == 0) {
+#pragma unroll
+        for (int i = 0; i < 8; ++i) s_rexp[buf][i * 16 + (tid >> 2)] = ex[i];
+      }
       for (int i = tid; i < p.n_tile; i += 64) s_inv[buf][i] = i < t.valid ? p.inv_scale[t.tok0 + i] : 0.0f;
       __syncwarp();
       if (lane == 0) um_mbar_arrive(&rs_full[buf]);
@@ -360,7 +486,12 @@ __global__ void __launch_bounds__(kPgThreads, 1) prefill_gemm_kernel(const PgPar
           v[i] = v[i] * rinv * cs.x, v[i + 1] = v[i + 1] * rinv * cs.y;
           v[i + 2] = v[i + 2] * rinv * cs.z, v[i + 3] = v[i + 3] * rinv * cs.w;
         }
-        if (silu) {
+        if (p.sums) {
+          float* d = p.sums + ((size_t)(idx % p.parts) * p.rows + t.tok0 + c0) * p.N + tensor_row(t, q * 32 + lane);
+#pragma unroll
+          for (int i = 0; i < 16; ++i)
+            if (c0 + i < t.valid) d[(size_t)i * p.N] = v[i];
+        } else if (silu) {
           // lanes 0..15 hold gate rows, 16..31 the up rows of the same features.  Of columns c, c + 1 the lower half
           // takes c, the upper c + 1; then neighbours pair up so that a lane stores two features of one token.
 #pragma unroll
@@ -406,91 +537,126 @@ __global__ void __launch_bounds__(kPgThreads, 1) prefill_gemm_kernel(const PgPar
     }
     if (!ok && lane == 0 && p.status) atomicExch(p.status, 3u);
   } else {
-    // ---- dequantisation ----
-    const int tid = threadIdx.x - 256, lrow = tid >> 1, h = tid & 1;
-    const int nsb = K >> 8;  // superblocks of four stages: 128 bytes of codes per row
-    const uint32_t* qrow = nullptr;
-    const uint16_t *srow = nullptr, *brow = nullptr;
-    auto set_row = [&](const PgTile& t) {
-      const size_t r = tensor_row(t, lrow);
-      qrow = p.qw + r * (size_t)(K >> 3) + h * 4;
-      srow = p.scales + r * (size_t)(K >> 6), brow = p.biases + r * (size_t)(K >> 6);
-    };
-    uint4 nxt[4];
-    uint2 nsc;
-    auto load_sb = [&](int sb) {
+    // ---- dequantisation: pair `grp` fills blocks b with b % 4 == grp (counted over all tiles), thread i rows i, i + 64 ----
+    const int grp = (warp - 8) >> 1, tid = (warp & 1) * 32 + lane;
+    // where the codes of tensor_row(row) are: with the SiLU epilogue a code slot holds 64 gate rows, then 64 up rows
+    const unsigned char* c_row[2];
+    int c_swz[2];
 #pragma unroll
-      for (int j = 0; j < 4; ++j) nxt[j] = ldg_stream(qrow + sb * 32 + j * 8);
-      nsc = *reinterpret_cast<const uint2*>(srow + sb * 4);
-    };
-    if (blockIdx.x < total) {
-      set_row(tile_at(blockIdx.x));
-      load_sb(0);
+    for (int i = 0; i < 2; ++i) {
+      const int row = tid + 64 * i, crow = silu ? (row >> 5) * 16 + (row & 15) + ((row & 16) ? 64 : 0) : row;
+      c_row[i] = sC + crow * 64, c_swz[i] = (crow >> 1) & 3;  // (64-byte swizzle)
     }
-    // where this thread's four 16-byte chunks of a stage go
-    unsigned char* a_row = sA + lrow * 128;
-    int a_off[4];
+    unsigned char* a_row = smem + tid * 128;
+    int a_off[8];  // rows 64 apart share the swizzle
 #pragma unroll
-    for (int i = 0; i < 4; ++i) a_off[i] = ((h * 4 + i) ^ (lrow & 7)) << 4;
-    int kb = 0, it = 0;
+    for (int i = 0; i < 8; ++i) a_off[i] = (i ^ (tid & 7)) << 4;
+    const uint16_t *srow[2], *brow[2];
+    uint16_t nsc[2] = {0, 0};
+    auto set_tile = [&](const PgTile& t) {
+#pragma unroll
+      for (int i = 0; i < 2; ++i) {
+        const size_t r = tensor_row(t, tid + 64 * i) * (size_t)kb_main;
+        srow[i] = p.scales + r, brow[i] = p.biases + r;
+      }
+    };
+    auto load_scales = [&](int j) {
+#pragma unroll
+      for (int i = 0; i < 2; ++i) nsc[i] = __ldg(srow[i] + j);
+    };
+    int base = 0;  // blocks before this tile, modulo 4
+    int s = grp, it = 0, c_slot = 0, c_seen = 0;  // c_seen: the code slot the pair looks at, counted from the tile's first
+    uint32_t phase = 1u, c_phase = 0u;
+    while (s >= NS) s -= NS, phase ^= 1u;
+    auto next_code_slot = [&](int n) {
+      for (int i = 0; i < n; ++i)
+        if (++c_slot == NC) c_slot = 0, c_phase ^= 1u;
+    };
     for (int idx = blockIdx.x; idx < total && ok; idx += gridDim.x, ++it) {
-      const int buf = it & 1;
-      if (!um_mbar_wait_warp(&rs_full[buf], (uint32_t)((it >> 1) & 1))) {
+      const int buf = it & 1, kb0 = tile_kb0(idx), kb1 = tile_kb1(idx), kc1 = min(kb1, kb_main);
+      int j = kb0 + ((grp - base) & 3);
+      set_tile(tile_at(idx));
+      if (j < kc1) load_scales(j);
+      if (it > 0 && !um_mbar_wait_warp(&rs_full[buf], (uint32_t)((it >> 1) & 1))) {
         ok = false;
         break;
       }
-      const float rs = pow2f(s_rexp[buf][lrow]);
-      const uint16_t* my_sb = h ? srow : brow;  // the bias stages: biases (h = 0) or 8 x scales (h = 1)
-      const float my_f = h ? 8.0f * rs : rs;
-      for (int sb = 0; sb < nsb && ok; ++sb) {
-        const uint4 cur[4] = {nxt[0], nxt[1], nxt[2], nxt[3]};
-        const uint2 csc = nsc;
-        if (sb + 1 < nsb) {
-          load_sb(sb + 1);
-        } else if (idx + (int)gridDim.x < total) {
-          set_row(tile_at(idx + gridDim.x));
-          load_sb(0);
-        }
+      float rs[2];
 #pragma unroll
-        for (int j = 0; j < 4; ++j, ++kb) {
-          const int s = kb % kPgStages;
-          const uint32_t sw = j < 2 ? csc.x : csc.y;
-          const __half2 s2 = __float2half2_rn(((j & 1) ? bf16_hi(sw) : bf16_lo(sw)) * rs);
-          uint4 a[4];
-          a[0] = dequant_word(cur[j].x, s2), a[1] = dequant_word(cur[j].y, s2);
-          a[2] = dequant_word(cur[j].z, s2), a[3] = dequant_word(cur[j].w, s2);
-          if (ok && !um_mbar_wait_warp(&empty[s], (uint32_t)(((kb / kPgStages) & 1) ^ 1))) ok = false;
-          if (!ok) break;
+      for (int i = 0; i < 2; ++i) rs[i] = pow2f(s_rexp[buf][tid + 64 * i]);
+      c_seen = 0;
+      for (; j < kb1; j += 4) {
+        unsigned char* dst = a_row + s * stage_bytes;
+        if (j < kb_main) {
+          const int slot_of = (j - kb0) >> 1;
+          next_code_slot(slot_of - c_seen);
+          c_seen = slot_of;
+          __half2 s2[2];
 #pragma unroll
-          for (int i = 0; i < 4; ++i) *reinterpret_cast<uint4*>(a_row + s * kPgAStage + a_off[i]) = a[i];
-          asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+          for (int i = 0; i < 2; ++i) s2[i] = __float2half2_rn(bf16_to_f32(nsc[i]) * rs[i]);
+          if (j + 4 < kc1) load_scales(j + 4);
+          if (!um_mbar_wait_warp(&c_full[c_slot], c_phase)) {
+            ok = false;
+            break;
+          }
+          uint4 w[2][2];
+#pragma unroll
+          for (int i = 0; i < 2; ++i)
+#pragma unroll
+            for (int c = 0; c < 2; ++c)
+              w[i][c] = *reinterpret_cast<const uint4*>(c_row[i] + c_slot * kPgCodes + ((((j & 1) * 2 + c) ^ c_swz[i]) << 4));
           __syncwarp();
-          if (lane == 0) um_mbar_arrive(&full[s]);
+          if (lane == 0) um_mbar_arrive(&c_empty[c_slot]);
+          uint4 a[8];
+          auto convert = [&](const uint4 (&v)[2], const __half2 sc) {
+            a[0] = dequant_word(v[0].x, sc), a[1] = dequant_word(v[0].y, sc), a[2] = dequant_word(v[0].z, sc), a[3] = dequant_word(v[0].w, sc);
+            a[4] = dequant_word(v[1].x, sc), a[5] = dequant_word(v[1].y, sc), a[6] = dequant_word(v[1].z, sc), a[7] = dequant_word(v[1].w, sc);
+          };
+          convert(w[0], s2[0]);
+          if (!um_mbar_wait_warp(&empty[s], phase)) {
+            ok = false;
+            break;
+          }
+#pragma unroll
+          for (int c = 0; c < 8; ++c) *reinterpret_cast<uint4*>(dst + a_off[c]) = a[c];
+          convert(w[1], s2[1]);
+#pragma unroll
+          for (int c = 0; c < 8; ++c) *reinterpret_cast<uint4*>(dst + 64 * 128 + a_off[c]) = a[c];
+        } else {
+          // 16 groups: {b, b} against {X1, X2}, {8 s, 8 s} against the same
+          const int e = (j - kb_main) * 16;
+          if (!um_mbar_wait_warp(&empty[s], phase)) {
+            ok = false;
+            break;
+          }
+#pragma unroll
+          for (int i = 0; i < 2; ++i)
+#pragma unroll
+            for (int q = 0; q < 2; ++q) {  // scales or biases of 16 groups
+              const uint16_t* src = (q ? srow[i] : brow[i]) + e;
+              const float f = q ? 8.0f * rs[i] : rs[i];
+              uint32_t o[8];
+#pragma unroll
+              for (int c = 0; c < 4; ++c) {
+                const uint2 v = e + c * 4 < kb_main ? __ldg(reinterpret_cast<const uint2*>(src + c * 4)) : make_uint2(0u, 0u);
+                o[2 * c] = pack_f16x2(bf16_lo(v.x) * f, bf16_hi(v.x) * f), o[2 * c + 1] = pack_f16x2(bf16_lo(v.y) * f, bf16_hi(v.y) * f);
+              }
+#pragma unroll
+              for (int c = 0; c < 4; ++c)
+                *reinterpret_cast<uint4*>(dst + i * (64 * 128) + a_off[q * 4 + c]) =
+                    make_uint4(o[(c & 1) * 4], o[(c & 1) * 4 + 1], o[(c & 1) * 4 + 2], o[(c & 1) * 4 + 3]);
+            }
         }
-      }
-      for (int e = 0; e < kb_all - kb_main && ok; ++e, ++kb) {
-        const int s = kb % kPgStages;
-        uint2 w[4];
-#pragma unroll
-        for (int i = 0; i < 4; ++i)
-          w[i] = e * 16 + i * 4 < kb_main ? *reinterpret_cast<const uint2*>(my_sb + e * 16 + i * 4) : make_uint2(0u, 0u);
-        uint4 c[2];
-#pragma unroll
-        for (int i = 0; i < 2; ++i)
-          c[i] = make_uint4(pack_f16x2(bf16_lo(w[2 * i].x) * my_f, bf16_hi(w[2 * i].x) * my_f),
-                            pack_f16x2(bf16_lo(w[2 * i].y) * my_f, bf16_hi(w[2 * i].y) * my_f),
-                            pack_f16x2(bf16_lo(w[2 * i + 1].x) * my_f, bf16_hi(w[2 * i + 1].x) * my_f),
-                            pack_f16x2(bf16_lo(w[2 * i + 1].y) * my_f, bf16_hi(w[2 * i + 1].y) * my_f));
-        if (!um_mbar_wait_warp(&empty[s], (uint32_t)(((kb / kPgStages) & 1) ^ 1))) {
-          ok = false;
-          break;
-        }
-#pragma unroll
-        for (int i = 0; i < 4; ++i) *reinterpret_cast<uint4*>(a_row + s * kPgAStage + a_off[i]) = c[i & 1];
         asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
         __syncwarp();
         if (lane == 0) um_mbar_arrive(&full[s]);
+        s += 4;
+        while (s >= NS) s -= NS, phase ^= 1u;
       }
+      base = (base + kb1 - kb0) & 3;
+      // the tile's code slots this pair did not look at go by as well
+      if (kc1 > kb0) next_code_slot(((kc1 - kb0) >> 1) - c_seen);
+      __syncwarp();
       if (ok && lane == 0) um_mbar_arrive(&rs_empty[buf]);
     }
     if (!ok && lane == 0 && p.status) atomicExch(p.status, 3u);
@@ -512,9 +678,16 @@ __global__ void __launch_bounds__(256) prefill_rope_kernel(const PrefillAttnArgs
   const float4 cs = *reinterpret_cast<const float4*>(p.rope + ((size_t)pos * 64 + 2 * lane) * 2);  // c0 s0 c1 s1
   const int blk = p.block_table[pos / kBlockSize], slot = pos % kBlockSize;
   for (int hd = warp; hd < heads; hd += 8) {
-    const uint16_t* src = p.qkv + ((size_t)r * heads + hd) * kHeadDim;
+    const size_t at = ((size_t)r * heads + hd) * kHeadDim + 2 * lane;
     // lane holds elements 2*lane, 2*lane+1 and their rotary partners 64 + 2*lane, 64 + 2*lane + 1
-    const uint32_t wa = *reinterpret_cast<const uint32_t*>(src + 2 * lane), wb = *reinterpret_cast<const uint32_t*>(src + 64 + 2 * lane);
+    uint32_t wa, wb;
+    if (p.sums) {
+      const size_t stride = (size_t)p.rows * heads * kHeadDim;
+      const float2 a = add_parts(p.sums, at, p.parts, stride), b = add_parts(p.sums, at + 64, p.parts, stride);
+      wa = pack_bf16x2(a.x, a.y), wb = pack_bf16x2(b.x, b.y);
+    } else {
+      wa = *reinterpret_cast<const uint32_t*>(p.qkv + at), wb = *reinterpret_cast<const uint32_t*>(p.qkv + at + 64);
+    }
     uint32_t oa = wa, ob = wb;
     if (hd < p.nq + p.nkv) {
       float a0 = bf16_lo(wa), a1 = bf16_hi(wa), b0 = bf16_lo(wb), b1 = bf16_hi(wb);
@@ -694,20 +867,20 @@ cudaError_t prefill_init() {
   int dev = 0, sms = 0;
   cudaError_t e = cudaGetDevice(&dev);
   if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-  if (e == cudaSuccess) e = cudaFuncSetAttribute(prefill_gemm_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kPgSmem);
+  if (e == cudaSuccess) e = cudaFuncSetAttribute(prefill_gemm_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kPgSmemBudget);
   if (e == cudaSuccess) e = cudaFuncSetAttribute(prefill_attention_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kPaSmem);
   if (e == cudaSuccess) g_prefill_sms = sms;
   return e;
 }
 
-cudaError_t launch_prefill_pack(const uint16_t* x, int x_stride, const uint16_t* norm_w, float eps, int rows, int K, uint16_t* y,
-                                uint16_t* operand, float* inv_scale, cudaStream_t s) {
-  if (rows <= 0) return cudaSuccess;
-  if (K % 256 || K > kPrefillMaxWidth || x_stride % 8) return cudaErrorInvalidValue;
+cudaError_t launch_prefill_pack(const PrefillPackArgs& a, cudaStream_t s) {
+  if (a.rows <= 0) return cudaSuccess;
+  const int K = a.K;
+  if (K % 256 || K > kPrefillMaxWidth || a.x_stride % 8) return cudaErrorInvalidValue;
   const size_t smem = (size_t)(K >> 6) * sizeof(float);
-  auto go = [&](auto kernel) { return launch_kernel(kernel, dim3(rows), dim3(256), smem, s, x, x_stride, norm_w, eps, K, y, operand, inv_scale); };
+  auto go = [&](auto kernel) { return launch_kernel(kernel, dim3(a.rows), dim3(256), smem, s, a); };
   const int nch = (K + 2047) / 2048;
-  if (norm_w) {
+  if (a.norm_w) {
     if (nch <= 1) return go(prefill_pack_kernel<1, true>);
     if (nch <= 2) return go(prefill_pack_kernel<2, true>);
     if (nch <= 4) return go(prefill_pack_kernel<4, true>);
@@ -719,6 +892,27 @@ cudaError_t launch_prefill_pack(const uint16_t* x, int x_stride, const uint16_t*
   return nch <= 8 ? go(prefill_pack_kernel<8, false>) : go(prefill_pack_kernel<16, false>);
 }
 
+// Token tiles of equal width (a multiple of 16, at most 256) so that waves x time per block is smallest.  Parts of K where
+// even so under half of the SMs get a tile: at least four blocks each.
+PrefillTiling prefill_tiling(int N, int K, int rows) {
+  const int sms = g_prefill_sms > 0 ? g_prefill_sms : 148, row_tiles = N / 128;
+  PrefillTiling best = {1, 16, 1};
+  long long best_cost = -1;
+  for (int k = (rows + 255) / 256; k <= (rows + 95) / 96 + 1; ++k) {
+    const int n = ((rows + k - 1) / k + 15) & ~15, tiles = (rows + n - 1) / n;
+    const long long waves = ((long long)row_tiles * tiles + sms - 1) / sms, cost = waves * (kPgBlockCycles + n);
+    if (best_cost < 0 || cost < best_cost) best_cost = cost, best.tok_tiles = tiles, best.n_tile = n;
+  }
+  const int tiles = row_tiles * best.tok_tiles, stages = (prefill_operand_stride(K) / 64 + 1) / 2;
+  if (tiles * 2 <= sms) {
+    best.parts = sms / tiles;
+    if (best.parts > stages / 2) best.parts = stages / 2;
+    if (best.parts > kPrefillMaxParts) best.parts = kPrefillMaxParts;
+    if (best.parts < 1) best.parts = 1;
+  }
+  return best;
+}
+
 cudaError_t launch_prefill_gemm(const PrefillGemmArgs& a, cudaStream_t s) {
   if (g_prefill_sms == 0) {
     cudaError_t e = prefill_init();
@@ -726,33 +920,51 @@ cudaError_t launch_prefill_gemm(const PrefillGemmArgs& a, cudaStream_t s) {
   }
   if (a.rows <= 0) return cudaSuccess;
   const bool grouped = a.units != nullptr;
-  if (a.N % 128 || a.K % 256 || a.K > kPrefillMaxWidth || (grouped && (!a.n_units || a.unit_rows % 16 || a.unit_rows < 16 || a.unit_rows > 256)))
+  if (a.N % 128 || a.K % 256 || a.K > kPrefillMaxWidth || (grouped && (!a.n_units || a.sums || a.unit_rows % 16 || a.unit_rows < 16 || a.unit_rows > 256)))
     return cudaErrorInvalidValue;
   PgParams p;
-  p.qw = a.qw, p.scales = a.scales, p.biases = a.biases, p.inv_scale = a.inv_scale, p.out = a.out, p.status = a.status;
+  p.scales = a.scales, p.biases = a.biases, p.inv_scale = a.inv_scale, p.out = a.out, p.status = a.status;
   p.units = a.units, p.n_units = a.n_units;
   p.N = a.N, p.K = a.K, p.rows = a.rows, p.out_stride = a.out_stride, p.epilogue = a.epilogue;
-  p.row_tiles = a.N / 128;
+  p.row_tiles = a.N / 128, p.parts = 1, p.sums = a.sums;
   if (grouped) {
     p.n_tile = a.unit_rows, p.tok_tiles = 0;
-  } else {  // equal token tiles of at most 256, a multiple of 16 each
-    p.tok_tiles = (a.rows + 255) / 256;
-    p.n_tile = ((a.rows + p.tok_tiles - 1) / p.tok_tiles + 15) & ~15;
+  } else {
+    const PrefillTiling t = prefill_tiling(a.N, a.K, a.rows);
+    p.tok_tiles = t.tok_tiles, p.n_tile = t.n_tile;
+    if (a.sums) p.parts = t.parts;
   }
+  // narrow tiles pass through a stage faster, and their smaller operand leaves room for more codes ahead
+  p.code_slots = p.n_tile <= 128 ? kPgMaxCodes : 3;
+  const int stage = kPgABlock + p.n_tile * 128;
+  p.stages = (kPgSmemBudget - 1024 - p.code_slots * kPgCodes) / stage;
+  if (p.stages > kPgMaxStages) p.stages = kPgMaxStages;
+  const size_t smem = 1024 + (size_t)p.stages * stage + (size_t)p.code_slots * kPgCodes;
   EncodeTiledFn encode = nullptr;
   cudaError_t e = encode_tiled_fn(&encode);
   if (e != cudaSuccess) return e;
   const int stride = prefill_operand_stride(a.K);
-  const cuuint64_t dims[2] = {(cuuint64_t)stride, (cuuint64_t)a.operand_rows}, strides[1] = {(cuuint64_t)stride * 2};
-  const cuuint32_t box[2] = {64u, (cuuint32_t)p.n_tile}, elem[2] = {1u, 1u};
-  CUtensorMap map;
-  if (encode(&map, CU_TENSOR_MAP_DATA_TYPE_FLOAT16, 2, const_cast<uint16_t*>(a.operand), dims, strides, box, elem,
-             CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
-             CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) != CUDA_SUCCESS)
-    return cudaErrorInvalidValue;
+  const cuuint32_t elem[2] = {1u, 1u};
+  CUtensorMap map_b, map_codes;
+  {
+    const cuuint64_t dims[2] = {(cuuint64_t)stride, (cuuint64_t)a.operand_rows}, strides[1] = {(cuuint64_t)stride * 2};
+    const cuuint32_t box[2] = {64u, (cuuint32_t)p.n_tile};
+    if (encode(&map_b, CU_TENSOR_MAP_DATA_TYPE_FLOAT16, 2, const_cast<uint16_t*>(a.operand), dims, strides, box, elem,
+               CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
+               CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) != CUDA_SUCCESS)
+      return cudaErrorInvalidValue;
+  }
+  {
+    const cuuint64_t dims[2] = {(cuuint64_t)(a.K / 2), (cuuint64_t)a.N * a.experts}, strides[1] = {(cuuint64_t)(a.K / 2)};
+    const cuuint32_t box[2] = {64u, 64u};
+    if (encode(&map_codes, CU_TENSOR_MAP_DATA_TYPE_UINT8, 2, const_cast<uint32_t*>(a.qw), dims, strides, box, elem,
+               CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_64B, CU_TENSOR_MAP_L2_PROMOTION_L2_128B,
+               CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) != CUDA_SUCCESS)
+      return cudaErrorInvalidValue;
+  }
   int ctas = g_prefill_sms;
-  if (!grouped) ctas = p.row_tiles * p.tok_tiles < ctas ? p.row_tiles * p.tok_tiles : ctas;
-  return launch_kernel(prefill_gemm_kernel, dim3(ctas), dim3(kPgThreads), kPgSmem, s, p, map);
+  if (!grouped && p.row_tiles * p.tok_tiles * p.parts < ctas) ctas = p.row_tiles * p.tok_tiles * p.parts;
+  return launch_kernel(prefill_gemm_kernel, dim3(ctas), dim3(kPgThreads), smem, s, p, map_b, map_codes);
 }
 
 cudaError_t launch_prefill_rope_append(const PrefillAttnArgs& a, cudaStream_t s) {

@@ -134,12 +134,6 @@ constexpr int kSliceSlots = 3;  // ring slots per warp
 __host__ __device__ constexpr int slice_slot_codes(int nt) { return slice_sub(nt) * 16 * 128; }
 constexpr int kSliceSb = 2 * 16 * 16;  // of a slot: scales, then biases, 16 bytes a row
 
-// one lane of the converged warp
-__device__ __forceinline__ bool elect_one() {
-  uint32_t is;
-  asm volatile("{\n\t.reg .pred p;\n\telect.sync _|p, 0xffffffff;\n\tselp.u32 %0, 1, 0, p;\n\t}" : "=r"(is));
-  return is != 0;
-}
 __device__ __forceinline__ void mbar_expect_tx_addr(uint32_t bar, uint32_t bytes) {
   asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(bar), "r"(bytes) : "memory");
 }

@@ -8,6 +8,14 @@
 
 namespace q4d {
 
+// one lane of the converged warp.  What follows under it stays uniform for the compiler: coordinates, descriptors and
+// addresses of TMA and tcgen05 instructions, which take uniform registers only, come from there instead of a loop per
+// instruction that moves them out of vector registers (as under `lane == 0`).
+__device__ __forceinline__ bool elect_one() {
+  uint32_t is;
+  asm volatile("{\n\t.reg .pred p;\n\telect.sync _|p, 0xffffffff;\n\tselp.u32 %0, 1, 0, p;\n\t}" : "=r"(is));
+  return is != 0;
+}
 __device__ __forceinline__ void um_mbar_init(uint64_t* bar, uint32_t count) {
   asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(smem_u32(bar)), "r"(count) : "memory");
 }
@@ -57,6 +65,15 @@ __device__ __forceinline__ bool um_mbar_wait_warp(uint64_t* bar, uint32_t parity
     if (__all_sync(0xffffffffu, done != 0u)) return true;
   }
   return false;
+}
+// Whether the phase has completed, without waiting; the verdict is the warp's.
+__device__ __forceinline__ bool um_mbar_test_warp(uint64_t* bar, uint32_t parity) {
+  uint32_t done;
+  asm volatile("{\n\t.reg .pred p;\n\tmbarrier.test_wait.parity.shared::cta.b64 p, [%1], %2;\n\tselp.u32 %0, 1, 0, p;\n\t}"
+               : "=r"(done)
+               : "r"(smem_u32(bar)), "r"(parity)
+               : "memory");
+  return __all_sync(0xffffffffu, done != 0u);
 }
 __device__ __forceinline__ void tc_fence_before() { asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory"); }
 __device__ __forceinline__ void tc_fence_after() { asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory"); }
