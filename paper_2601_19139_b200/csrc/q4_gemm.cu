@@ -123,6 +123,7 @@ struct SliceParams {
   int T;       // row tiles of 16 rows (SiLU epilogue: 8 gate rows and the 8 matching up rows)
   int kw, rg;  // kslices and row groups of a CTA: kw * rg warps
   int batch;   // rounds between two meetings
+  int slots;   // ring slots of a warp in use (kSliceSlots, or fewer where a warp has fewer stages)
   int vec_ok;
 };
 // A CTA covers at most 4096 features: 16 warps of one stage (256 features) each, or with 16 requests, whose operand takes 64
@@ -185,8 +186,9 @@ __device__ __forceinline__ void silu_epilogue(const float (&v)[4], uint16_t* out
 // Epilogue of 16 rows x 8 requests (nt: which 8) from an accumulator fragment (lane holds rows g, g + 8 and requests 2t,
 // 2t + 1), without a detour through shared memory: fp32 results leave in 32-byte pieces as they lie, bf16 results are
 // transposed in registers.  best, bidx: the lane's running argmax for its two requests (EPI_F32).
-__device__ __forceinline__ void slice_epilogue(const SliceParams& p, float (&v)[4], int tile, int nt, int g, int t,
-                                               float (&best)[2], int (&bidx)[2]) {
+// old: the residual stream's values there, where the caller has them already (EPI_RESIDUAL).
+__device__ __forceinline__ void slice_epilogue(const SliceParams& p, float (&v)[4], int tile, int nt, int g, int t, bool have_old,
+                                               const uint32_t (&old_pair)[2], float (&best)[2], int (&bidx)[2]) {
 #pragma unroll
   for (int c = 0; c < 4; ++c) v[c] *= kOperandUnscale;
   if (p.epilogue == EPI_F32) {
@@ -214,7 +216,7 @@ __device__ __forceinline__ void slice_epilogue(const SliceParams& p, float (&v)[
       uint16_t* o = reinterpret_cast<uint16_t*>(p.out) + (size_t)req * p.out_stride + row;
       if (row + 1 < p.N && p.vec_ok) {
         if (p.epilogue == EPI_RESIDUAL) {
-          const uint32_t old = *reinterpret_cast<const uint32_t*>(o);
+          const uint32_t old = have_old ? old_pair[half] : *reinterpret_cast<const uint32_t*>(o);
           y = pack_bf16x2(bf16_lo(old) + bf16_lo(y), bf16_hi(old) + bf16_hi(y));
         }
         *reinterpret_cast<uint32_t*>(o) = y;
@@ -243,15 +245,15 @@ __global__ void __launch_bounds__(32 * slice_max_warps(NT), 1) q4_slice_kernel(c
   // the warp's number from lane 0: known to be uniform, so that the coordinates and addresses of its copies are
   // uniform registers (a TMA instruction takes nothing else; from vector registers each one cost a loop of ~15)
   const int warp = __shfl_sync(0xffffffffu, threadIdx.x >> 5, 0), lane = threadIdx.x & 31, g = lane >> 2, t = lane & 3;
-  const int warps = blockDim.x >> 5, rg = p.rg;
+  const int warps = blockDim.x >> 5, rg = p.rg, slots = p.slots;
   const int ksl = warp / rg, rgi = warp - ksl * rg;
   const bool silu = p.epilogue == EPI_SILU_PACK;
   const int half_n = p.N >> 1;
 
   unsigned char* smem = reinterpret_cast<unsigned char*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~(uintptr_t)1023);
-  unsigned char* ring = smem + warp * (kSliceSlots * kSliceCodes);
-  unsigned char* ring_sb = smem + warps * (kSliceSlots * kSliceCodes) + warp * (kSliceSlots * kSliceSb);
-  float4* sP = reinterpret_cast<float4*>(smem + warps * (kSliceSlots * (kSliceCodes + kSliceSb)));  // two buffers of [tile of the batch][kslice][NT][32]
+  unsigned char* ring = smem + warp * (slots * kSliceCodes);
+  unsigned char* ring_sb = smem + warps * (slots * kSliceCodes) + warp * (slots * kSliceSb);
+  float4* sP = reinterpret_cast<float4*>(smem + warps * (slots * (kSliceCodes + kSliceSb)));  // two buffers of [tile of the batch][kslice][NT][32]
 
   // this CTA's tiles and part of K; this warp's stages of K (SUB, or one less at the end) and tiles
   const int stages = p.K >> 8, m = (stages + SUB - 1) / SUB, parts = gridDim.y;
@@ -299,34 +301,50 @@ __global__ void __launch_bounds__(32 * slice_max_warps(NT), 1) q4_slice_kernel(c
   // Weights do not depend on the preceding kernel: fill the ring before waiting for it.
 #pragma unroll
   for (int i = 0; i < kSliceSlots; ++i) {
-    if (i < my_n) issue(t0 + i * rg + rgi, i);
+    if (i < my_n && i < slots) issue(t0 + i * rg + rgi, i);
     if (!SB_TMA) cp_async_commit();
   }
 
+  // Everything up to the first multiplication that does not need the operand is done before the preceding kernel is
+  // awaited: what comes after it is the step's critical path, a few hundred nanoseconds at a time.
+  bool ok = true;
+  auto wait = [&](uint32_t bar, uint32_t parity) {
+    if (!mbar_wait_addr(bar, parity)) {
+      ok = false;  // a copy or a warp that never came: report, results are void
+      if (p.status) atomicExch(p.status, 3u);
+    }
+  };
+  const uint32_t full_a = smem_u32(&s_full[0]), free_a = smem_u32(&s_free[0]);
+  const int buf_f4 = p.batch * rg * p.kw * (NT * 32);  // float4 of a buffer
+  // this lane's offsets in slot 0: codes of row g, its scales and its pair of biases
+  const uint32_t codes0 = (uint32_t)(ring - smem) + g * 128 + (((t >> 1) ^ g) << 4) + (t & 1) * 8;
+  const uint32_t sc0 = (uint32_t)(ring_sb - smem) + g * 16 + sb_half, bi0 = sc0 + 256 + (t & 1) * 4;
+  const int part_step = rg * p.kw * (NT * 32);
+  const int batches = (Tc + p.batch * rg - 1) / (p.batch * rg);
+  const uint4* op_src = reinterpret_cast<const uint4*>(p.xp) + (size_t)j * (SUB * 16 * 32) + lane;
   __syncthreads();  // the barriers of the partial tiles exist
+  if (my_n > 0) wait(bar_a, 0u);  // the first stage's codes
   grid_dependency_wait();
 
   // the operand of this warp's features, as B fragments, and the terms of its group sums
   uint4 bf[SUB][4][NT][2];
   uint2 x[SUB][NT];
+  // Only the fragments of requests that exist are read: with one request a warp's 4 KB are 512 bytes, and the time is the
+  // bytes' (148 CTAs x 16 warps).  The other columns' results are never stored.
 #pragma unroll
-  for (int sub = 0; sub < SUB; ++sub) {
-    if (my_n > 0 && (sub == 0 || both)) {
-      const int js = SUB * j + sub;
-      const uint4* src = reinterpret_cast<const uint4*>(p.xp) + (size_t)js * 16 * 32 + lane;
+  for (int sub = 0; sub < SUB; ++sub)
+#pragma unroll
+    for (int nt = 0; nt < NT; ++nt) {
+      const bool in = my_n > 0 && (sub == 0 || both) && nt * 8 + g < p.n;
 #pragma unroll
       for (int gi = 0; gi < 4; ++gi)
 #pragma unroll
-        for (int nt = 0; nt < NT; ++nt)
-#pragma unroll
-          for (int h = 0; h < 2; ++h) bf[sub][gi][nt][h] = __ldcg(src + ((gi * 2 + nt) * 2 + h) * 32);
-      if (p.xs) {
-#pragma unroll
-        for (int nt = 0; nt < NT; ++nt)
-          x[sub][nt] = __ldcg(reinterpret_cast<const uint2*>(p.xs + ((size_t)js * 16 + nt * 8 + g) * kOperandSumBytes + t * 8));
-      }
+        for (int h = 0; h < 2; ++h)
+          bf[sub][gi][nt][h] = in ? __ldcg(op_src + (sub * 16 + (gi * 2 + nt) * 2 + h) * 32) : make_uint4(0u, 0u, 0u, 0u);
+      x[sub][nt] = make_uint2(0u, 0u);
+      if (p.xs && in)
+        x[sub][nt] = __ldcg(reinterpret_cast<const uint2*>(p.xs + ((size_t)(SUB * j + sub) * 16 + nt * 8 + g) * kOperandSumBytes + t * 8));
     }
-  }
   if (!p.xs && my_n > 0) {
     // the producer left no group sums: the four lanes of a request hold a group's 64 elements
 #pragma unroll
@@ -347,36 +365,40 @@ __global__ void __launch_bounds__(32 * slice_max_warps(NT), 1) q4_slice_kernel(c
       }
   }
 
+  // the residual stream under the warp's first tile of the first batch, so that its epilogue waits for no load
+  uint32_t old_pair[2] = {0u, 0u};
+  if (p.epilogue == EPI_RESIDUAL && p.vec_ok && warp < min(p.batch * rg, Tc) * NT) {
+    const int req = (warp % NT) * 8 + g;
+#pragma unroll
+    for (int half = 0; half < 2; ++half) {
+      const int row = (t0 + warp / NT) * 16 + half * 8 + 2 * t;
+      if (req < p.n && row + 1 < p.N)
+        old_pair[half] = __ldcg(reinterpret_cast<const uint32_t*>(reinterpret_cast<const uint16_t*>(p.out) + (size_t)req * p.out_stride + row));
+    }
+  }
+
   float best[NT][2];
   int bidx[NT][2];
 #pragma unroll
   for (int nt = 0; nt < NT; ++nt) best[nt][0] = best[nt][1] = -INFINITY, bidx[nt][0] = bidx[nt][1] = 0x7fffffff;
 
-  bool ok = true;
-  auto wait = [&](uint32_t bar, uint32_t parity) {
-    if (!mbar_wait_addr(bar, parity)) {
-      ok = false;  // a copy or a warp that never came: report, results are void
-      if (p.status) atomicExch(p.status, 3u);
-    }
-  };
-  const uint32_t full_a = smem_u32(&s_full[0]), free_a = smem_u32(&s_free[0]);
-  const int buf_f4 = p.batch * rg * p.kw * (NT * 32);  // float4 of a buffer
-
   // The tiles of batch b, one warp per (tile, 8 requests), dealt round robin over the batches: the kslices' sums in
   // kslice order, then the epilogue.
+  int task = warp;  // of the coming batch, dealt round robin over the batches
   auto finish_batch = [&](int b) {
     const int first = b * p.batch * rg, tiles = min(p.batch * rg, Tc - first), buf = b & 1;
     wait(full_a + buf * 8, (uint32_t)((b >> 1) & 1));
     __syncwarp();
-    int task = (warp - (first * NT) % warps + warps) % warps;
-    for (; task < tiles * NT; task += warps) {
+    for (bool first_task = true; task < tiles * NT; task += warps, first_task = false) {
       const int tl = task / NT, nt = task - tl * NT, tile = t0 + first + tl;
       float v[4] = {0.0f, 0.0f, 0.0f, 0.0f};
       const float4* src = sP + buf * buf_f4 + tl * (p.kw * NT * 32) + nt * 32 + lane;
-#pragma unroll 8
-      for (int k = 0; k < nks; ++k) {
-        const float4 a = src[k * (NT * 32)];
-        v[0] += a.x, v[1] += a.y, v[2] += a.z, v[3] += a.w;
+      for (int k0 = 0; k0 < nks; k0 += 4) {  // four at a time: their loads go out together
+        float4 a[4];
+#pragma unroll
+        for (int k = 0; k < 4; ++k) a[k] = k0 + k < nks ? src[(k0 + k) * (NT * 32)] : make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+#pragma unroll
+        for (int k = 0; k < 4; ++k) v[0] += a[k].x, v[1] += a[k].y, v[2] += a[k].z, v[3] += a[k].w;
       }
       bool finish = true;
       if (parts > 1) {
@@ -407,20 +429,16 @@ __global__ void __launch_bounds__(32 * slice_max_warps(NT), 1) q4_slice_kernel(c
       if (finish) {
 #pragma unroll
         for (int q = 0; q < NT; ++q)
-          if (q == nt) slice_epilogue(p, v, tile, q, g, t, best[q], bidx[q]);
+          if (q == nt) slice_epilogue(p, v, tile, q, g, t, first_task && b == 0, old_pair, best[q], bidx[q]);
       }
     }
+    task -= tiles * NT;  // the next batch's first task of this warp
     __syncwarp();
     if (lane == 0) um_mbar_arrive(&s_free[buf]);
   };
 
-  int it = 0, slot = 0, next_tile = t0 + kSliceSlots * rg + rgi;
+  int it = 0, slot = 0, next_tile = t0 + slots * rg + rgi;
   uint32_t phase = 0;
-  // this lane's offsets in slot 0: codes of row g, its scales and its pair of biases
-  const uint32_t codes0 = (uint32_t)(ring - smem) + g * 128 + (((t >> 1) ^ g) << 4) + (t & 1) * 8;
-  const uint32_t sc0 = (uint32_t)(ring_sb - smem) + g * 16 + sb_half, bi0 = sc0 + 256 + (t & 1) * 4;
-  const int part_step = rg * p.kw * (NT * 32);
-  const int batches = (Tc + p.batch * rg - 1) / (p.batch * rg);
   for (int b = 0; b < batches; ++b) {
     const int buf = b & 1;
     if (b >= 2) wait(free_a + buf * 8, (uint32_t)(((b >> 1) - 1) & 1));
@@ -428,7 +446,7 @@ __global__ void __launch_bounds__(32 * slice_max_warps(NT), 1) q4_slice_kernel(c
     const int it_end = min(my_n, (b + 1) * p.batch);
     for (; it < it_end; ++it, dst += part_step) {
       if (!SB_TMA) cp_async_wait<kSliceSlots - 1>();
-      wait(bar_a + slot * 8, phase);
+      if (it > 0) wait(bar_a + slot * 8, phase);
       __syncwarp();
       float acc[NT][4];
 #pragma unroll
@@ -446,12 +464,12 @@ __global__ void __launch_bounds__(32 * slice_max_warps(NT), 1) q4_slice_kernel(c
 #pragma unroll
       for (int nt = 0; nt < NT; ++nt) dst[nt * 32] = make_float4(acc[nt][0], acc[nt][1], acc[nt][2], acc[nt][3]);
       __syncwarp();
-      if (it + kSliceSlots < my_n) {  // refill the slot just multiplied
+      if (it + slots < my_n) {  // refill the slot just multiplied
         if (ok) issue(next_tile, slot);
         next_tile += rg;
       }
       if (!SB_TMA) cp_async_commit();
-      if (++slot == kSliceSlots) slot = 0, phase ^= 1u;
+      if (++slot == slots) slot = 0, phase ^= 1u;
     }
     __syncwarp();
     if (lane == 0) um_mbar_arrive(&s_full[buf]);
@@ -480,7 +498,7 @@ __global__ void __launch_bounds__(32 * slice_max_warps(NT), 1) q4_slice_kernel(c
 }
 
 struct SlicePlan {
-  int nt, parts, kw, rg, T, ctas, batch;
+  int nt, parts, kw, rg, T, ctas, batch, slots;
   size_t smem, partial_bytes;
 };
 
@@ -495,10 +513,18 @@ SlicePlan plan_slices(int N, int K, int n, int epilogue, int sm_count) {
   if (ctas < 1) ctas = 1;
   t.ctas = t.T < ctas ? t.T : ctas;
   const int per_cta = (t.T + t.ctas - 1) / t.ctas;
+  // A small projection runs on half the warps: then the next kernel's CTAs fit on the SMs beside it (the register file is
+  // what they share) and have their first codes by the time they are released, which is worth more than a shorter
+  // multiplication (1024 -> 6144 at one request, launch to launch: 4.31 us with 12 warps, which leave the next CTA no
+  // room, so that its codes arrive 1.8 us after the release; 3.67 with 8).  It is not worth a third stage per warp, nor a
+  // second one with 16 requests, where a stage takes twice as long (2048 -> 5120, 1024 -> 6144: slower).
   t.rg = max_warps / t.kw;
+  const int half = max_warps / 2 / t.kw;
+  if (half >= 1 && (per_cta + half - 1) / half <= (t.nt == 1 ? 2 : 1)) t.rg = half;
   if (t.rg > per_cta) t.rg = per_cta;
   const int warps = t.kw * t.rg, rounds = (per_cta + t.rg - 1) / t.rg;
-  const size_t fixed = 1024 + (size_t)warps * kSliceSlots * (slice_slot_codes(t.nt) + kSliceSb);
+  t.slots = rounds < kSliceSlots ? rounds : kSliceSlots;
+  const size_t fixed = 1024 + (size_t)warps * t.slots * (slice_slot_codes(t.nt) + kSliceSb);
   const size_t per_round = 2 * (size_t)warps * t.nt * 512;  // two buffers
   const int most = (int)((220 * 1024 - fixed) / per_round);  // rounds whose partial tiles fit
   const int batches = (rounds + most - 1) / most;
@@ -612,12 +638,14 @@ __global__ void __launch_bounds__(32 * slice_max_warps(1), 1) q4_expert_kernel(c
     if (GATE_UP) r = ((g < 4 ? u.z : u.w) >> ((g & 3) * 8)) & 15;
     else base += (size_t)unit * p.unit_stride;
     const uint4* src = reinterpret_cast<const uint4*>(base) + (size_t)j * 16 * 32 + (r >> 3) * 64 + (r & 7) * 4 + t;
+    const bool in = g < u.y;  // only the unit's requests are read
 #pragma unroll
     for (int gi = 0; gi < 4; ++gi)
 #pragma unroll
-      for (int h = 0; h < 2; ++h) bf[gi][0][h] = __ldcg(src + (gi * 4 + h) * 32);
+      for (int h = 0; h < 2; ++h) bf[gi][0][h] = in ? __ldcg(src + (gi * 4 + h) * 32) : make_uint4(0u, 0u, 0u, 0u);
     if (GATE_UP) {
-      x[0] = __ldcg(reinterpret_cast<const uint2*>(p.xs + ((size_t)j * 16 + r) * kOperandSumBytes + t * 8));
+      x[0] = make_uint2(0u, 0u);
+      if (in) x[0] = __ldcg(reinterpret_cast<const uint2*>(p.xs + ((size_t)j * 16 + r) * kOperandSumBytes + t * 8));
     } else {
       float v[4];
 #pragma unroll
@@ -641,19 +669,22 @@ __global__ void __launch_bounds__(32 * slice_max_warps(1), 1) q4_expert_kernel(c
   const uint32_t full_a = smem_u32(&s_full[0]), free_a = smem_u32(&s_free[0]);
   const int buf_f4 = p.batch * rg * p.kw * 32;  // float4 of a buffer
 
+  int task = warp;  // of the coming batch, dealt round robin over the batches
   auto finish_batch = [&](int b) {
     const int first = b * p.batch * rg, tiles = min(p.batch * rg, Tc - first), buf = b & 1;
     wait(full_a + buf * 8, (uint32_t)((b >> 1) & 1));
     __syncwarp();
-    for (int tl = (warp - first % warps + warps) % warps; tl < tiles; tl += warps) {
-      const int gt = t0 + first + tl, unit = gt / p.tiles, tile = gt - unit * p.tiles;
+    for (; task < tiles; task += warps) {
+      const int gt = t0 + first + task, unit = gt / p.tiles, tile = gt - unit * p.tiles;
       const int count = s_units[unit].y;
       float v[4] = {0.0f, 0.0f, 0.0f, 0.0f};
-      const float4* src = sP + buf * buf_f4 + tl * (p.kw * 32) + lane;
-#pragma unroll 8
-      for (int k = 0; k < p.kw; ++k) {
-        const float4 a = src[k * 32];
-        v[0] += a.x, v[1] += a.y, v[2] += a.z, v[3] += a.w;
+      const float4* src = sP + buf * buf_f4 + task * (p.kw * 32) + lane;
+      for (int k0 = 0; k0 < p.kw; k0 += 4) {  // four at a time: their loads go out together
+        float4 a[4];
+#pragma unroll
+        for (int k = 0; k < 4; ++k) a[k] = k0 + k < p.kw ? src[(k0 + k) * 32] : make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+#pragma unroll
+        for (int k = 0; k < 4; ++k) v[0] += a[k].x, v[1] += a[k].y, v[2] += a[k].z, v[3] += a[k].w;
       }
 #pragma unroll
       for (int c = 0; c < 4; ++c) v[c] *= kOperandUnscale;
@@ -668,6 +699,7 @@ __global__ void __launch_bounds__(32 * slice_max_warps(1), 1) q4_expert_kernel(c
         }
       }
     }
+    task -= tiles;
     __syncwarp();
     if (lane == 0) um_mbar_arrive(&s_free[buf]);
   };
@@ -857,7 +889,7 @@ cudaError_t launch_q4_gemm(const GemmArgs& a, cudaStream_t s) {
   p.scales = a.scales, p.biases = a.biases, p.xp = a.xp, p.xs = static_cast<const unsigned char*>(a.xs), p.out = a.out;
   p.out_xp = a.out_xp, p.argmax_partial = a.argmax_partial, p.status = a.status;
   p.N = a.N, p.K = a.K, p.n = a.n, p.out_stride = a.out_stride, p.epilogue = a.epilogue;
-  p.T = t.T, p.kw = t.kw, p.rg = t.rg, p.batch = t.batch;
+  p.T = t.T, p.kw = t.kw, p.rg = t.rg, p.batch = t.batch, p.slots = t.slots;
   p.partial = a.partial, p.counters = a.counters;
   if (t.parts > 1 && (!a.partial || !a.counters || t.partial_bytes > a.partial_bytes || t.T > a.counters_len))
     return cudaErrorInvalidValue;
