@@ -43,15 +43,32 @@ __device__ __forceinline__ void mma_free_first(float (&d)[4], uint32_t a0, uint3
       : "r"(a0), "r"(a1), "r"(a2), "r"(a3), "r"(b0), "r"(b1), "f"(0.0f));
 }
 
-// acc += 16 rows x 256 features with the operand's fragments in registers.  codes: offset in smem of this lane's first 8
+// shared-memory accesses by 32-bit address (a generic pointer costs 64-bit arithmetic on the busiest pipe here)
+__device__ __forceinline__ uint32_t lds32(uint32_t a) {
+  uint32_t v;
+  asm volatile("ld.shared.u32 %0, [%1];" : "=r"(v) : "r"(a));
+  return v;
+}
+__device__ __forceinline__ uint2 lds64(uint32_t a) {
+  uint2 v;
+  asm volatile("ld.shared.v2.u32 {%0, %1}, [%2];" : "=r"(v.x), "=r"(v.y) : "r"(a));
+  return v;
+}
+__device__ __forceinline__ uint4 lds128(uint32_t a) {
+  uint4 v;
+  asm volatile("ld.shared.v4.u32 {%0, %1, %2, %3}, [%4];" : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w) : "r"(a));
+  return v;
+}
+
+// acc += 16 rows x 256 features with the operand's fragments in registers.  codes: shared address of this lane's first 8
 // bytes of the stage's row g (a group further is an XOR with 32 in the swizzled, 1024-byte-aligned stage; row g + 8 is 1024
-// bytes on).  bi: offset of this lane's pair of biases (8 rows are 128 bytes); sc_lo, sc_hi: the 4 scales of rows g, g + 8.
+// bytes on).  bi: address of this lane's pair of biases (8 rows are 128 bytes); sc_lo, sc_hi: the 4 scales of rows g, g + 8.
 // The pipe that shifts and masks issues every other cycle and is the busiest one here, so nothing but the unpacking is
 // left to it: scalar FMAs instead of packed ones (whose operand pairs cost moves), no address arithmetic.
 template <int NT>
-__device__ __forceinline__ void multiply_regs(const unsigned char* smem, uint32_t codes, uint32_t bi, const uint2 sc_lo, const uint2 sc_hi,
+__device__ __forceinline__ void multiply_regs(uint32_t codes, uint32_t bi, const uint2 sc_lo, const uint2 sc_hi,
                                               const uint4 (&bf)[4][NT][2], const uint2 (&x)[NT], float (&acc)[NT][4]) {
-  const uint32_t b_lo = *reinterpret_cast<const uint32_t*>(smem + bi), b_hi = *reinterpret_cast<const uint32_t*>(smem + bi + 128);
+  const uint32_t b_lo = lds32(bi), b_hi = lds32(bi + 128);
 #pragma unroll
   for (int nt = 0; nt < NT; ++nt) mma_free(acc[nt], b_lo, b_hi, b_lo, b_hi, x[nt].x, x[nt].y);
   // The four MMAs of a group and 8 requests are a chain; four chains side by side hide the pipe's latency.
@@ -62,8 +79,8 @@ __device__ __forceinline__ void multiply_regs(const unsigned char* smem, uint32_
     float pc[GP][NT][4];
 #pragma unroll
     for (int i = 0; i < GP; ++i) {
-      const unsigned char* at = smem + (codes ^ (uint32_t)((g0 + i) << 5));
-      wl[i] = *reinterpret_cast<const uint2*>(at), wh[i] = *reinterpret_cast<const uint2*>(at + 1024);
+      const uint32_t at = codes ^ (uint32_t)((g0 + i) << 5);
+      wl[i] = lds64(at), wh[i] = lds64(at + 1024);
     }
 #pragma unroll
     for (int step = 0; step < 4; ++step) {
@@ -316,9 +333,9 @@ __global__ void __launch_bounds__(32 * slice_max_warps(NT), 1) q4_slice_kernel(c
   };
   const uint32_t full_a = smem_u32(&s_full[0]), free_a = smem_u32(&s_free[0]);
   const int buf_f4 = p.batch * rg * p.kw * (NT * 32);  // float4 of a buffer
-  // this lane's offsets in slot 0: codes of row g, its scales and its pair of biases
-  const uint32_t codes0 = (uint32_t)(ring - smem) + g * 128 + (((t >> 1) ^ g) << 4) + (t & 1) * 8;
-  const uint32_t sc0 = (uint32_t)(ring_sb - smem) + g * 16 + sb_half, bi0 = sc0 + 256 + (t & 1) * 4;
+  // this lane's addresses in slot 0: codes of row g, its scales and its pair of biases
+  const uint32_t codes0 = ring_a + g * 128 + (((t >> 1) ^ g) << 4) + (t & 1) * 8;
+  const uint32_t sc0 = sb_a + g * 16 + sb_half, bi0 = sc0 + 256 + (t & 1) * 4;
   const int part_step = rg * p.kw * (NT * 32);
   const int batches = (Tc + p.batch * rg - 1) / (p.batch * rg);
   const uint4* op_src = reinterpret_cast<const uint4*>(p.xp) + (size_t)j * (SUB * 16 * 32) + lane;
@@ -452,14 +469,14 @@ __global__ void __launch_bounds__(32 * slice_max_warps(NT), 1) q4_slice_kernel(c
 #pragma unroll
       for (int nt = 0; nt < NT; ++nt) acc[nt][0] = acc[nt][1] = acc[nt][2] = acc[nt][3] = 0.0f;
       const uint32_t codes = codes0 + slot * kSliceCodes, bi = bi0 + slot * kSliceSb;
-      const unsigned char* sc = smem + sc0 + slot * kSliceSb;
+      const uint32_t sc = sc0 + slot * kSliceSb;
       if (SUB == 1) {
-        multiply_regs<NT>(smem, codes, bi, *reinterpret_cast<const uint2*>(sc), *reinterpret_cast<const uint2*>(sc + 128), bf[0], x[0], acc);
+        multiply_regs<NT>(codes, bi, lds64(sc), lds64(sc + 128), bf[0], x[0], acc);
       } else {
-        const uint4 sc_lo = *reinterpret_cast<const uint4*>(sc), sc_hi = *reinterpret_cast<const uint4*>(sc + 128);
-        multiply_regs<NT>(smem, codes, bi, make_uint2(sc_lo.x, sc_lo.y), make_uint2(sc_hi.x, sc_hi.y), bf[0], x[0], acc);
+        const uint4 sc_lo = lds128(sc), sc_hi = lds128(sc + 128);
+        multiply_regs<NT>(codes, bi, make_uint2(sc_lo.x, sc_lo.y), make_uint2(sc_hi.x, sc_hi.y), bf[0], x[0], acc);
         if (both)
-          multiply_regs<NT>(smem, codes + 2048, bi + 8, make_uint2(sc_lo.z, sc_lo.w), make_uint2(sc_hi.z, sc_hi.w), bf[SUB - 1], x[SUB - 1], acc);
+          multiply_regs<NT>(codes + 2048, bi + 8, make_uint2(sc_lo.z, sc_lo.w), make_uint2(sc_hi.z, sc_hi.w), bf[SUB - 1], x[SUB - 1], acc);
       }
 #pragma unroll
       for (int nt = 0; nt < NT; ++nt) dst[nt * 32] = make_float4(acc[nt][0], acc[nt][1], acc[nt][2], acc[nt][3]);
@@ -706,8 +723,8 @@ __global__ void __launch_bounds__(32 * slice_max_warps(1), 1) q4_expert_kernel(c
 
   int it = 0, slot = 0, gt = t0 + rgi, unit = -1, unit_end = 0;
   uint32_t phase = 0;
-  const uint32_t codes0 = (uint32_t)(ring - smem) + g * 128 + (((t >> 1) ^ g) << 4) + (t & 1) * 8;
-  const uint32_t sc0 = (uint32_t)(ring_sb - smem) + g * 16 + sb_half, bi0 = sc0 + 256 + (t & 1) * 4;
+  const uint32_t codes0 = ring_a + g * 128 + (((t >> 1) ^ g) << 4) + (t & 1) * 8;
+  const uint32_t sc0 = sb_a + g * 16 + sb_half, bi0 = sc0 + 256 + (t & 1) * 4;
   const int part_step = rg * p.kw * 32;
   const int batches = (Tc + p.batch * rg - 1) / (p.batch * rg);
   for (int b = 0; b < batches; ++b) {
@@ -724,9 +741,9 @@ __global__ void __launch_bounds__(32 * slice_max_warps(1), 1) q4_expert_kernel(c
       wait(bar_a + slot * 8, phase);
       __syncwarp();
       float acc[1][4] = {{0.0f, 0.0f, 0.0f, 0.0f}};
-      const unsigned char* sc = smem + sc0 + slot * kSliceSb;
-      multiply_regs<1>(smem, codes0 + slot * kCodes, bi0 + slot * kSliceSb, *reinterpret_cast<const uint2*>(sc),
-                       *reinterpret_cast<const uint2*>(sc + 128), bf, x, acc);
+      const uint32_t sc = sc0 + slot * kSliceSb;
+      multiply_regs<1>(codes0 + slot * kCodes, bi0 + slot * kSliceSb, lds64(sc),
+                       lds64(sc + 128), bf, x, acc);
       dst[0] = make_float4(acc[0][0], acc[0][1], acc[0][2], acc[0][3]);
       __syncwarp();
       if (ok && it + kSliceSlots < my_n) issue(gt + kSliceSlots * rg, slot);  // refill the slot just multiplied
