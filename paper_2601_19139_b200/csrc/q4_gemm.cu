@@ -314,6 +314,9 @@ __global__ void __launch_bounds__(32 * slice_max_warps(NT), 1) q4_slice_kernel(c
     }
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
+  if (!SB_TMA && SUB == 2 && !both) {  // the scales and biases of a stage that does not exist are zeros too
+    for (int i = lane; i < slots * 32; i += 32) *reinterpret_cast<uint2*>(ring_sb + i * 16 + 8) = make_uint2(0u, 0u);
+  }
   __syncwarp();
   // Weights do not depend on the preceding kernel: fill the ring before waiting for it.
 #pragma unroll
@@ -475,7 +478,7 @@ __global__ void __launch_bounds__(32 * slice_max_warps(NT), 1) q4_slice_kernel(c
       } else {
         const uint4 sc_lo = lds128(sc), sc_hi = lds128(sc + 128);
         multiply_regs<NT>(codes, bi, make_uint2(sc_lo.x, sc_lo.y), make_uint2(sc_hi.x, sc_hi.y), bf[0], x[0], acc);
-        if (both)
+        // a slice without its second stage multiplies it with an operand of zeros: no branch between the halves
           multiply_regs<NT>(codes + 2048, bi + 8, make_uint2(sc_lo.z, sc_lo.w), make_uint2(sc_hi.z, sc_hi.w), bf[SUB - 1], x[SUB - 1], acc);
       }
 #pragma unroll
