@@ -30,49 +30,82 @@ constexpr int kTileBytes = 16 * 128 * 2;    // one block of one kv head: 16 toke
 constexpr int kAttnStage = 2 * kTileBytes;  // K then V
 constexpr float kScaleLog2 = 0.08838834764831845f * 1.4426950408889634f;  // log2(e) / sqrt(128)
 
-// out[r][a] = bf16(sum_c 2^(m_c - M) acc_c / sum_c 2^(m_c - M) l_c) over the request's chunks, in chunk order.
-// One call handles 8 consecutive elements (index ch of 16) of head a; the 8 lanes of an aligned lane group must hold
-// the 8 chunks of one 64-element group and all call together (group sums).  Writes the plain layout and/or the
-// fragment-ordered operand of the O projection (K = nq * 128) with its group sums.
-__device__ __forceinline__ void merge_head_chunk(const AttnArgs& p, int r, int a, int ch, bool valid) {
-  const int s0 = p.slot_base[r], nc = p.nchunks[r];
-  float acc[8] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
-  float den = 0.0f;
-  if (valid) {
-    float M = -INFINITY;
-    // the merge runs in the last CTA of a request, after everything else: its loads go out in batches (16 maxima,
-    // then 8 chunks' partial results at a time) so that a request of a dozen chunks costs two round trips, not four
-#pragma unroll 16
-    for (int c = 0; c < nc; ++c) M = fmaxf(M, __ldcg(p.part_ml + ((size_t)(s0 + c) * p.nq + a) * 2));
-#pragma unroll 8
-    for (int c = 0; c < nc; ++c) {
-      const size_t qh = (size_t)(s0 + c) * p.nq + a;
-      const float2 ml = __ldcg(reinterpret_cast<const float2*>(p.part_ml + qh * 2));
-      const float4 u = __ldcg(reinterpret_cast<const float4*>(p.part_acc + qh * kHeadDim + ch * 8));
-      const float4 v = __ldcg(reinterpret_cast<const float4*>(p.part_acc + qh * kHeadDim + ch * 8 + 4));
-      const float e = exp2f(ml.x - M);
-      acc[0] = fmaf(e, u.x, acc[0]), acc[1] = fmaf(e, u.y, acc[1]), acc[2] = fmaf(e, u.z, acc[2]);
-      acc[3] = fmaf(e, u.w, acc[3]), acc[4] = fmaf(e, v.x, acc[4]), acc[5] = fmaf(e, v.y, acc[5]);
-      acc[6] = fmaf(e, v.z, acc[6]), acc[7] = fmaf(e, v.w, acc[7]);
-      den = fmaf(e, ml.y, den);
+// out[r][a] = bf16(sum_c 2^(m_c - M) acc_c / sum_c 2^(m_c - M) l_c) over the request's nc chunks from slot s0, by a warp:
+// four elements of head a per lane.  Writes the plain layout and/or the operand of the O projection (K = nq * 128) with
+// its group sums.
+// This runs once per request and kv head, in the CTA that ends last, with everything behind it waiting: what it costs is
+// round trips to L2 and the fetching of its instructions, which no other CTA of the SM has just run.  So the chunks'
+// maxima and weights are a lane each, the partial results come eight at a time, ahead of their use, and the code is a page
+// (16 threads a head with the loops over chunks unrolled: 4 us for five chunks, 7 us for sixteen).
+__device__ __forceinline__ void merge_head(const AttnArgs& p, int r, int s0, int nc, int a) {
+  const int lane = threadIdx.x & 31;
+  const size_t stride = (size_t)p.nq * kHeadDim;  // floats from a chunk's result to the next one's
+  const float* src = p.part_acc + (size_t)s0 * stride + (size_t)a * kHeadDim + 4 * lane;
+  const float* ml = p.part_ml + ((size_t)s0 * p.nq + a) * 2;
+  float4 v[8];
+  auto load = [&](int c0) {
+#pragma unroll
+    for (int c = 0; c < 8; ++c) {
+      v[c] = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+      if (c0 + c < nc) v[c] = __ldcg(reinterpret_cast<const float4*>(src + (size_t)(c0 + c) * stride));
     }
-  } else {
-    den = 1.0f;
+  };
+  load(0);
+  float M = -INFINITY, den = 0.0f, e = 0.0f, acc[4] = {0.0f, 0.0f, 0.0f, 0.0f};
+#pragma unroll 1
+  for (int c0 = 0; c0 < nc; c0 += 8) {
+    if ((c0 & 31) == 0) {  // the next 32 chunks' weights; what there is already is rescaled
+      float2 mine = make_float2(-INFINITY, 0.0f);
+      if (c0 + lane < nc) mine = __ldcg(reinterpret_cast<const float2*>(ml + (size_t)(c0 + lane) * p.nq * 2));
+      float Mn = fmaxf(M, mine.x);
+#pragma unroll
+      for (int o = 16; o > 0; o >>= 1) Mn = fmaxf(Mn, __shfl_xor_sync(0xffffffffu, Mn, o));
+      e = exp2f(mine.x - Mn);
+      const float scale = exp2f(M - Mn);
+      den = fmaf(den, scale, warp_sum(e * mine.y)), M = Mn;
+#pragma unroll
+      for (int i = 0; i < 4; ++i) acc[i] *= scale;
+    }
+#pragma unroll
+    for (int c = 0; c < 8; ++c) {
+      const float w = __shfl_sync(0xffffffffu, e, (c0 + c) & 31);
+      acc[0] = fmaf(w, v[c].x, acc[0]), acc[1] = fmaf(w, v[c].y, acc[1]), acc[2] = fmaf(w, v[c].z, acc[2]), acc[3] = fmaf(w, v[c].w, acc[3]);
+    }
+    load(c0 + 8);
   }
-  uint4 o;
-  o.x = pack_bf16x2(acc[0] / den, acc[1] / den);
-  o.y = pack_bf16x2(acc[2] / den, acc[3] / den);
-  o.z = pack_bf16x2(acc[4] / den, acc[5] / den);
-  o.w = pack_bf16x2(acc[6] / den, acc[7] / den);
-  const float gsum = group_sum_8lanes(chunk_sum(o));  // 8 lanes = 64 elements = one group of the O projection's K
-  if (!valid) return;
-  const size_t col = (size_t)a * kHeadDim + ch * 8;
-  const size_t K = (size_t)p.nq * kHeadDim;
-  if (p.out) *reinterpret_cast<uint4*>(p.out + (size_t)r * K + col) = o;
+  const uint2 o = make_uint2(pack_bf16x2(acc[0] / den, acc[1] / den), pack_bf16x2(acc[2] / den, acc[3] / den));
+  const int col = a * kHeadDim + 4 * lane, K = p.nq * kHeadDim;
+  if (p.out) *reinterpret_cast<uint2*>(p.out + (size_t)r * K + col) = o;
   if (p.out_xp) {
-    store_operand_chunk(p.out_layout, p.out_xp, (int)K, r, (int)(col >> 3), o);
-    if ((ch & 7) == 0) store_operand_sum(p.out_layout, p.out_xs, r, (int)(col >> 6), gsum);
+    float gsum = (bf16_lo(o.x) + bf16_hi(o.x)) + (bf16_lo(o.y) + bf16_hi(o.y));  // pairs, chunks of 8, the 8 chunks
+#pragma unroll
+    for (int sh = 1; sh <= 8; sh <<= 1) gsum += __shfl_xor_sync(0xffffffffu, gsum, sh);
+    const uint2 other = make_uint2(__shfl_xor_sync(0xffffffffu, o.x, 1), __shfl_xor_sync(0xffffffffu, o.y, 1));
+    if ((lane & 1) == 0) store_operand_chunk(p.out_layout, p.out_xp, K, r, col >> 3, make_uint4(o.x, o.y, other.x, other.y));
+    if ((lane & 15) == 0) store_operand_sum(p.out_layout, p.out_xs, r, col >> 6, gsum);
   }
+}
+
+// The CTA that finishes the last chunk of a (request, kv head) merges all of them.  nc, s0: the request's chunks and the
+// first one's slot.
+__device__ __forceinline__ void merge_if_last(const AttnArgs& p, int r, int h, int G, int nc, int s0) {
+  __shared__ int s_last;
+  if (nc > 1) {
+    __threadfence();
+    __syncthreads();
+    if (threadIdx.x == 0) {
+      const int prev = atomicAdd(p.merge_counters + r * p.nkv + h, 1);
+      s_last = prev == nc - 1;
+      if (s_last) p.merge_counters[r * p.nkv + h] = 0;
+      __threadfence();
+    }
+    __syncthreads();
+    if (!s_last) return;
+  } else {
+    __syncthreads();
+  }
+#pragma unroll 1
+  for (int a = threadIdx.x >> 5; a < G; a += kAttnWarps) merge_head(p, r, s0, nc, h * G + a);
 }
 
 __global__ void __launch_bounds__(kAttnThreads) paged_attention_kernel(const AttnArgs p) {
@@ -353,25 +386,7 @@ __global__ void __launch_bounds__(kAttnThreads) paged_attention_kernel(const Att
         }
       }
     }
-    if (p.merge_counters) {
-      // the CTA that finishes the last chunk of this (request, kv head) merges all of them in chunk order
-      __shared__ int s_last;
-      __threadfence();
-      __syncthreads();
-      if (threadIdx.x == 0) {
-        const int prev = atomicAdd(p.merge_counters + r * p.nkv + h, 1);
-        s_last = prev == p.nchunks[r] - 1;
-        if (s_last) p.merge_counters[r * p.nkv + h] = 0;
-      }
-      __syncthreads();
-      if (s_last) {
-        __threadfence();
-        for (int a0 = 0; a0 < G; a0 += 8) {  // 16 threads per head, 8 heads per pass
-          const int a = a0 + (threadIdx.x >> 4);
-          merge_head_chunk(p, r, h * G + a, threadIdx.x & 15, a < G);
-        }
-      }
-    }
+    if (p.merge_counters) merge_if_last(p, r, h, G, p.nchunks[r], p.slot_base[r]);
     __syncthreads();
   }
 }
@@ -450,11 +465,29 @@ __global__ void __launch_bounds__(kAttnThreads) paged_attention_t_kernel(const A
       }
     }
 
+    // the new token's place, and what its k takes besides itself
+    const int last_tile = pos >> 4, new_blk = bt[last_tile];
+    const bool appends = prep && last_tile >= first && last_tile < tile_end && ((last_tile - first) % kAttnWarps) == 0;
+    uint32_t kn_a = 0u, kn_b = 0u;  // elements 2*lane, 2*lane+1 and 64+2*lane, 64+2*lane+1, as below
+    float4 k_cs = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+    if (appends) {
+      k_cs = __ldg(reinterpret_cast<const float4*>(p.rope + ((size_t)pos * 64 + 2 * lane) * 2));
+      if (p.k_norm) kn_a = __ldg(reinterpret_cast<const uint32_t*>(p.k_norm + 2 * lane)), kn_b = __ldg(reinterpret_cast<const uint32_t*>(p.k_norm + 64 + 2 * lane));
+    }
+    const int nc = p.merge_counters ? p.nchunks[r] : 0, s0 = p.merge_counters ? p.slot_base[r] : 0;
+
     if (!waited) {
       grid_dependency_wait();
       waited = true;
     }
 
+    uint32_t nw_a = 0u, nw_b = 0u, nv_a = 0u, nv_b = 0u;  // requested together with q: one round trip
+    if (appends) {
+      const uint16_t* ksrc = p.qkv + ((size_t)r * (p.nq + 2 * p.nkv) + p.nq + h) * kHeadDim;
+      const uint16_t* vsrc = ksrc + (size_t)p.nkv * kHeadDim;
+      nw_a = *reinterpret_cast<const uint32_t*>(ksrc + 2 * lane), nw_b = *reinterpret_cast<const uint32_t*>(ksrc + 64 + 2 * lane);
+      nv_a = *reinterpret_cast<const uint32_t*>(vsrc + 2 * lane), nv_b = *reinterpret_cast<const uint32_t*>(vsrc + 64 + 2 * lane);
+    }
     // q of head g of this kv head (zero beyond G): dims 16ks + 2t, +1 and 16ks + 2t + 8, +9 -- the B fragments
     uint32_t qb[8][2];
     {
@@ -498,32 +531,20 @@ __global__ void __launch_bounds__(kAttnThreads) paged_attention_t_kernel(const A
     }
     // k, v of the new token: prepared and appended by the warp that walks the request's last tile, which later puts
     // them into its staged copy of that tile (fetched before they existed)
-    const int last_tile = pos >> 4;
-    const bool appends = prep && last_tile >= first && last_tile < tile_end && ((last_tile - first) % kAttnWarps) == 0;
-    uint32_t nk_a = 0u, nk_b = 0u, nv_a = 0u, nv_b = 0u;  // elements 2*lane, 2*lane+1 and 64+2*lane, 64+2*lane+1
+    uint32_t nk_a = 0u, nk_b = 0u;
     if (appends) {
-      const int heads = p.nq + 2 * p.nkv;
-      const uint16_t* ksrc = p.qkv + ((size_t)r * heads + p.nq + h) * kHeadDim;
-      const uint16_t* vsrc = ksrc + (size_t)p.nkv * kHeadDim;
-      const uint32_t wa = *reinterpret_cast<const uint32_t*>(ksrc + 2 * lane);
-      const uint32_t wb = *reinterpret_cast<const uint32_t*>(ksrc + 64 + 2 * lane);
-      nv_a = *reinterpret_cast<const uint32_t*>(vsrc + 2 * lane);
-      nv_b = *reinterpret_cast<const uint32_t*>(vsrc + 64 + 2 * lane);
-      float a0 = bf16_lo(wa), a1 = bf16_hi(wa), b0 = bf16_lo(wb), b1 = bf16_hi(wb);
+      float a0 = bf16_lo(nw_a), a1 = bf16_hi(nw_a), b0 = bf16_lo(nw_b), b1 = bf16_hi(nw_b);
       if (p.k_norm) {
         const float ss = warp_sum(a0 * a0 + a1 * a1 + b0 * b0 + b1 * b1);
         const float inv = 1.0f / sqrtf(ss * (1.0f / kHeadDim) + p.eps);
-        const uint32_t na = *reinterpret_cast<const uint32_t*>(p.k_norm + 2 * lane);
-        const uint32_t nb = *reinterpret_cast<const uint32_t*>(p.k_norm + 64 + 2 * lane);
-        a0 = bf16_to_f32(f32_to_bf16(a0 * inv * bf16_lo(na)));
-        a1 = bf16_to_f32(f32_to_bf16(a1 * inv * bf16_hi(na)));
-        b0 = bf16_to_f32(f32_to_bf16(b0 * inv * bf16_lo(nb)));
-        b1 = bf16_to_f32(f32_to_bf16(b1 * inv * bf16_hi(nb)));
+        a0 = bf16_to_f32(f32_to_bf16(a0 * inv * bf16_lo(kn_a)));
+        a1 = bf16_to_f32(f32_to_bf16(a1 * inv * bf16_hi(kn_a)));
+        b0 = bf16_to_f32(f32_to_bf16(b0 * inv * bf16_lo(kn_b)));
+        b1 = bf16_to_f32(f32_to_bf16(b1 * inv * bf16_hi(kn_b)));
       }
-      const float4 cs = *reinterpret_cast<const float4*>(p.rope + ((size_t)pos * 64 + 2 * lane) * 2);
-      nk_a = pack_bf16x2(a0 * cs.x - b0 * cs.y, a1 * cs.z - b1 * cs.w);
-      nk_b = pack_bf16x2(b0 * cs.x + a0 * cs.y, b1 * cs.z + a1 * cs.w);
-      const size_t dst = (((size_t)bt[last_tile] * p.nkv + h) * kBlockSize + (pos & 15)) * kHeadDim;
+      nk_a = pack_bf16x2(a0 * k_cs.x - b0 * k_cs.y, a1 * k_cs.z - b1 * k_cs.w);
+      nk_b = pack_bf16x2(b0 * k_cs.x + a0 * k_cs.y, b1 * k_cs.z + a1 * k_cs.w);
+      const size_t dst = (((size_t)new_blk * p.nkv + h) * kBlockSize + (pos & 15)) * kHeadDim;
       *reinterpret_cast<uint32_t*>(p.kpool_w + dst + 2 * lane) = nk_a;
       *reinterpret_cast<uint32_t*>(p.kpool_w + dst + 64 + 2 * lane) = nk_b;
       *reinterpret_cast<uint32_t*>(p.vpool_w + dst + 2 * lane) = nv_a;
@@ -669,32 +690,17 @@ __global__ void __launch_bounds__(kAttnThreads) paged_attention_t_kernel(const A
         }
       }
     }
-    if (p.merge_counters) {
-      // the CTA that finishes the last chunk of this (request, kv head) merges all of them in chunk order
-      __shared__ int s_last;
-      __threadfence();
-      __syncthreads();
-      if (threadIdx.x == 0) {
-        const int prev = atomicAdd(p.merge_counters + r * p.nkv + h, 1);
-        s_last = prev == p.nchunks[r] - 1;
-        if (s_last) p.merge_counters[r * p.nkv + h] = 0;
-      }
-      __syncthreads();
-      if (s_last) {
-        __threadfence();
-        merge_head_chunk(p, r, h * G + (threadIdx.x >> 4), threadIdx.x & 15, (threadIdx.x >> 4) < G);  // 16 threads per head
-      }
-    }
+    if (p.merge_counters) merge_if_last(p, r, h, G, nc, s0);
     __syncthreads();
   }
 }
 
-// The merge as a kernel of its own: 16 threads per head; a CTA of 128 threads takes 8 heads.
+// The merge as a kernel of its own: a warp per head.
 __global__ void __launch_bounds__(128) attention_merge_kernel(const AttnArgs p) {
   grid_launch_dependents();
   grid_dependency_wait();
-  const int r = blockIdx.x, a = blockIdx.y * 8 + (threadIdx.x >> 4), ch = threadIdx.x & 15;
-  merge_head_chunk(p, r, a, ch, a < p.nq);
+  const int r = blockIdx.x, a = blockIdx.y * 4 + (threadIdx.x >> 5);
+  if (a < p.nq) merge_head(p, r, p.slot_base[r], p.nchunks[r], a);
 }
 
 // One warp per (request, head of qkv): optional RMSNorm over the head, rotary embedding at the
@@ -842,7 +848,7 @@ cudaError_t launch_paged_attention(const AttnArgs& a, cudaStream_t s) {
 
 cudaError_t launch_attention_merge(const AttnArgs& a, cudaStream_t s) {
   if (a.n <= 0) return cudaSuccess;
-  return launch_kernel(attention_merge_kernel, dim3(a.n, (a.nq + 7) / 8), dim3(128), 0, s, a);
+  return launch_kernel(attention_merge_kernel, dim3(a.n, (a.nq + 3) / 4), dim3(128), 0, s, a);
 }
 
 cudaError_t launch_rope_append(const RopeArgs& a, cudaStream_t s) {
