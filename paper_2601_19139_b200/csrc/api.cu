@@ -483,7 +483,7 @@ int read_back_status(q4d_model* m, cudaStream_t s) {
   } while (0)
 
 // What follows the attention in a layer, for n rows of the residual stream x (rows H apart): O projection of the operand
-// the attention left, norm, MLP or experts.
+// the attention left, norm, MLP or experts.  With experts it ends with the next layer's norm, or the final one.
 int layer_tail(q4d_model* m, int l, int n, uint16_t* x, cudaStream_t s) {
   const q4d_shape& sh = m->sh;
   const q4d_layer_weights& lw = m->layers[l];
@@ -521,19 +521,22 @@ int layer_tail(q4d_model* m, int l, int n, uint16_t* x, cudaStream_t s) {
     Q4D_LAUNCH(Q4D_K_MOE_DOWN, launch_q4_experts(ea, s));
     MoeCombineArgs mc;
     mc.x = x, mc.o = eo, mc.pos = mr.pos, mc.wgt = mr.wgt, mc.H = H, mc.top_k = sh.top_k;
-    Q4D_LAUNCH(Q4D_K_MOE_DOWN, launch_moe_combine(mc, n, s));
+    mc.norm = l + 1 < sh.n_layers ? m->layers[l + 1].attn_norm : m->w.final_norm, mc.eps = sh.rms_eps;
+    mc.yp = yp, mc.ys = ys, mc.layout = dense_layout;
+    Q4D_LAUNCH(Q4D_K_MOE_DOWN, launch_moe_combine_norm(mc, n, s));
   }
   return Q4D_OK;
 }
 
-// Final norm, head and argmax of n rows.
+// Final norm (unless the last layer has ended with it), head and argmax of n rows.
 int head_launches(q4d_model* m, int n, const uint16_t* x, float* logits, int32_t* next_dev, cudaStream_t s) {
   const q4d_shape& sh = m->sh;
   const int H = sh.hidden, V = sh.vocab;
   uint16_t* yp = at<uint16_t>(m, m->lay.yp);
   void* ys = at<unsigned char>(m, m->lay.ys);
   float2* amax = at<float2>(m, m->lay.amax);
-  Q4D_LAUNCH(Q4D_K_RMSNORM, launch_rmsnorm(x, m->w.final_norm, sh.rms_eps, n, H, nullptr, yp, ys, gemm_operand_layout(), s));
+  if (sh.n_experts == 0)
+    Q4D_LAUNCH(Q4D_K_RMSNORM, launch_rmsnorm(x, m->w.final_norm, sh.rms_eps, n, H, nullptr, yp, ys, gemm_operand_layout(), s));
   GemmArgs lm = gemm_args(m, m->w.lm_head, V, H, yp, ys, n, EPI_F32, logits, V, 4 * sh.n_layers);
   lm.argmax_partial = amax;
   const int lm_blocks = gemm_row_blocks(V, H, n, EPI_F32);
@@ -686,7 +689,8 @@ int step_impl(q4d_model* m, q4d_kv_pool* pool, int32_t n, const int64_t* ids, co
     const q4d_layer_weights& lw = m->layers[l];
     uint16_t* kpool = pool->mem + (size_t)(2 * l) * layer_elems;
     uint16_t* vpool = kpool + layer_elems;
-    Q4D_LAUNCH(Q4D_K_RMSNORM, launch_rmsnorm(x, lw.attn_norm, sh.rms_eps, n, H, nullptr, yp, ys, dense_layout, s));
+    if (l == (range ? range->begin : 0) || sh.n_experts == 0)
+      Q4D_LAUNCH(Q4D_K_RMSNORM, launch_rmsnorm(x, lw.attn_norm, sh.rms_eps, n, H, nullptr, yp, ys, dense_layout, s));
     Q4D_LAUNCH(Q4D_K_GEMM_QKV, launch_q4_gemm(gemm_args(m, lw.wqkv, nqkv, H, yp, ys, n, EPI_BF16, qkv, nqkv, 4 * l), s));
     AttnArgs aa;
     aa.q = qbuf, aa.kpool = kpool, aa.vpool = vpool, aa.block_tables = d_bt, aa.lens = d_lens;

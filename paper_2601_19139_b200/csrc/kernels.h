@@ -183,9 +183,14 @@ struct MoeCombineArgs {
   const int32_t* pos;
   const float* wgt;
   int H, top_k;
+  const uint16_t* norm;  // the next norm's weights; its output is the operand yp, ys
+  float eps;
+  uint16_t* yp;
+  void* ys;
+  int layout;
 };
 cudaError_t launch_moe_router(const MoeRouteArgs& a, int n, cudaStream_t s);
-cudaError_t launch_moe_combine(const MoeCombineArgs& a, int n, cudaStream_t s);
+cudaError_t launch_moe_combine_norm(const MoeCombineArgs& a, int n, cudaStream_t s);
 
 // ---- prompt processing (prefill.cu): many tokens of one request at once ------------------
 // Operand of a prompt projection: f16 [rows][prefill_operand_stride(K)], every row scaled by a power of two of its own

@@ -612,8 +612,9 @@ __global__ void __launch_bounds__(32 * slice_max_warps(1), 1) q4_expert_kernel(c
   } else {
     grid_launch_dependents();
   }
+  // the whole list without waiting for its length: one round trip
   const int n_units = min(__ldcg(p.n_units), kMaxExpertUnits);
-  for (int i = threadIdx.x; i < n_units; i += blockDim.x) s_units[i] = __ldcg(p.units + i);
+  for (int i = threadIdx.x; i < kMaxExpertUnits; i += blockDim.x) s_units[i] = __ldcg(p.units + i);
   __syncthreads();
   const int total = n_units * p.tiles;
   const int t0 = (int)((long long)blockIdx.x * total / gridDim.x), Tc = (int)((long long)(blockIdx.x + 1) * total / gridDim.x) - t0;
