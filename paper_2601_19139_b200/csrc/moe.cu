@@ -62,10 +62,11 @@ __device__ __forceinline__ void select_experts(const float* sz, int E, int top_k
   if (norm) my_w = my_w / warp_sum(my_w);
 }
 
-constexpr int kRouterThreads = 256;
+constexpr int kRouterThreads = 512;  // a warp per 128 features, and per request
 constexpr int kRouterWarps = kRouterThreads / 32;
+constexpr int kExpertWarps = kMaxExperts / 32;
 
-// One CTA per 8 experts, for all requests at once: the warps split the features (256 each), multiply their part of the
+// One CTA per 8 experts, for all requests at once: the warps split the features (128 each), multiply their part of the
 // requests (MMA rows) with their part of the 8 router rows (columns) straight from global memory, all loads in flight
 // together, and add up in shared memory in feature order.  The CTA that finishes last selects every request's experts (a
 // warp per request) and turns the choices into the list of units the expert projections walk.  (One CTA per 8 experts and
@@ -74,30 +75,30 @@ constexpr int kRouterWarps = kRouterThreads / 32;
 __global__ void __launch_bounds__(kRouterThreads) moe_router_kernel(const MoeRouteArgs p, int n) {
   __shared__ float s_part[kRouterWarps][16][8];
   __shared__ float sz[kMaxBatch][kMaxExperts];
-  __shared__ int s_last, s_base[kMaxExperts], s_warp_units[kRouterWarps], s_warp_touched[kRouterWarps];
+  __shared__ int s_last, s_base[kMaxExperts], s_warp_units[kExpertWarps], s_warp_touched[kExpertWarps];
   __shared__ uint32_t s_mask[kMaxExperts];      // requests of an expert
   __shared__ short s_idx[kMaxBatch * 32];       // [request][top_k]
   grid_launch_dependents();
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, g = lane >> 2, t = lane & 3;
   const int e0 = blockIdx.x * 8;
-  const bool active = warp * 256 < p.H;
-  uint4 wv[8];
+  const bool active = warp * 128 < p.H;
+  uint4 wv[4];
   if (active) {  // the router does not depend on the preceding kernel
-    const uint16_t* w = p.router + (size_t)min(e0 + g, p.E - 1) * p.H + warp * 256 + t * 8;
+    const uint16_t* w = p.router + (size_t)min(e0 + g, p.E - 1) * p.H + warp * 128 + t * 8;
 #pragma unroll
-    for (int i = 0; i < 8; ++i) wv[i] = __ldg(reinterpret_cast<const uint4*>(w + i * 32));
+    for (int i = 0; i < 4; ++i) wv[i] = __ldg(reinterpret_cast<const uint4*>(w + i * 32));
   }
-  s_mask[threadIdx.x] = 0u;
+  if (threadIdx.x < kMaxExperts) s_mask[threadIdx.x] = 0u;
   grid_dependency_wait();
   float acc[4] = {0.0f, 0.0f, 0.0f, 0.0f};
   if (active) {
-    const uint16_t* y = p.y + warp * 256 + t * 8;
+    const uint16_t* y = p.y + warp * 128 + t * 8;
     const uint16_t *lo = y + (size_t)min(g, n - 1) * p.H, *hi = y + (size_t)min(g + 8, n - 1) * p.H;
-    uint4 a[8], b[8];
+    uint4 a[4], b[4];
 #pragma unroll
-    for (int i = 0; i < 8; ++i) a[i] = *reinterpret_cast<const uint4*>(lo + i * 32), b[i] = *reinterpret_cast<const uint4*>(hi + i * 32);
+    for (int i = 0; i < 4; ++i) a[i] = *reinterpret_cast<const uint4*>(lo + i * 32), b[i] = *reinterpret_cast<const uint4*>(hi + i * 32);
 #pragma unroll
-    for (int i = 0; i < 8; ++i) {  // a 16-byte load is two k-steps of the same permutation of k on both sides
+    for (int i = 0; i < 4; ++i) {  // a 16-byte load is two k-steps of the same permutation of k on both sides
       mma_bf16(acc, a[i].x, b[i].x, a[i].y, b[i].y, wv[i].x, wv[i].y);
       mma_bf16(acc, a[i].z, b[i].z, a[i].w, b[i].w, wv[i].z, wv[i].w);
     }
@@ -139,7 +140,7 @@ __global__ void __launch_bounds__(kRouterThreads) moe_router_kernel(const MoeRou
   __syncthreads();
   // units in ascending expert order, an expert's requests in ascending order: thread e serves expert e
   const int e = threadIdx.x;
-  uint32_t left = s_mask[e];
+  uint32_t left = e < kMaxExperts ? s_mask[e] : 0u;
   const int count = __popc(left), mine = (count + 7) >> 3;
   int units = mine;  // inclusive prefix sum over the experts
 #pragma unroll
@@ -148,21 +149,25 @@ __global__ void __launch_bounds__(kRouterThreads) moe_router_kernel(const MoeRou
     if (lane >= o) units += a;
   }
   const unsigned touched = __ballot_sync(0xffffffffu, count > 0);
-  if (lane == 31) s_warp_units[warp] = units, s_warp_touched[warp] = __popc(touched);
+  if (lane == 31 && warp < kExpertWarps) s_warp_units[warp] = units, s_warp_touched[warp] = __popc(touched);
   __syncthreads();
-  for (int w = 0; w < warp; ++w) units += s_warp_units[w];
-  s_base[e] = units - mine;
-  for (int u = 0; u < mine; ++u) {
-    uint32_t ids[2] = {0u, 0u};
-    int k = 0;
-    for (; k < 8 && left; ++k, left &= left - 1u) ids[k >> 2] |= (uint32_t)(__ffs(left) - 1) << ((k & 3) * 8);
-    p.units[units - mine + u] = make_int4(e, k, (int)ids[0], (int)ids[1]);
-  }
-  if (e == kRouterThreads - 1) {
-    *p.n_units = units;
-    int tot = 0;
-    for (int w = 0; w < kRouterWarps; ++w) tot += s_warp_touched[w];
-    if (p.touched_total) atomicAdd(p.touched_total, tot);  // nobody waits for it
+  if (e < kMaxExperts) {
+#pragma unroll
+    for (int w = 0; w < kExpertWarps; ++w) units += w < warp ? s_warp_units[w] : 0;
+    s_base[e] = units - mine;
+    for (int u = 0; u < mine; ++u) {
+      uint32_t ids[2] = {0u, 0u};
+      int k = 0;
+      for (; k < 8 && left; ++k, left &= left - 1u) ids[k >> 2] |= (uint32_t)(__ffs(left) - 1) << ((k & 3) * 8);
+      p.units[units - mine + u] = make_int4(e, k, (int)ids[0], (int)ids[1]);
+    }
+    if (e == kMaxExperts - 1) {
+      *p.n_units = units;
+      int tot = 0;
+#pragma unroll
+      for (int w = 0; w < kExpertWarps; ++w) tot += s_warp_touched[w];
+      if (p.touched_total) atomicAdd(p.touched_total, tot);  // nobody waits for it
+    }
   }
   __syncthreads();
   for (int i = threadIdx.x; i < n * p.top_k; i += kRouterThreads) {
@@ -252,9 +257,11 @@ __global__ void __launch_bounds__(256) moe_combine_norm_kernel(const MoeCombineA
 }
 
 // ---- many tokens (prompt processing) -------------------------------------------------------------------------------
+constexpr int kPrefillRouterThreads = 256;
+
 // Router of 16 tokens per CTA: logits on m16n8k16 MMAs with fp32 accumulation (rows = experts, columns = tokens; a lane's
 // 16-byte loads hold two k-steps of the same permutation of k on both sides), then one warp per token selects.
-__global__ void __launch_bounds__(kRouterThreads) prefill_router_kernel(const PrefillMoeArgs p) {
+__global__ void __launch_bounds__(kPrefillRouterThreads) prefill_router_kernel(const PrefillMoeArgs p) {
   extern __shared__ __align__(16) unsigned char router_smem[];
   const int stride = p.H * 2 + 16;                                      // bytes per token row: 16 apart modulo 128
   float* sz = reinterpret_cast<float*>(router_smem + 16 * stride);      // [16][E]
@@ -262,13 +269,13 @@ __global__ void __launch_bounds__(kRouterThreads) prefill_router_kernel(const Pr
   grid_dependency_wait();
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, g = lane >> 2, t = lane & 3;
   const int t0 = blockIdx.x * 16, chunks = p.H >> 3;
-  for (int c = threadIdx.x; c < 16 * chunks; c += kRouterThreads) {
+  for (int c = threadIdx.x; c < 16 * chunks; c += kPrefillRouterThreads) {
     const int r = c / chunks, k = c - r * chunks;
     *reinterpret_cast<uint4*>(router_smem + r * stride + k * 16) =
         *reinterpret_cast<const uint4*>(p.y + (size_t)min(t0 + r, p.rows - 1) * p.H + k * 8);
   }
   __syncthreads();
-  for (int e0 = warp * 16; e0 < p.E; e0 += kRouterWarps * 16) {
+  for (int e0 = warp * 16; e0 < p.E; e0 += (kPrefillRouterThreads / 32) * 16) {
     const uint16_t* w_lo = p.router + (size_t)min(e0 + g, p.E - 1) * p.H + t * 8;
     const uint16_t* w_hi = p.router + (size_t)min(e0 + g + 8, p.E - 1) * p.H + t * 8;
     float acc[2][4] = {{0.f, 0.f, 0.f, 0.f}, {0.f, 0.f, 0.f, 0.f}};
@@ -291,7 +298,7 @@ __global__ void __launch_bounds__(kRouterThreads) prefill_router_kernel(const Pr
       }
   }
   __syncthreads();
-  for (int i = warp; i < 16 && t0 + i < p.rows; i += kRouterWarps) {
+  for (int i = warp; i < 16 && t0 + i < p.rows; i += (kPrefillRouterThreads / 32)) {
     int e;
     float w;
     select_experts(sz + i * p.E, p.E, p.top_k, p.norm, lane, e, w);
@@ -367,7 +374,7 @@ __global__ void __launch_bounds__(256) prefill_combine_kernel(const PrefillMoeAr
 cudaError_t launch_moe_router(const MoeRouteArgs& a, int n, cudaStream_t s) {
   if (n <= 0) return cudaSuccess;
   if (a.E < 1 || a.E > kMaxExperts || a.top_k < 1 || a.top_k > 32 || a.top_k > a.E || a.H % 8) return cudaErrorInvalidValue;
-  if (a.H % 256 || a.H > 2048 || n > kMaxBatch || !a.logits) return cudaErrorInvalidValue;
+  if (a.H % 128 || a.H > kRouterWarps * 128 || n > kMaxBatch || !a.logits) return cudaErrorInvalidValue;
   return launch_kernel(moe_router_kernel, dim3((a.E + 7) / 8), dim3(kRouterThreads), 0, s, a, n);
 }
 
@@ -388,7 +395,7 @@ cudaError_t launch_prefill_route(const PrefillMoeArgs& a, cudaStream_t s) {
     attr_set = true;
   }
   if (smem > 160 * 1024) return cudaErrorInvalidValue;
-  cudaError_t e = launch_kernel(prefill_router_kernel, dim3((a.rows + 15) / 16), dim3(kRouterThreads), smem, s, a);
+  cudaError_t e = launch_kernel(prefill_router_kernel, dim3((a.rows + 15) / 16), dim3(kPrefillRouterThreads), smem, s, a);
   if (e == cudaSuccess) e = launch_kernel(prefill_units_kernel, dim3(1), dim3(kMaxExperts), 0, s, a);
   if (e == cudaSuccess) e = launch_kernel(prefill_scatter_kernel, dim3(a.rows), dim3(256), 0, s, a);
   return e;

@@ -574,6 +574,7 @@ struct ExpertParams {
   const int* n_units;
   size_t unit_stride, out_unit_stride;  // elements
   int N, K, tiles;           // rows and row tiles of an expert
+  unsigned tiles_inv;        // 2^32 / tiles, rounded up: the high word of a product with it divides a tile's number
   int kw, rg, batch;
 };
 
@@ -623,7 +624,7 @@ __global__ void __launch_bounds__(32 * slice_max_warps(1), 1) q4_expert_kernel(c
   const uint32_t ring_a = smem_u32(ring), sb_a = smem_u32(ring_sb), bar_a = smem_u32(&s_bar[warp][0]);
   const int gx = (j * 4) & ~7, sb_half = SB_TMA ? (j & 1) * 8 : 0;
   auto issue = [&](int gt, int slot) {  // tile gt of the list
-    const int unit = gt / p.tiles, tile = gt - unit * p.tiles;
+    const int unit = (int)__umulhi((unsigned)gt, p.tiles_inv), tile = gt - unit * p.tiles;
     const int e = __shfl_sync(0xffffffffu, s_units[unit].x, 0);
     const int y = GATE_UP ? tile * 8 : e * p.N + tile * 16, z = GATE_UP ? 2 * e : 0;
     if (elect_one()) {
@@ -696,7 +697,7 @@ __global__ void __launch_bounds__(32 * slice_max_warps(1), 1) q4_expert_kernel(c
     wait(full_a + buf * 8, (uint32_t)((b >> 1) & 1));
     __syncwarp();
     for (; task < tiles; task += warps) {
-      const int gt = t0 + first + task, unit = gt / p.tiles, tile = gt - unit * p.tiles;
+      const int gt = t0 + first + task, unit = (int)__umulhi((unsigned)gt, p.tiles_inv), tile = gt - unit * p.tiles;
       const int count = s_units[unit].y;
       float v[4] = {0.0f, 0.0f, 0.0f, 0.0f};
       const float4* src = sP + buf * buf_f4 + task * (p.kw * 32) + lane;
@@ -738,7 +739,7 @@ __global__ void __launch_bounds__(32 * slice_max_warps(1), 1) q4_expert_kernel(c
     const int it_end = min(my_n, (b + 1) * p.batch);
     for (; it < it_end; ++it, dst += part_step, gt += rg) {
       if (gt >= unit_end) {
-        unit = gt / p.tiles, unit_end = (unit + 1) * p.tiles;
+        unit = (int)__umulhi((unsigned)gt, p.tiles_inv), unit_end = (unit + 1) * p.tiles;
         load_operand(unit);
       }
       if (!SB_TMA) cp_async_wait<kSliceSlots - 1>();
@@ -936,10 +937,12 @@ cudaError_t launch_q4_experts(const ExpertArgs& a, cudaStream_t s) {
   }
   if (a.N % 16 || a.K % 256 || a.K / 256 > slice_max_warps(1) || !a.maps || !a.units || !a.n_units) return cudaErrorInvalidValue;
   const ExpertPlan t = plan_experts(a.N, a.K);
+  if (t.tiles < 2 || t.tiles > 3600) return cudaErrorInvalidValue;  // where tiles_inv is exact for every tile of the list
   ExpertParams p;
   p.scales = a.scales, p.biases = a.biases, p.xp = a.xp, p.xs = static_cast<const unsigned char*>(a.xs), p.out = a.out, p.out_xp = a.out_xp;
   p.status = a.status, p.units = a.units, p.n_units = a.n_units, p.unit_stride = a.unit_stride, p.out_unit_stride = a.out_unit_stride;
   p.N = a.N, p.K = a.K, p.tiles = t.tiles, p.kw = t.kw, p.rg = t.rg, p.batch = t.batch;
+  p.tiles_inv = (unsigned)((((unsigned long long)1 << 32) + t.tiles - 1) / t.tiles);
   const dim3 grid(g_sm_count), block(32 * t.kw * t.rg);
   auto go = [&](auto kernel) { return launch_kernel(kernel, grid, block, t.smem, s, p, *a.maps); };
   if (a.gate_up) return a.maps->sb_tma ? go(q4_expert_kernel<true, true>) : go(q4_expert_kernel<true, false>);
