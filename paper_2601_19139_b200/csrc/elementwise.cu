@@ -38,40 +38,33 @@ __global__ void embed_kernel(const uint32_t* q, const uint16_t* scales, const ui
   }
 }
 
-__device__ __forceinline__ float block_sum(float v, float* red) {
-  v = warp_sum(v);
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, nw = blockDim.x >> 5;
-  if (lane == 0) red[warp] = v;
-  __syncthreads();
-  float tot = 0.0f;
-  for (int i = 0; i < nw; ++i) tot += red[i];  // same order in every thread
-  __syncthreads();
-  return tot;
-}
-
-// y = bf16(x / sqrt(mean(x^2) + eps) * w); one CTA per request row.  The row is held in registers (up to 8 chunks
-// of 8 elements per thread: H <= 16384).  Writes y in plain layout and/or as the next GEMM's operand.
+// y = bf16(x / sqrt(mean(x^2) + eps) * w); one CTA per request row, held in registers: CH chunks of 8 elements per thread
+// (H <= CH * 2048).  Writes y in plain layout and/or as the next GEMM's operand.
+// Registers are what the CTAs of an SM share, and the next projection's CTA is to be beside this one, fetching its first
+// weights, not behind it: with 8 chunks for every H the SMs that held a row started the projection 3 to 4 us after the
+// others (8B shape: gate/up 17.7 us from release to release, of which its own work 13.4).
+template <int CH>
 __global__ void __launch_bounds__(256) rmsnorm_kernel(const uint16_t* x, const uint16_t* w, float eps, int H,
                                                        uint16_t* y, uint16_t* yp, void* ys, int layout) {
   __shared__ float red[8];
   grid_launch_dependents();
   const int r = blockIdx.x, nch = H >> 3;
-  uint4 wv[8];
+  uint4 wv[CH];
 #pragma unroll
-  for (int i = 0; i < 8; ++i) {  // norm weights do not depend on the preceding kernel
+  for (int i = 0; i < CH; ++i) {  // norm weights do not depend on the preceding kernel
     const int c = threadIdx.x + i * 256;
     wv[i] = c < nch ? *reinterpret_cast<const uint4*>(w + c * 8) : make_uint4(0u, 0u, 0u, 0u);
   }
   grid_dependency_wait();
-  uint4 xv[8];
+  uint4 xv[CH];
   float ss = 0.0f;
 #pragma unroll
-  for (int i = 0; i < 8; ++i) {
+  for (int i = 0; i < CH; ++i) {
     const int c = threadIdx.x + i * 256;
     xv[i] = c < nch ? *reinterpret_cast<const uint4*>(x + (size_t)r * H + c * 8) : make_uint4(0u, 0u, 0u, 0u);
   }
 #pragma unroll
-  for (int i = 0; i < 8; ++i) {
+  for (int i = 0; i < CH; ++i) {
     const uint32_t e[4] = {xv[i].x, xv[i].y, xv[i].z, xv[i].w};
 #pragma unroll
     for (int j = 0; j < 4; ++j) {
@@ -80,10 +73,15 @@ __global__ void __launch_bounds__(256) rmsnorm_kernel(const uint16_t* x, const u
       ss = fmaf(b, b, ss);
     }
   }
-  ss = block_sum(ss, red);
+  ss = warp_sum(ss);
+  if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = ss;
+  __syncthreads();
+  ss = 0.0f;
+#pragma unroll
+  for (int i = 0; i < 8; ++i) ss += red[i];  // same order in every thread
   const float inv = 1.0f / sqrtf(ss / (float)H + eps);
 #pragma unroll
-  for (int i = 0; i < 8; ++i) {
+  for (int i = 0; i < CH; ++i) {
     const int c = threadIdx.x + i * 256;
     if (i * 256 >= nch) break;  // uniform across the CTA
     const uint32_t e[4] = {xv[i].x, xv[i].y, xv[i].z, xv[i].w}, ww[4] = {wv[i].x, wv[i].y, wv[i].z, wv[i].w};
@@ -206,7 +204,11 @@ cudaError_t launch_rmsnorm(const uint16_t* x, const uint16_t* w, float eps, int 
                            uint16_t* yp, void* ys, int layout, cudaStream_t s) {
   if (n <= 0) return cudaSuccess;
   if (H % 64 || H > 16384 || (yp && !ys)) return cudaErrorInvalidValue;
-  return launch_kernel(rmsnorm_kernel, dim3(n), dim3(256), 0, s, x, w, eps, H, y, yp, ys, layout);
+  auto go = [&](auto kernel) { return launch_kernel(kernel, dim3(n), dim3(256), 0, s, x, w, eps, H, y, yp, ys, layout); };
+  // More than 8 rows of more than 3072 elements go to a projection whose CTA fills the register file: nothing stands beside it,
+  // and CTAs of few registers, several to an SM, make the step slower (8B shape, 16 requests: 12260 -> 12470 us).
+  if (n > 8 && H > 3072) return go(rmsnorm_kernel<8>);
+  return H <= 2048 ? go(rmsnorm_kernel<1>) : H <= 4096 ? go(rmsnorm_kernel<2>) : H <= 8192 ? go(rmsnorm_kernel<4>) : go(rmsnorm_kernel<8>);
 }
 
 cudaError_t launch_pack_operand(const uint16_t* x, int x_stride, int K, int n, int prologue, uint16_t* xp, void* xs,

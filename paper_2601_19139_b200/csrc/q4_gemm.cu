@@ -250,8 +250,11 @@ __device__ __forceinline__ void slice_epilogue(const SliceParams& p, float (&v)[
   }
 }
 
+// The bound on registers for 8 requests is that of more threads than a CTA has (92 a thread instead of 106): it leaves the
+// register file room for a CTA of the norm before, which this one is to stand beside, not behind (3B shape, eight requests:
+// 5940 -> 5720 us).  With 16 requests it cannot (a bound of 208 costs the LM head 9 us).
 template <int NT, bool SB_TMA>
-__global__ void __launch_bounds__(32 * slice_max_warps(NT), 1) q4_slice_kernel(const SliceParams p, const __grid_constant__ GemmMaps maps) {
+__global__ void __launch_bounds__(NT == 1 ? 608 : 256, 1) q4_slice_kernel(const SliceParams p, const __grid_constant__ GemmMaps maps) {
   constexpr int SUB = slice_sub(NT), kSliceCodes = slice_slot_codes(NT);
   extern __shared__ unsigned char smem_raw[];
   __shared__ __align__(8) uint64_t s_bar[slice_max_warps(NT)][kSliceSlots];
@@ -531,15 +534,15 @@ SlicePlan plan_slices(int N, int K, int n, int epilogue, int sm_count) {
   t.T = epilogue == EPI_SILU_PACK ? (N / 2 + 7) / 8 : (N + 15) / 16;
   int ctas = sm_count / t.parts;
   if (ctas < 1) ctas = 1;
-  t.ctas = t.T < ctas ? t.T : ctas;
-  const int per_cta = (t.T + t.ctas - 1) / t.ctas;
   // A small projection runs on half the warps: then the next kernel's CTAs fit on the SMs beside it (the register file is
   // what they share) and have their first codes by the time they are released, which is worth more than a shorter
   // multiplication (1024 -> 6144 at one request, launch to launch: 4.31 us with 12 warps, which leave the next CTA no
   // room, so that its codes arrive 1.8 us after the release; 3.67 with 8).  It is not worth a third stage per warp, nor a
   // second one with 16 requests, where a stage takes twice as long (2048 -> 5120, 1024 -> 6144: slower).
-  t.rg = max_warps / t.kw;
   const int half = max_warps / 2 / t.kw;
+  t.ctas = t.T < ctas ? t.T : ctas;
+  const int per_cta = (t.T + t.ctas - 1) / t.ctas;
+  t.rg = max_warps / t.kw;
   if (half >= 1 && (per_cta + half - 1) / half <= (t.nt == 1 ? 2 : 1)) t.rg = half;
   if (t.rg > per_cta) t.rg = per_cta;
   const int warps = t.kw * t.rg, rounds = (per_cta + t.rg - 1) / t.rg;
