@@ -412,9 +412,9 @@ __global__ void __launch_bounds__(NT == 1 ? 608 : 256, 1) q4_slice_kernel(const 
     const int first = b * p.batch * rg, tiles = min(p.batch * rg, Tc - first), buf = b & 1;
     wait(full_a + buf * 8, (uint32_t)((b >> 1) & 1));
     __syncwarp();
-    for (bool first_task = true; task < tiles * NT; task += warps, first_task = false) {
-      const int tl = task / NT, nt = task - tl * NT, tile = t0 + first + tl;
-      float v[4] = {0.0f, 0.0f, 0.0f, 0.0f};
+    const int all = tiles * NT;
+    auto add_kslices = [&](int tl, int nt, float (&v)[4]) {
+      v[0] = v[1] = v[2] = v[3] = 0.0f;
       const float4* src = sP + buf * buf_f4 + tl * (p.kw * NT * 32) + nt * 32 + lane;
       for (int k0 = 0; k0 < nks; k0 += 4) {  // four at a time: their loads go out together
         float4 a[4];
@@ -423,37 +423,52 @@ __global__ void __launch_bounds__(NT == 1 ? 608 : 256, 1) q4_slice_kernel(const 
 #pragma unroll
         for (int k = 0; k < 4; ++k) v[0] += a[k].x, v[1] += a[k].y, v[2] += a[k].z, v[3] += a[k].w;
       }
-      bool finish = true;
-      if (parts > 1) {
-        // several CTAs hold parts of this tile's sums: publish, and the last to arrive adds them in part order
-        float4* part = reinterpret_cast<float4*>(p.partial) + (size_t)tile * (NT * 32) + nt * 32 + lane;
-        const size_t stride = (size_t)p.T * (NT * 32);
-        part[blockIdx.y * stride] = make_float4(v[0], v[1], v[2], v[3]);
+    };
+    // Where several CTAs hold parts of a tile's sums they publish them, and the last to arrive adds them in part order.  The
+    // warp publishes all its tiles of the batch before it counts any (a lane per tile, 28 at most): one fence and one round
+    // trip of the counters, not one of each per tile.
+    unsigned last = 0u;
+    const size_t stride = (size_t)p.T * (NT * 32);
+    if (parts > 1) {
+      int mine = 0;
+      for (int tk = task; tk < all; tk += warps, ++mine) {
+        const int tl = tk / NT, nt = tk - tl * NT;
+        float v[4];
+        add_kslices(tl, nt, v);
+        reinterpret_cast<float4*>(p.partial)[blockIdx.y * stride + (size_t)(t0 + first + tl) * (NT * 32) + nt * 32 + lane] = make_float4(v[0], v[1], v[2], v[3]);
+      }
+      __threadfence();
+      __syncwarp();
+      bool is_last = false;
+      if (lane < mine) {
+        const int tk = task + lane * warps, tl = tk / NT, sh = (tk - tl * NT) * 16;  // a tile's two halves count in the halves of its counter
+        int* counter = p.counters + t0 + first + tl;
+        is_last = ((atomicAdd(counter, 1 << sh) >> sh) & 0xffff) == parts - 1;
+        if (is_last) atomicSub(counter, parts << sh);
         __threadfence();
-        __syncwarp();
-        const int sh = nt * 16;  // a tile's two halves count in the two halves of its counter
-        int prev = 0;
-        if (lane == 0) prev = (atomicAdd(p.counters + tile, 1 << sh) >> sh) & 0xffff;
-        prev = __shfl_sync(0xffffffffu, prev, 0);
-        finish = prev == parts - 1;
-        if (finish) {
-          __threadfence();
-          if (lane == 0) atomicSub(p.counters + tile, parts << sh);
-          v[0] = v[1] = v[2] = v[3] = 0.0f;
-          for (int y0 = 0; y0 < parts; y0 += 4) {  // four parts at a time: their loads go out together
-            float4 a[4];
+      }
+      last = __ballot_sync(0xffffffffu, is_last);
+    }
+    for (int i = 0; task < all; task += warps, ++i) {
+      const int tl = task / NT, nt = task - tl * NT, tile = t0 + first + tl;
+      float v[4];
+      if (parts == 1) {
+        add_kslices(tl, nt, v);
+      } else {
+        if (!((last >> i) & 1u)) continue;
+        const float4* part = reinterpret_cast<const float4*>(p.partial) + (size_t)tile * (NT * 32) + nt * 32 + lane;
+        v[0] = v[1] = v[2] = v[3] = 0.0f;
+        for (int y0 = 0; y0 < parts; y0 += 4) {  // four parts at a time: their loads go out together
+          float4 a[4];
 #pragma unroll
-            for (int y = 0; y < 4; ++y) a[y] = y0 + y < parts ? __ldcg(part + (y0 + y) * stride) : make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+          for (int y = 0; y < 4; ++y) a[y] = y0 + y < parts ? __ldcg(part + (y0 + y) * stride) : make_float4(0.0f, 0.0f, 0.0f, 0.0f);
 #pragma unroll
-            for (int y = 0; y < 4; ++y) v[0] += a[y].x, v[1] += a[y].y, v[2] += a[y].z, v[3] += a[y].w;
-          }
+          for (int y = 0; y < 4; ++y) v[0] += a[y].x, v[1] += a[y].y, v[2] += a[y].z, v[3] += a[y].w;
         }
       }
-      if (finish) {
 #pragma unroll
-        for (int q = 0; q < NT; ++q)
-          if (q == nt) slice_epilogue(p, v, tile, q, g, t, first_task && b == 0, old_pair, best[q], bidx[q]);
-      }
+      for (int q = 0; q < NT; ++q)
+        if (q == nt) slice_epilogue(p, v, tile, q, g, t, i == 0 && b == 0, old_pair, best[q], bidx[q]);
     }
     task -= tiles * NT;  // the next batch's first task of this warp
     __syncwarp();
