@@ -204,7 +204,11 @@ constexpr int kPgBlockCycles = 600;   // a block takes about this many cycles an
 constexpr int kPgABlock = 128 * 128;  // 128 rows x 64 f16
 constexpr int kPgCodes = 128 * 64;    // the codes of two blocks
 constexpr int kPgMaxStages = 6, kPgMaxCodes = 8;
-constexpr int kPgSmemBudget = 223 * 1024;
+// Tiles whose exponents and token scales are kept: a narrow tile of a mixture of experts is through before the epilogue of
+// the one before has given its set back (four sets instead of two: the down projection's tiles 5.5 -> 5.0 us).
+__host__ __device__ constexpr int pg_scale_sets(bool grouped) { return grouped ? 4 : 2; }
+__host__ __device__ constexpr int pg_smem_budget(bool grouped) { return (grouped ? 220 : 223) * 1024; }
+constexpr int kPgUnits = 448;         // units kept in shared memory (with one and a half shares each, 256 experts are 427 at most)
 
 struct PgParams {
   const uint16_t* scales;
@@ -265,15 +269,18 @@ struct PgTile {
   int row_tile, tok0, valid, expert;
 };
 
+// GROUPED: the tiles are those of a list of units, 16 to 256 tokens of one expert each.
+template <bool GROUPED>
 __global__ void __launch_bounds__(kPgThreads, 1)
 prefill_gemm_kernel(const PgParams p, const __grid_constant__ CUtensorMap map_b, const __grid_constant__ CUtensorMap map_codes) {
+  constexpr int SETS = pg_scale_sets(GROUPED);
   extern __shared__ unsigned char smem_raw[];
   __shared__ __align__(8) uint64_t full[kPgMaxStages], empty[kPgMaxStages];      // operands of a stage
   __shared__ __align__(8) uint64_t c_full[kPgMaxCodes], c_empty[kPgMaxCodes];    // codes of two blocks
-  __shared__ __align__(8) uint64_t d_full[2], d_empty[2], rs_full[2], rs_empty[2];
+  __shared__ __align__(8) uint64_t d_full[2], d_empty[2], rs_full[SETS], rs_empty[SETS];
   __shared__ uint32_t s_tmem_base;
-  __shared__ int s_rexp[2][128];
-  __shared__ __align__(16) float s_inv[2][256];
+  __shared__ int s_rexp[SETS][128];
+  __shared__ __align__(16) float s_inv[SETS][256];
 
   grid_launch_dependents();
 
@@ -281,32 +288,41 @@ prefill_gemm_kernel(const PgParams p, const __grid_constant__ CUtensorMap map_b,
   const int NS = p.stages, NC = p.code_slots, b_block = p.n_tile * 128, stage_bytes = kPgABlock + b_block;
   unsigned char* sC = smem + NS * stage_bytes;
   const int warp = __shfl_sync(0xffffffffu, threadIdx.x >> 5, 0), lane = threadIdx.x & 31;
-  const bool grouped = p.units != nullptr, silu = p.epilogue == EPI_SILU_PACK;
+  const bool silu = p.epilogue == EPI_SILU_PACK;
   const int half_n = p.N >> 1, K = p.K;
   const int kb_main = K >> 6, kb_all = prefill_operand_stride(K) >> 6, kst = (kb_all + 1) >> 1;  // blocks, pairs of blocks
 
   if (threadIdx.x == 0) {
     for (int s = 0; s < NS; ++s) um_mbar_init(&full[s], 3), um_mbar_init(&empty[s], 1);
     for (int s = 0; s < NC; ++s) um_mbar_init(&c_full[s], 1), um_mbar_init(&c_empty[s], 4);
-    for (int b = 0; b < 2; ++b)
-      um_mbar_init(&d_full[b], 1), um_mbar_init(&d_empty[b], 4), um_mbar_init(&rs_full[b], 2), um_mbar_init(&rs_empty[b], 12);
+    for (int b = 0; b < 2; ++b) um_mbar_init(&d_full[b], 1), um_mbar_init(&d_empty[b], 4);
+    for (int b = 0; b < SETS; ++b) um_mbar_init(&rs_full[b], 2), um_mbar_init(&rs_empty[b], 12);
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
   if (warp == 1) {
     asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(&s_tmem_base)), "n"(512) : "memory");
     asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
   }
-  if (grouped) grid_dependency_wait();  // the list of units is the preceding kernel's
-  const int total = p.row_tiles * (grouped ? *p.n_units : p.tok_tiles) * p.parts;
+  // The list of units is the preceding kernel's.  Every role looks a tile up when it comes to it: from shared memory, for a
+  // tile of the down projection (K = 768) is through in the time of a few loads.
+  int4* s_units = reinterpret_cast<int4*>(sC + NC * kPgCodes);
+  int n_units = 0;
+  if (GROUPED) {
+    grid_dependency_wait();
+    n_units = *p.n_units;
+    for (int i = threadIdx.x; i < min(n_units, kPgUnits); i += kPgThreads) s_units[i] = p.units[i];
+    __syncthreads();
+  }
+  const int total = p.row_tiles * (GROUPED ? n_units : p.tok_tiles) * p.parts;
   // with K in parts, the parts of a tile are neighbours in the list; a part is whole pairs of blocks
   auto tile_kb0 = [&](int idx) -> int { return p.parts == 1 ? 0 : kst * (idx % p.parts) / p.parts * 2; };
   auto tile_kb1 = [&](int idx) -> int { return p.parts == 1 ? kb_all : min(kb_all, kst * (idx % p.parts + 1) / p.parts * 2); };
   auto tile_at = [&](int idx) -> PgTile {
     PgTile t;
     if (p.parts > 1) idx /= p.parts;
-    if (grouped) {
+    if (GROUPED) {
       const int u = idx / p.row_tiles;
-      const int4 un = p.units[u];
+      const int4 un = u < kPgUnits ? s_units[u] : p.units[u];
       t.row_tile = idx - u * p.row_tiles, t.expert = un.x, t.tok0 = un.y, t.valid = un.z;
     } else {
       t.row_tile = idx / p.tok_tiles;
@@ -325,6 +341,12 @@ prefill_gemm_kernel(const PgParams p, const __grid_constant__ CUtensorMap map_b,
     return (size_t)t.expert * p.N + r;
   };
   // exponent of a row over the scales and biases of its whole K, by four neighbouring lanes
+  auto exponent_of = [&](uint32_t ms, uint32_t mb) -> int {
+    float m = fmaxf(8.0f * fmaxf(bf16_lo(ms), bf16_hi(ms)), fmaxf(bf16_lo(mb), bf16_hi(mb)));
+    m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, 1));
+    m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, 2));
+    return range_exponent(m);
+  };
   auto row_exponent = [&](const PgTile& t, int lrow) -> int {
     const size_t off = tensor_row(t, lrow) * (size_t)kb_main + (lane & 3) * 4;
     uint32_t ms = 0, mb = 0;
@@ -333,10 +355,7 @@ prefill_gemm_kernel(const PgParams p, const __grid_constant__ CUtensorMap map_b,
       ms = max_magnitude(ms, __ldg(reinterpret_cast<const uint2*>(p.scales + off + g)));
       mb = max_magnitude(mb, __ldg(reinterpret_cast<const uint2*>(p.biases + off + g)));
     }
-    float m = fmaxf(8.0f * fmaxf(bf16_lo(ms), bf16_hi(ms)), fmaxf(bf16_lo(mb), bf16_hi(mb)));
-    m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, 1));
-    m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, 2));
-    return range_exponent(m);
+    return exponent_of(ms, mb);
   };
   // the first tile's exponents, by everybody at once: nothing can be dequantised without them
   if ((int)blockIdx.x < total) {
@@ -384,7 +403,7 @@ prefill_gemm_kernel(const PgParams p, const __grid_constant__ CUtensorMap map_b,
       }
     };
     issue_codes();
-    if (!grouped) grid_dependency_wait();
+    if (!GROUPED) grid_dependency_wait();
     int s = 0;
     uint32_t phase = 1u;
     for (int idx = blockIdx.x; idx < total && ok; idx += gridDim.x) {
@@ -441,48 +460,68 @@ prefill_gemm_kernel(const PgParams p, const __grid_constant__ CUtensorMap map_b,
   } else if (warp < 4) {
     // ---- token scales of a tile, and the row exponents of the next one ----
     const int tid = threadIdx.x - 64;
-    if (!grouped) grid_dependency_wait();
+    if (!GROUPED) grid_dependency_wait();
     int it = 0;
     for (int idx = blockIdx.x; idx < total && ok; idx += gridDim.x, ++it) {
       const PgTile t = tile_at(idx);
-      const int buf = it & 1;
+      const int set = it % SETS;
       int ex[8];
       if (it > 0) {
+        if (GROUPED) {
+          // eight rows side by side: one after another their loads took as long as a narrow tile (12 us at K = 2048)
+          const uint16_t *sp[8], *bp[8];
+          uint32_t ms[8], mb[8];
 #pragma unroll
-        for (int i = 0; i < 8; ++i) ex[i] = row_exponent(t, i * 16 + (tid >> 2));
+          for (int i = 0; i < 8; ++i) {
+            const size_t off = tensor_row(t, i * 16 + (tid >> 2)) * (size_t)kb_main + (lane & 3) * 4;
+            sp[i] = p.scales + off, bp[i] = p.biases + off, ms[i] = mb[i] = 0u;
+          }
+          for (int g = 0; g + (lane & 3) * 4 < kb_main; g += 16) {
+            uint2 a[8], b[8];
+#pragma unroll
+            for (int i = 0; i < 8; ++i) a[i] = __ldg(reinterpret_cast<const uint2*>(sp[i] + g)), b[i] = __ldg(reinterpret_cast<const uint2*>(bp[i] + g));
+#pragma unroll
+            for (int i = 0; i < 8; ++i) ms[i] = max_magnitude(ms[i], a[i]), mb[i] = max_magnitude(mb[i], b[i]);
+          }
+#pragma unroll
+          for (int i = 0; i < 8; ++i) ex[i] = exponent_of(ms[i], mb[i]);
+        } else {
+#pragma unroll
+          for (int i = 0; i < 8; ++i) ex[i] = row_exponent(t, i * 16 + (tid >> 2));
+        }
       }
-      if (!um_mbar_wait_warp(&rs_empty[buf], (uint32_t)(((it >> 1) & 1) ^ 1))) ok = false;
+      if (!um_mbar_wait_warp(&rs_empty[set], (uint32_t)((it / SETS & 1) ^ 1))) ok = false;
       if (it > 0 && (lane & 3) == 0) {
 #pragma unroll
-        for (int i = 0; i < 8; ++i) s_rexp[buf][i * 16 + (tid >> 2)] = ex[i];
+        for (int i = 0; i < 8; ++i) s_rexp[set][i * 16 + (tid >> 2)] = ex[i];
       }
-      for (int i = tid; i < p.n_tile; i += 64) s_inv[buf][i] = i < t.valid ? p.inv_scale[t.tok0 + i] : 0.0f;
+      for (int i = tid; i < p.n_tile; i += 64) s_inv[set][i] = i < t.valid ? p.inv_scale[t.tok0 + i] : 0.0f;
       __syncwarp();
-      if (lane == 0) um_mbar_arrive(&rs_full[buf]);
+      if (lane == 0) um_mbar_arrive(&rs_full[set]);
     }
     if (!ok && lane == 0 && p.status) atomicExch(p.status, 3u);
   } else if (warp < 8) {
     // ---- epilogue ----
     const int q = warp - 4;
     const uint32_t lane_addr = tbase + ((uint32_t)(q * 32) << 16);
-    if (!grouped) grid_dependency_wait();  // the output may still be read by the preceding kernels
+    if (!GROUPED) grid_dependency_wait();  // the output may still be read by the preceding kernels
     int it = 0;
     for (int idx = blockIdx.x; idx < total && ok; idx += gridDim.x, ++it) {
       const PgTile t = tile_at(idx);
-      const int buf = it & 1;
+      const int buf = it & 1, set = it % SETS;
       const uint32_t par = (uint32_t)((it >> 1) & 1);
-      if (!um_mbar_wait_warp(&rs_full[buf], par) || !um_mbar_wait_warp(&d_full[buf], par)) {
+      if (!um_mbar_wait_warp(&rs_full[set], (uint32_t)(it / SETS & 1)) || !um_mbar_wait_warp(&d_full[buf], par)) {
         ok = false;
         break;
       }
       tc_fence_after();
-      const float rinv = pow2f(-s_rexp[buf][q * 32 + lane]);
+      const float rinv = pow2f(-s_rexp[set][q * 32 + lane]);
       for (int c0 = 0; c0 < t.valid; c0 += 16) {
         float v[16];
         tmem_ld16f(lane_addr + (uint32_t)(buf * 256 + c0), v);
 #pragma unroll
         for (int i = 0; i < 16; i += 4) {
-          const float4 cs = *reinterpret_cast<const float4*>(&s_inv[buf][c0 + i]);
+          const float4 cs = *reinterpret_cast<const float4*>(&s_inv[set][c0 + i]);
           v[i] = v[i] * rinv * cs.x, v[i + 1] = v[i + 1] * rinv * cs.y;
           v[i + 2] = v[i + 2] * rinv * cs.z, v[i + 3] = v[i + 3] * rinv * cs.w;
         }
@@ -533,7 +572,7 @@ prefill_gemm_kernel(const PgParams p, const __grid_constant__ CUtensorMap map_b,
       }
       tc_fence_before();
       __syncwarp();
-      if (lane == 0) um_mbar_arrive(&d_empty[buf]), um_mbar_arrive(&rs_empty[buf]);
+      if (lane == 0) um_mbar_arrive(&d_empty[buf]), um_mbar_arrive(&rs_empty[set]);
     }
     if (!ok && lane == 0 && p.status) atomicExch(p.status, 3u);
   } else {
@@ -551,14 +590,12 @@ prefill_gemm_kernel(const PgParams p, const __grid_constant__ CUtensorMap map_b,
     int a_off[8];  // rows 64 apart share the swizzle
 #pragma unroll
     for (int i = 0; i < 8; ++i) a_off[i] = (i ^ (tid & 7)) << 4;
-    const uint16_t *srow[2], *brow[2];
+    const uint16_t* srow[2];
+    const ptrdiff_t to_biases = p.biases - p.scales;
     uint16_t nsc[2] = {0, 0};
     auto set_tile = [&](const PgTile& t) {
 #pragma unroll
-      for (int i = 0; i < 2; ++i) {
-        const size_t r = tensor_row(t, tid + 64 * i) * (size_t)kb_main;
-        srow[i] = p.scales + r, brow[i] = p.biases + r;
-      }
+      for (int i = 0; i < 2; ++i) srow[i] = p.scales + tensor_row(t, tid + 64 * i) * (size_t)kb_main;
     };
     auto load_scales = [&](int j) {
 #pragma unroll
@@ -573,17 +610,17 @@ prefill_gemm_kernel(const PgParams p, const __grid_constant__ CUtensorMap map_b,
         if (++c_slot == NC) c_slot = 0, c_phase ^= 1u;
     };
     for (int idx = blockIdx.x; idx < total && ok; idx += gridDim.x, ++it) {
-      const int buf = it & 1, kb0 = tile_kb0(idx), kb1 = tile_kb1(idx), kc1 = min(kb1, kb_main);
+      const int set = it % SETS, kb0 = tile_kb0(idx), kb1 = tile_kb1(idx), kc1 = min(kb1, kb_main);
       int j = kb0 + ((grp - base) & 3);
       set_tile(tile_at(idx));
       if (j < kc1) load_scales(j);
-      if (it > 0 && !um_mbar_wait_warp(&rs_full[buf], (uint32_t)((it >> 1) & 1))) {
+      if (it > 0 && !um_mbar_wait_warp(&rs_full[set], (uint32_t)(it / SETS & 1))) {
         ok = false;
         break;
       }
       float rs[2];
 #pragma unroll
-      for (int i = 0; i < 2; ++i) rs[i] = pow2f(s_rexp[buf][tid + 64 * i]);
+      for (int i = 0; i < 2; ++i) rs[i] = pow2f(s_rexp[set][tid + 64 * i]);
       c_seen = 0;
       for (; j < kb1; j += 4) {
         unsigned char* dst = a_row + s * stage_bytes;
@@ -623,8 +660,17 @@ prefill_gemm_kernel(const PgParams p, const __grid_constant__ CUtensorMap map_b,
 #pragma unroll
           for (int c = 0; c < 8; ++c) *reinterpret_cast<uint4*>(dst + 64 * 128 + a_off[c]) = a[c];
         } else {
-          // 16 groups: {b, b} against {X1, X2}, {8 s, 8 s} against the same
+          // 16 groups: {b, b} against {X1, X2}, {8 s, 8 s} against the same.  Narrow tiles: all loads go out together, before
+          // the wait for the stage.
           const int e = (j - kb_main) * 16;
+          auto load_groups = [&](int i, int q, int c) {  // row, biases or scales, four groups
+            return e + c * 4 < kb_main ? __ldg(reinterpret_cast<const uint2*>(srow[i] + (q ? 0 : to_biases) + e + c * 4)) : make_uint2(0u, 0u);
+          };
+          uint2 v[2][2][4];
+          if (GROUPED) {
+#pragma unroll
+            for (int k = 0; k < 16; ++k) v[k >> 3][(k >> 2) & 1][k & 3] = load_groups(k >> 3, (k >> 2) & 1, k & 3);
+          }
           if (!um_mbar_wait_warp(&empty[s], phase)) {
             ok = false;
             break;
@@ -632,14 +678,13 @@ prefill_gemm_kernel(const PgParams p, const __grid_constant__ CUtensorMap map_b,
 #pragma unroll
           for (int i = 0; i < 2; ++i)
 #pragma unroll
-            for (int q = 0; q < 2; ++q) {  // scales or biases of 16 groups
-              const uint16_t* src = (q ? srow[i] : brow[i]) + e;
+            for (int q = 0; q < 2; ++q) {
               const float f = q ? 8.0f * rs[i] : rs[i];
               uint32_t o[8];
 #pragma unroll
               for (int c = 0; c < 4; ++c) {
-                const uint2 v = e + c * 4 < kb_main ? __ldg(reinterpret_cast<const uint2*>(src + c * 4)) : make_uint2(0u, 0u);
-                o[2 * c] = pack_f16x2(bf16_lo(v.x) * f, bf16_hi(v.x) * f), o[2 * c + 1] = pack_f16x2(bf16_lo(v.y) * f, bf16_hi(v.y) * f);
+                const uint2 w = GROUPED ? v[i][q][c] : load_groups(i, q, c);
+                o[2 * c] = pack_f16x2(bf16_lo(w.x) * f, bf16_hi(w.x) * f), o[2 * c + 1] = pack_f16x2(bf16_lo(w.y) * f, bf16_hi(w.y) * f);
               }
 #pragma unroll
               for (int c = 0; c < 4; ++c)
@@ -657,7 +702,7 @@ prefill_gemm_kernel(const PgParams p, const __grid_constant__ CUtensorMap map_b,
       // the tile's code slots this pair did not look at go by as well
       if (kc1 > kb0) next_code_slot(((kc1 - kb0) >> 1) - c_seen);
       __syncwarp();
-      if (ok && lane == 0) um_mbar_arrive(&rs_empty[buf]);
+      if (ok && lane == 0) um_mbar_arrive(&rs_empty[set]);
     }
     if (!ok && lane == 0 && p.status) atomicExch(p.status, 3u);
   }
@@ -867,7 +912,8 @@ cudaError_t prefill_init() {
   int dev = 0, sms = 0;
   cudaError_t e = cudaGetDevice(&dev);
   if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-  if (e == cudaSuccess) e = cudaFuncSetAttribute(prefill_gemm_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kPgSmemBudget);
+  if (e == cudaSuccess) e = cudaFuncSetAttribute(prefill_gemm_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, pg_smem_budget(false));
+  if (e == cudaSuccess) e = cudaFuncSetAttribute(prefill_gemm_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, pg_smem_budget(true));
   if (e == cudaSuccess) e = cudaFuncSetAttribute(prefill_attention_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kPaSmem);
   if (e == cudaSuccess) g_prefill_sms = sms;
   return e;
@@ -937,9 +983,10 @@ cudaError_t launch_prefill_gemm(const PrefillGemmArgs& a, cudaStream_t s) {
   // narrow tiles pass through a stage faster, and their smaller operand leaves room for more codes ahead
   p.code_slots = p.n_tile <= 128 ? kPgMaxCodes : 3;
   const int stage = kPgABlock + p.n_tile * 128;
-  p.stages = (kPgSmemBudget - 1024 - p.code_slots * kPgCodes) / stage;
+  const int units_bytes = grouped ? kPgUnits * (int)sizeof(int4) : 0;
+  p.stages = (pg_smem_budget(grouped) - 1024 - units_bytes - p.code_slots * kPgCodes) / stage;
   if (p.stages > kPgMaxStages) p.stages = kPgMaxStages;
-  const size_t smem = 1024 + (size_t)p.stages * stage + (size_t)p.code_slots * kPgCodes;
+  const size_t smem = 1024 + (size_t)p.stages * stage + (size_t)p.code_slots * kPgCodes + units_bytes;
   EncodeTiledFn encode = nullptr;
   cudaError_t e = encode_tiled_fn(&encode);
   if (e != cudaSuccess) return e;
@@ -964,7 +1011,8 @@ cudaError_t launch_prefill_gemm(const PrefillGemmArgs& a, cudaStream_t s) {
   }
   int ctas = g_prefill_sms;
   if (!grouped && p.row_tiles * p.tok_tiles * p.parts < ctas) ctas = p.row_tiles * p.tok_tiles * p.parts;
-  return launch_kernel(prefill_gemm_kernel, dim3(ctas), dim3(kPgThreads), smem, s, p, map_b, map_codes);
+  auto go = [&](auto kernel) { return launch_kernel(kernel, dim3(ctas), dim3(kPgThreads), smem, s, p, map_b, map_codes); };
+  return grouped ? go(prefill_gemm_kernel<true>) : go(prefill_gemm_kernel<false>);
 }
 
 cudaError_t launch_prefill_rope_append(const PrefillAttnArgs& a, cudaStream_t s) {
