@@ -257,30 +257,37 @@ __global__ void __launch_bounds__(256) moe_combine_norm_kernel(const MoeCombineA
 }
 
 // ---- many tokens (prompt processing) -------------------------------------------------------------------------------
-constexpr int kPrefillRouterThreads = 256;
+constexpr int kPrefillRouterThreads = 512;
+constexpr int kPrefillRouterWarps = kPrefillRouterThreads / 32;
+// Parts of the features, so that sixteen warps have a tile of 16 experts each (128 experts: two parts).
+__host__ __device__ inline int prefill_router_parts(int E) { return E <= 64 ? 4 : E <= 128 ? 2 : 1; }
 
 // Router of 16 tokens per CTA: logits on m16n8k16 MMAs with fp32 accumulation (rows = experts, columns = tokens; a lane's
-// 16-byte loads hold two k-steps of the same permutation of k on both sides), then one warp per token selects.
+// 16-byte loads hold two k-steps of the same permutation of k on both sides), then one warp per token selects.  A warp's
+// time is the latency of its router loads, one batch after another: sixteen of them in flight, and the features split
+// over the warps that the experts leave (eight loads, unsplit, and two tokens per warp: 31 us for 500 tokens).
 __global__ void __launch_bounds__(kPrefillRouterThreads) prefill_router_kernel(const PrefillMoeArgs p) {
   extern __shared__ __align__(16) unsigned char router_smem[];
   const int stride = p.H * 2 + 16;                                      // bytes per token row: 16 apart modulo 128
-  float* sz = reinterpret_cast<float*>(router_smem + 16 * stride);      // [16][E]
+  float* sz = reinterpret_cast<float*>(router_smem + 16 * stride);      // [part][16][E]
   grid_launch_dependents();
   grid_dependency_wait();
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, g = lane >> 2, t = lane & 3;
-  const int t0 = blockIdx.x * 16, chunks = p.H >> 3;
-  for (int c = threadIdx.x; c < 16 * chunks; c += kPrefillRouterThreads) {
-    const int r = c / chunks, k = c - r * chunks;
-    *reinterpret_cast<uint4*>(router_smem + r * stride + k * 16) =
-        *reinterpret_cast<const uint4*>(p.y + (size_t)min(t0 + r, p.rows - 1) * p.H + k * 8);
+  const int t0 = blockIdx.x * 16, chunks = p.H >> 3, parts = prefill_router_parts(p.E), len = p.H / parts;
+  for (int r = warp; r < 16; r += kPrefillRouterWarps) {
+    const uint4* src = reinterpret_cast<const uint4*>(p.y + (size_t)min(t0 + r, p.rows - 1) * p.H);
+#pragma unroll 8
+    for (int k = lane; k < chunks; k += 32) *reinterpret_cast<uint4*>(router_smem + r * stride + k * 16) = src[k];
   }
   __syncthreads();
-  for (int e0 = warp * 16; e0 < p.E; e0 += (kPrefillRouterThreads / 32) * 16) {
+  const int tiles = (p.E + 15) >> 4;
+  for (int w = warp; w < tiles * parts; w += kPrefillRouterWarps) {
+    const int part = w / tiles, e0 = (w - part * tiles) * 16, k1 = (part + 1) * len;
     const uint16_t* w_lo = p.router + (size_t)min(e0 + g, p.E - 1) * p.H + t * 8;
     const uint16_t* w_hi = p.router + (size_t)min(e0 + g + 8, p.E - 1) * p.H + t * 8;
     float acc[2][4] = {{0.f, 0.f, 0.f, 0.f}, {0.f, 0.f, 0.f, 0.f}};
-#pragma unroll 4
-    for (int k = 0; k < p.H; k += 32) {
+#pragma unroll 8
+    for (int k = part * len; k < k1; k += 32) {
       const uint4 a = __ldg(reinterpret_cast<const uint4*>(w_lo + k)), b = __ldg(reinterpret_cast<const uint4*>(w_hi + k));
 #pragma unroll
       for (int nt = 0; nt < 2; ++nt) {
@@ -294,11 +301,17 @@ __global__ void __launch_bounds__(kPrefillRouterThreads) prefill_router_kernel(c
 #pragma unroll
       for (int c = 0; c < 4; ++c) {
         const int e = e0 + g + 8 * (c >> 1);
-        if (e < p.E) sz[(nt * 8 + 2 * t + (c & 1)) * p.E + e] = acc[nt][c];
+        if (e < p.E) sz[(part * 16 + nt * 8 + 2 * t + (c & 1)) * p.E + e] = acc[nt][c];
       }
   }
   __syncthreads();
-  for (int i = warp; i < 16 && t0 + i < p.rows; i += (kPrefillRouterThreads / 32)) {
+  for (int i = warp; i < 16 && t0 + i < p.rows; i += kPrefillRouterWarps) {
+    for (int e = lane; e < p.E; e += 32) {  // the parts in order; a lane reads what it has added up
+      float z = sz[i * p.E + e];
+      for (int q = 1; q < parts; ++q) z += sz[(q * 16 + i) * p.E + e];
+      sz[i * p.E + e] = z;
+    }
+    __syncwarp();
     int e;
     float w;
     select_experts(sz + i * p.E, p.E, p.top_k, p.norm, lane, e, w);
@@ -387,7 +400,7 @@ cudaError_t launch_moe_combine_norm(const MoeCombineArgs& a, int n, cudaStream_t
 cudaError_t launch_prefill_route(const PrefillMoeArgs& a, cudaStream_t s) {
   if (a.rows <= 0) return cudaSuccess;
   if (a.E < 1 || a.E > kMaxExperts || a.top_k < 1 || a.top_k > 32 || a.top_k > a.E || a.H % 256) return cudaErrorInvalidValue;
-  const size_t smem = 16 * ((size_t)a.H * 2 + 16) + (size_t)16 * a.E * sizeof(float);
+  const size_t smem = 16 * ((size_t)a.H * 2 + 16) + (size_t)prefill_router_parts(a.E) * 16 * a.E * sizeof(float);
   static bool attr_set = false;
   if (!attr_set) {
     cudaError_t e = cudaFuncSetAttribute(prefill_router_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, 160 * 1024);
