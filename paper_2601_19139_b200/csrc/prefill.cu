@@ -36,6 +36,7 @@ __device__ __forceinline__ uint32_t pack_f16x2(float lo, float hi) { return half
 // fp32 results of a projection whose K was cut into parts, in part order: elements i, i + 1
 __device__ __forceinline__ float2 add_parts(const float* sums, size_t i, int parts, size_t stride) {
   float2 v = *reinterpret_cast<const float2*>(sums + i);
+#pragma unroll 4
   for (int q = 1; q < parts; ++q) {
     const float2 a = *reinterpret_cast<const float2*>(sums + q * stride + i);
     v.x += a.x, v.y += a.y;
@@ -714,15 +715,16 @@ prefill_gemm_kernel(const PgParams p, const __grid_constant__ CUtensorMap map_b,
 
 // ---- rotary embedding and append ---------------------------------------------------------------------------------
 // One warp per (token, head of qkv): optional RMSNorm over the head, rotary embedding at the token's position, then
-// q -> q, k and v -> the token's slot of the pool.
+// q -> q, k and v -> the token's slot of the pool.  A head is a chain of two round trips: with few tokens their heads are
+// spread over CTAs (blockIdx.y) until the chip has a wave of them (77 tokens of the 0.6B shape: 9.9 us with four heads per warp).
 __global__ void __launch_bounds__(256) prefill_rope_kernel(const PrefillAttnArgs p) {
   grid_launch_dependents();
-  grid_dependency_wait();
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int heads = p.nq + 2 * p.nkv, r = blockIdx.x, pos = p.start + r;
   const float4 cs = *reinterpret_cast<const float4*>(p.rope + ((size_t)pos * 64 + 2 * lane) * 2);  // c0 s0 c1 s1
   const int blk = p.block_table[pos / kBlockSize], slot = pos % kBlockSize;
-  for (int hd = warp; hd < heads; hd += 8) {
+  grid_dependency_wait();  // the rotary table and the block table are older than the preceding kernel
+  for (int hd = blockIdx.y * 8 + warp; hd < heads; hd += 8 * gridDim.y) {
     const size_t at = ((size_t)r * heads + hd) * kHeadDim + 2 * lane;
     // lane holds elements 2*lane, 2*lane+1 and their rotary partners 64 + 2*lane, 64 + 2*lane + 1
     uint32_t wa, wb;
@@ -1017,7 +1019,8 @@ cudaError_t launch_prefill_gemm(const PrefillGemmArgs& a, cudaStream_t s) {
 
 cudaError_t launch_prefill_rope_append(const PrefillAttnArgs& a, cudaStream_t s) {
   if (a.rows <= 0) return cudaSuccess;
-  return launch_kernel(prefill_rope_kernel, dim3(a.rows), dim3(256), 0, s, a);
+  const int most = (a.nq + 2 * a.nkv + 7) / 8, fit = g_prefill_sms * 8 / a.rows;  // CTAs of a token's heads; of a wave
+  return launch_kernel(prefill_rope_kernel, dim3(a.rows, fit < 1 ? 1 : (fit < most ? fit : most)), dim3(256), 0, s, a);
 }
 
 cudaError_t launch_prefill_attention(const PrefillAttnArgs& a, cudaStream_t s) {
