@@ -180,8 +180,8 @@ int q4d_decode_step(q4d_model* model, q4d_kv_pool* pool, int32_t n, const int64_
  * K, V, e.g. from q4d_prefix_lookup; a partly cached block that receives new tokens must be the request's own).
  * next_token (device, 1 value) and logits (device f32 [vocab]) may be NULL.  The result is, by definition, what
  * n_tokens - start_pos decode steps feeding the prompt's tokens one by one would leave behind; the library gets
- * there sixteen tokens at a time (one pass over the weights per sixteen tokens, each token attending to the cached
- * ones and to the earlier tokens of its chunk).  On success the request is admitted with n_tokens cached tokens.
+ * there with one pass over the weights per 2048 tokens (up to sixteen tokens: as the rows of one decode step), each
+ * token attending to the cached ones and to the earlier tokens of its pass.  On success the request is admitted with n_tokens cached tokens.
  * Errors: DUPLICATE_REQUEST (already admitted), POSITION_OVERFLOW, BLOCK_TABLE_TOO_SHORT, BLOCK_OUT_OF_RANGE,
  * INVALID_ARG (start_pos outside [0, n_tokens): to reuse a fully cached prompt pass start_pos = n_tokens - 1). */
 int q4d_prefill(q4d_model* model, q4d_kv_pool* pool, int64_t request_id, const int32_t* tokens, int32_t n_tokens,

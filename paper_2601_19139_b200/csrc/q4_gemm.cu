@@ -841,7 +841,7 @@ __global__ void __launch_bounds__(256) argmax_finish_kernel(const float2* partia
 
 }  // namespace
 
-// Dense projections run on the span/round kernels; Q4D_GEMM_KERNEL=tcgen05 (read once per process) selects the
+// Dense projections run on the slice kernel; Q4D_GEMM_KERNEL=tcgen05 (read once per process) selects the
 // tcgen05 kernel of q4_umma.cu instead, which is correct on every shape but, as measured, not yet faster.
 static bool g_legacy = true;
 static bool use_umma(int N, int K, int epilogue) { return !g_legacy && umma_supported(N, K, epilogue); }

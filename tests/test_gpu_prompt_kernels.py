@@ -14,8 +14,12 @@ def _dense(**kw):
     return shapes.toy("prompt-toy-" + "-".join(f"{k}{v}" for k, v in sorted(kw.items())), **a)
 
 
-MOE = shapes.toy("prompt-toy-moe", n_layers=1, hidden=256, n_q_heads=4, n_kv_heads=2, mlp_inter=256, vocab=512, n_experts=12,
-                 top_k=3, expert_inter=256, norm_topk_prob=1, max_positions=1024)
+def _moe(n_experts, top_k):
+    return shapes.toy(f"prompt-toy-moe{n_experts}", n_layers=1, hidden=256, n_q_heads=4, n_kv_heads=2, mlp_inter=256, vocab=512,
+                      n_experts=n_experts, top_k=top_k, expert_inter=256, norm_topk_prob=1, max_positions=1024)
+
+
+MOE = _moe(12, 3)
 
 
 @pytest.mark.gpu
@@ -25,6 +29,7 @@ MOE = shapes.toy("prompt-toy-moe", n_layers=1, hidden=256, n_q_heads=4, n_kv_hea
     (_dense(hidden=1280, mlp_inter=2304), 40, 0),                     # 20 and 36 groups: partly filled stages
     (_dense(qk_norm=0, n_q_heads=6, mlp_inter=768), 50, 16),
     (MOE, 17, 0), (MOE, 150, 0), (MOE, 61, 32),
+    (_moe(80, 8), 70, 0), (_moe(144, 2), 33, 0),                      # the router's features in two parts, and in one
 ], ids=lambda v: getattr(v, "name", str(v)))
 def test_prompt_kernels_at_tile_edges(shape, n_tokens, start):
     from gpu_util import bits, from_bits
