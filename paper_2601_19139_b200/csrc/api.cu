@@ -868,7 +868,7 @@ int prefill_rows(q4d_model* m, q4d_kv_pool* pool, const int32_t* tokens, int row
       mo.counts = at<int32_t>(m, lay.p_counts), mo.cursor = at<int32_t>(m, lay.p_cursor);
       mo.units = at<int4>(m, lay.p_units), mo.n_units = reinterpret_cast<int*>(mo.units + (E + cap / 16 + 1));
       // a unit holds one and a half times an expert's share: most experts are one unit, and little of it is padding
-      mo.unit_rows = std::min(256, std::max(16, (pairs * 3 / (2 * E) + 15) / 16 * 16));
+      mo.unit_rows = std::min(240, std::max(16, (pairs * 3 / (2 * E) + 15) / 16 * 16));
       mo.operand = op, mo.inv_scale = inv, mo.sorted = at<uint16_t>(m, lay.p_pairs), mo.sorted_inv_scale = at<float>(m, lay.p_pairs_inv);
       mo.o = mo.sorted, mo.x = x;
       uint16_t *eh = at<uint16_t>(m, lay.p_eh), *eop = at<uint16_t>(m, lay.p_eop);

@@ -208,7 +208,7 @@ constexpr int kPgMaxStages = 6, kPgMaxCodes = 8;
 // Tiles whose exponents and token scales are kept: a narrow tile of a mixture of experts is through before the epilogue of
 // the one before has given its set back (four sets instead of two: the down projection's tiles 5.5 -> 5.0 us).
 __host__ __device__ constexpr int pg_scale_sets(bool grouped) { return grouped ? 4 : 2; }
-__host__ __device__ constexpr int pg_smem_budget(bool grouped) { return (grouped ? 220 : 223) * 1024; }
+constexpr int kPgSmemBudget = 225 * 1024;
 constexpr int kPgUnits = 448;         // units kept in shared memory (with one and a half shares each, 256 experts are 427 at most)
 
 struct PgParams {
@@ -270,7 +270,7 @@ struct PgTile {
   int row_tile, tok0, valid, expert;
 };
 
-// GROUPED: the tiles are those of a list of units, 16 to 256 tokens of one expert each.
+// GROUPED: the tiles are those of a list of units, 16 to 240 tokens of one expert each.
 template <bool GROUPED>
 __global__ void __launch_bounds__(kPgThreads, 1)
 prefill_gemm_kernel(const PgParams p, const __grid_constant__ CUtensorMap map_b, const __grid_constant__ CUtensorMap map_codes) {
@@ -280,8 +280,8 @@ prefill_gemm_kernel(const PgParams p, const __grid_constant__ CUtensorMap map_b,
   __shared__ __align__(8) uint64_t c_full[kPgMaxCodes], c_empty[kPgMaxCodes];    // codes of two blocks
   __shared__ __align__(8) uint64_t d_full[2], d_empty[2], rs_full[SETS], rs_empty[SETS];
   __shared__ uint32_t s_tmem_base;
-  __shared__ int s_rexp[SETS][128];
-  __shared__ __align__(16) float s_inv[SETS][256];
+  __shared__ signed char s_rexp[SETS][128];             // powers of two of the weight rows
+  __shared__ __align__(16) signed char s_inv[SETS][256];  // and of the tokens (as exponents: shared memory is full)
 
   grid_launch_dependents();
 
@@ -361,7 +361,7 @@ prefill_gemm_kernel(const PgParams p, const __grid_constant__ CUtensorMap map_b,
   // the first tile's exponents, by everybody at once: nothing can be dequantised without them
   if ((int)blockIdx.x < total) {
     const int ex = row_exponent(tile_at(blockIdx.x), threadIdx.x >> 2);
-    if ((lane & 3) == 0) s_rexp[0][threadIdx.x >> 2] = ex;
+    if ((lane & 3) == 0) s_rexp[0][threadIdx.x >> 2] = (signed char)ex;
   }
   tc_fence_before();
   __syncthreads();
@@ -494,9 +494,9 @@ prefill_gemm_kernel(const PgParams p, const __grid_constant__ CUtensorMap map_b,
       if (!um_mbar_wait_warp(&rs_empty[set], (uint32_t)((it / SETS & 1) ^ 1))) ok = false;
       if (it > 0 && (lane & 3) == 0) {
 #pragma unroll
-        for (int i = 0; i < 8; ++i) s_rexp[set][i * 16 + (tid >> 2)] = ex[i];
+        for (int i = 0; i < 8; ++i) s_rexp[set][i * 16 + (tid >> 2)] = (signed char)ex[i];
       }
-      for (int i = tid; i < p.n_tile; i += 64) s_inv[set][i] = i < t.valid ? p.inv_scale[t.tok0 + i] : 0.0f;
+      for (int i = tid; i < p.n_tile; i += 64) s_inv[set][i] = i < t.valid ? (signed char)((int)(__float_as_uint(p.inv_scale[t.tok0 + i]) >> 23) - 127) : (signed char)0;
       __syncwarp();
       if (lane == 0) um_mbar_arrive(&rs_full[set]);
     }
@@ -522,7 +522,8 @@ prefill_gemm_kernel(const PgParams p, const __grid_constant__ CUtensorMap map_b,
         tmem_ld16f(lane_addr + (uint32_t)(buf * 256 + c0), v);
 #pragma unroll
         for (int i = 0; i < 16; i += 4) {
-          const float4 cs = *reinterpret_cast<const float4*>(&s_inv[set][c0 + i]);
+          const char4 ce = *reinterpret_cast<const char4*>(&s_inv[set][c0 + i]);
+          const float4 cs = make_float4(pow2f(ce.x), pow2f(ce.y), pow2f(ce.z), pow2f(ce.w));
           v[i] = v[i] * rinv * cs.x, v[i + 1] = v[i + 1] * rinv * cs.y;
           v[i + 2] = v[i + 2] * rinv * cs.z, v[i + 3] = v[i + 3] * rinv * cs.w;
         }
@@ -643,8 +644,6 @@ prefill_gemm_kernel(const PgParams p, const __grid_constant__ CUtensorMap map_b,
 #pragma unroll
             for (int c = 0; c < 2; ++c)
               w[i][c] = *reinterpret_cast<const uint4*>(c_row[i] + c_slot * kPgCodes + ((((j & 1) * 2 + c) ^ c_swz[i]) << 4));
-          __syncwarp();
-          if (lane == 0) um_mbar_arrive(&c_empty[c_slot]);
           uint4 a[8];
           auto convert = [&](const uint4 (&v)[2], const __half2 sc) {
             a[0] = dequant_word(v[0].x, sc), a[1] = dequant_word(v[0].y, sc), a[2] = dequant_word(v[0].z, sc), a[3] = dequant_word(v[0].w, sc);
@@ -660,6 +659,10 @@ prefill_gemm_kernel(const PgParams p, const __grid_constant__ CUtensorMap map_b,
           convert(w[1], s2[1]);
 #pragma unroll
           for (int c = 0; c < 8; ++c) *reinterpret_cast<uint4*>(dst + 64 * 128 + a_off[c]) = a[c];
+          // The slot goes back when its codes have been used: loads that are merely issued do not hold back the arrival, and
+          // the next codes overtook those of the second row.
+          __syncwarp();
+          if (lane == 0) um_mbar_arrive(&c_empty[c_slot]);
         } else {
           // 16 groups: {b, b} against {X1, X2}, {8 s, 8 s} against the same.  Narrow tiles: all loads go out together, before
           // the wait for the stage.
@@ -914,8 +917,8 @@ cudaError_t prefill_init() {
   int dev = 0, sms = 0;
   cudaError_t e = cudaGetDevice(&dev);
   if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-  if (e == cudaSuccess) e = cudaFuncSetAttribute(prefill_gemm_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, pg_smem_budget(false));
-  if (e == cudaSuccess) e = cudaFuncSetAttribute(prefill_gemm_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, pg_smem_budget(true));
+  if (e == cudaSuccess) e = cudaFuncSetAttribute(prefill_gemm_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, kPgSmemBudget);
+  if (e == cudaSuccess) e = cudaFuncSetAttribute(prefill_gemm_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, kPgSmemBudget);
   if (e == cudaSuccess) e = cudaFuncSetAttribute(prefill_attention_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kPaSmem);
   if (e == cudaSuccess) g_prefill_sms = sms;
   return e;
@@ -968,7 +971,7 @@ cudaError_t launch_prefill_gemm(const PrefillGemmArgs& a, cudaStream_t s) {
   }
   if (a.rows <= 0) return cudaSuccess;
   const bool grouped = a.units != nullptr;
-  if (a.N % 128 || a.K % 256 || a.K > kPrefillMaxWidth || (grouped && (!a.n_units || a.sums || a.unit_rows % 16 || a.unit_rows < 16 || a.unit_rows > 256)))
+  if (a.N % 128 || a.K % 256 || a.K > kPrefillMaxWidth || (grouped && (!a.n_units || a.sums || a.unit_rows % 16 || a.unit_rows < 16 || a.unit_rows > 240)))
     return cudaErrorInvalidValue;
   PgParams p;
   p.scales = a.scales, p.biases = a.biases, p.inv_scale = a.inv_scale, p.out = a.out, p.status = a.status;
@@ -982,11 +985,16 @@ cudaError_t launch_prefill_gemm(const PrefillGemmArgs& a, cudaStream_t s) {
     p.tok_tiles = t.tok_tiles, p.n_tile = t.n_tile;
     if (a.sums) p.parts = t.parts;
   }
-  // narrow tiles pass through a stage faster, and their smaller operand leaves room for more codes ahead
-  p.code_slots = p.n_tile <= 128 ? kPgMaxCodes : 3;
+  // Narrow tiles pass through a stage faster, and their smaller operand leaves room for more codes ahead.  A wait on a ring
+  // tells a phase from the one before it only, so whoever reads a ring has to meet every turn of it.  A pair reads every
+  // second slot of codes: their number is even, or a pair would meet a slot every second turn and could take codes that
+  // are a turn old for its own.  And it fills every fourth stage: there are at least four.
   const int stage = kPgABlock + p.n_tile * 128;
   const int units_bytes = grouped ? kPgUnits * (int)sizeof(int4) : 0;
-  p.stages = (pg_smem_budget(grouped) - 1024 - units_bytes - p.code_slots * kPgCodes) / stage;
+  auto stages_with = [&](int slots) { return (kPgSmemBudget - 1024 - units_bytes - slots * kPgCodes) / stage; };
+  p.code_slots = p.n_tile <= 128 ? kPgMaxCodes : 4;
+  p.stages = stages_with(p.code_slots);
+  if (p.stages < 4) return cudaErrorInvalidValue;
   if (p.stages > kPgMaxStages) p.stages = kPgMaxStages;
   const size_t smem = 1024 + (size_t)p.stages * stage + (size_t)p.code_slots * kPgCodes + units_bytes;
   EncodeTiledFn encode = nullptr;
