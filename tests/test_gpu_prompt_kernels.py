@@ -69,3 +69,26 @@ def test_prompt_kernels_at_tile_edges(shape, n_tokens, start):
     assert np.abs(g - o_logits).max() <= (0.15 if shape.n_experts else 3e-2) * rms
     pool.close()
     model.close()
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("shape,n_tokens", [(_dense(hidden=2048, mlp_inter=6144, n_layers=2), 1000), (_dense(hidden=3072, mlp_inter=4096), 760),
+                                            (_moe(24, 8), 1000)], ids=lambda v: getattr(v, "name", str(v)))
+def test_wide_tiles_repeat_bit_for_bit(shape, n_tokens):
+    """Several tiles per CTA, so that the rings of codes and operands turn many times: any order of the warps gives the same."""
+    from gpu_util import bits
+    from paper_2601_19139_b200 import binding as q4d
+    weights, pool_t = gen.make_weights(shape, 5, "cuda"), gen.make_pool(shape, 64, "cuda")
+    model = q4d.Model(shape, weights)
+    pool = q4d.KVPool(model, pool_t)
+    prompt = np.random.default_rng(3).integers(0, shape.vocab, size=n_tokens).astype(np.int32)
+    table = list(range(1, 1 + (n_tokens + 15) // 16))
+    lg = torch.zeros(shape.vocab, dtype=torch.float32, device="cuda")
+    seen = []
+    for _ in range(6):
+        q4d.prefill(model, pool, 7, prompt, 0, table, None, lg)
+        pool.request_release(7)
+        torch.cuda.synchronize()
+        seen.append((bits(pool_t)[:, :, table].copy(), lg.cpu().numpy().copy()))
+    for kv, logits in seen[1:]:
+        assert np.array_equal(kv, seen[0][0]) and np.array_equal(logits, seen[0][1])
